@@ -601,10 +601,8 @@ __global__ void __launch_bounds__(32 * kFusedWarps, sizeof(T) == 4 ? 4 : 2) vms_
 // ------------------------------------------------------------------------------------------
 template <bool JV>
 __global__ void __launch_bounds__(128) nitsche_penalty(Args A, const int32_t* __restrict__ pe,
-                                                       const int64_t* __restrict__ pq, const int64_t* __restrict__ pslot,
-                                                       const double* __restrict__ pen, const double* __restrict__ xr,
-                                                       const double* __restrict__ wr, const double* __restrict__ taub,
-                                                       int64_t n) {
+                                                       const int64_t* __restrict__ pslot,
+                                                       const double* __restrict__ pen, int64_t n) {
     // eight threads per element: thread c fetches corner c's jump, then forms row c
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = t >> 3;
@@ -636,21 +634,90 @@ __global__ void __launch_bounds__(128) nitsche_penalty(Args A, const int32_t* __
         for (int k = 0; k < 3; ++k) r[k] = fma(m, __shfl_sync(0xffffffffu, dc[k], base | b), r[k]);
     }
     if (!live) return;
-    if (!JV && A.gpts) {
-        for (int64_t q = pq[i]; q < pq[i + 1]; ++q) {
-            const double* gq = point_g(A, q);
-            double phi[8];
-            basis_values_d(xr + 3 * q, phi);
-            const double cq = cbmu * wr[q] * taub[q] * phi[c];
-            for (int k = 0; k < 3; ++k) r[k] = fma(cq, A.g[k] - gq[k], r[k]);
-        }
-    }
     if (A.ss) {
         double* dst = A.ss + 32 * pslot[i] + 4 * c;
         for (int k = 0; k < 3; ++k) dst[k] += r[k];
     } else {
         const double rr[4] = {r[0], r[1], r[2], 0.0};
         scatter(A, id, rr);
+    }
+}
+
+// The residual's penalty with a velocity per surface point (the second sum above too): a warp per
+// element, a lane per point.  Bound by the latency of the point data (two dependent loads, position
+// then velocity) and by the narrow FP64 pipe, so every point is read and its basis formed once, by one
+// lane, not by the eight threads of a corner in turn: 24 sums per lane, then halved over the lanes
+// (27 additions) until lane 4 c + k holds row (c, k).  41 k element truck pair, 19,898 points:
+// the residual with a velocity per point went from 325 to 81 us (this sum was 269 of them).
+__global__ void __launch_bounds__(128) nitsche_penalty_points(Args A, const int32_t* __restrict__ pe,
+                                                              const int64_t* __restrict__ pq,
+                                                              const int64_t* __restrict__ pslot,
+                                                              const double* __restrict__ pen, const double* __restrict__ xr,
+                                                              const double* __restrict__ wr, const double* __restrict__ taub,
+                                                              int64_t n) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n) return;              // uniform over the warp
+    if (A.skip && *A.skip) return;   // a captured solver step after its cycle ended
+    const int lane = threadIdx.x & 31, c = lane >> 2, k = lane & 3;
+    const int32_t e = pe[i];
+    const double cbmu = A.Cb * Phys<double>(A, prob_of(A, e)).mu;
+    const int32_t id = A.conn[8 * (int64_t)e + c];
+    // component k of corner c's u_s - g_body (k = 3: unused)
+    double u4[4], up4[4];
+    gather(A, A.U, id, u4);
+    if (!A.theta1) gather(A, A.Up, id, up4);
+    double dc = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        if (k == j) dc = (A.theta1 ? u4[j] : A.theta * u4[j] + (1.0 - A.theta) * up4[j]) - A.g[j];
+    double s[24];   // [corner][component] of this lane's points
+#pragma unroll
+    for (int j = 0; j < 24; ++j) s[j] = 0.0;
+    for (int64_t q = pq[i] + lane, q1 = pq[i + 1]; q < q1; q += 32) {
+        const double* gq = point_g(A, q);
+        double phi[8], t[3];
+        basis_values_d(xr + 3 * q, phi);
+        const double wq = wr[q] * taub[q];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) t[j] = wq * (A.g[j] - gq[j]);
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) s[3 * a + j] = fma(phi[a], t[j], s[3 * a + j]);
+    }
+    // lanes with bit 4, 3, 2 set keep the upper half of the corners, the others the lower half
+#pragma unroll
+    for (int h = 12, o = 16; h >= 3; h /= 2, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < 12; ++j)
+            if (j < h) {
+                const double keep = up ? s[h + j] : s[j], give = up ? s[j] : s[h + j];
+                s[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+    }
+    double r = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        double x = s[j];
+        x += __shfl_xor_sync(0xffffffffu, x, 1);
+        x += __shfl_xor_sync(0xffffffffu, x, 2);
+        if (k == j) r = x;
+    }
+    const double* P = pen + 36 * i;   // as in nitsche_penalty
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const int lo = c < b ? c : b, hi = c < b ? b : c;
+        r = fma(P[lo * 8 - lo * (lo - 1) / 2 + hi - lo], __shfl_sync(0xffffffffu, dc, 4 * b + k), r);
+    }
+    r *= cbmu;
+    if (A.ss) {
+        if (k < 3) A.ss[32 * pslot[i] + lane] += r;
+    } else {
+        double rr[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) rr[j] = __shfl_sync(0xffffffffu, r, (lane & ~3) + j);
+        if (k == 0) scatter(A, id, rr);
     }
 }
 
@@ -948,8 +1015,11 @@ void launch_penalty(const Mesh& m, const Args& A, cudaStream_t s, bool timed) {
     const int64_t np = (int64_t)m.pen_elem.size();
     if (np <= 0) return;
     Timed t(m, 2, s, 1, timed);
-    nitsche_penalty<JV><<<(unsigned)((8 * np + 127) / 128), 128, 0, s>>>(A, m.d.pen_elem, m.d.pen_q, m.d.pen_slot, m.d.pen,
+    if (!JV && A.gpts)
+        nitsche_penalty_points<<<(unsigned)((np + 3) / 4), 128, 0, s>>>(A, m.d.pen_elem, m.d.pen_q, m.d.pen_slot, m.d.pen,
                                                                         m.d.sq_x, m.d.sq_w, m.d.sq_taub, np);
+    else
+        nitsche_penalty<JV><<<(unsigned)((8 * np + 127) / 128), 128, 0, s>>>(A, m.d.pen_elem, m.d.pen_slot, m.d.pen, np);
 }
 
 // the surface buckets: thread-per-point and warp-per-element Nitsche kernels, then the float64
