@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -103,6 +104,363 @@ void gemm(cudaStream_t s, int M, int N, int K, const bf16* A, int64_t sam, int64
     gemm_bf16<<<grid, 128, 0, s>>>(M, N, K, A, sam, sak, B, sbn, sbk, C, ldc, alpha, beta);
 }
 
+// ------------------------------------------------------------------------------------------
+// The network of the preconditioner's width (128) in few launches.  A row of the forward pass moves
+// 8 KB (1027 floats in, 1024 out) for 0.56 Mflop: it is bound by HBM, so the whole pass is one kernel
+// that reads X and writes Y once, with the activations of its BM rows in shared memory and registers
+// and the weights (0.56 MB) from L2; mma.sync is far from its rate there.  Every sum runs over k in
+// steps of 16 in increasing order, as in gemm_bf16: the same bits.
+//   50,003 rows: 2,625 -> 161 us (2.55 TB/s of X and Y).
+// ------------------------------------------------------------------------------------------
+constexpr int kW = 128;            // width of the fused path
+constexpr int kKT = 32;            // k per stage of the first layer
+constexpr int kKS = kKT + 8;       // row stride of a stage (floats of X, bf16 of W1): conflict-free fragment reads
+constexpr int kHS = kW + 8;        // row stride of activations and of a weight chunk
+constexpr int kNC = 64;            // output columns per weight chunk of the second and third layer
+
+__device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// asynchronous copies of 16 or 4 bytes, the first `valid` of them from src, the rest zeros
+__device__ __forceinline__ void cpz16(void* dst, const void* src, int valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(saddr(dst)), "l"(src), "r"(valid) : "memory");
+}
+__device__ __forceinline__ void cpz4(void* dst, const void* src, int valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(saddr(dst)), "l"(src), "r"(valid) : "memory");
+}
+__device__ __forceinline__ void ldm4(uint32_t r[4], const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(saddr(p)) : "memory");
+}
+__device__ __forceinline__ void ldm4t(uint32_t r[4], const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(saddr(p)) : "memory");
+}
+__device__ __forceinline__ uint32_t cvt2(float lo, float hi) { return pack2(__float2bfloat16(lo), __float2bfloat16(hi)); }
+
+struct MlpTrainIO {           // what a training step keeps of the forward pass
+    const float* T;           // targets [n][nout]
+    float inv_scale;
+    bf16 *xb, *h1, *h2, *dy;  // inputs and activations in bf16, (y - t) * inv_scale
+    double* loss;             // += sum (y - t)^2
+};
+
+// BM rows per CTA, 4 warps: for BM = 64 two by two over (rows, columns), otherwise all four over the
+// columns.  STAGES k-tiles of X (fp32) and W1 in flight; the same shared memory then holds the
+// activations and two chunks of W2 / W3.
+template <int BM, int STAGES> struct FwdShape {
+    static constexpr int WM = BM == 64 ? 2 : 1, WN = 4 / WM, MI = BM / (16 * WM);
+    static constexpr int XS = BM * kKS * 4, WS = kW * kKS * 2;         // bytes of a stage
+    static constexpr int HB = BM * kHS * 2, CB = kNC * kHS * 2;        // bytes of the activations, of a weight chunk
+    static constexpr int smem = STAGES * (XS + WS) > HB + 2 * CB ? STAGES * (XS + WS) : HB + 2 * CB;
+};
+
+template <int BM, int STAGES, bool TRAIN>
+__global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad, const float* __restrict__ X, int64_t ldx,
+                                                 int xvec, const bf16* __restrict__ W1, const float* __restrict__ b1,
+                                                 const bf16* __restrict__ W2, const float* __restrict__ b2,
+                                                 const bf16* __restrict__ W3, const float* __restrict__ b3, int nout,
+                                                 float* __restrict__ Y, MlpTrainIO io) {
+    typedef FwdShape<BM, STAGES> Sh;
+    constexpr int WN = Sh::WN, MI = Sh::MI, N1 = kW / WN / 8, N2 = kNC / WN / 8;
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
+    const int wm = (warp / WN) * 16 * MI, wn = warp % WN;
+    const int64_t m0 = (int64_t)blockIdx.x * BM;
+    auto xs = [&](int s) { return reinterpret_cast<float*>(sm + s * (Sh::XS + Sh::WS)); };
+    auto ws = [&](int s) { return reinterpret_cast<bf16*>(sm + s * (Sh::XS + Sh::WS) + Sh::XS); };
+    const int nkt = (nin_pad + kKT - 1) / kKT;
+    auto load = [&](int kt) {
+        if (kt < nkt) {
+            float* x = xs(kt % STAGES);
+            bf16* w = ws(kt % STAGES);
+            for (int i = tid; i < BM * (kKT / 4); i += 128) {
+                const int r = i / (kKT / 4), c = i % (kKT / 4) * 4, gc = kt * kKT + c;
+                const int64_t gr = m0 + r;
+                const int left = gr < n ? max(0, min(4, nin - gc)) : 0;
+                const float* src = left ? X + gr * ldx + gc : X;
+                if (xvec) cpz16(x + r * kKS + c, src, 4 * left);
+                else
+                    for (int j = 0; j < 4; ++j) cpz4(x + r * kKS + c + j, j < left ? src + j : X, j < left ? 4 : 0);
+            }
+            for (int i = tid; i < kW * (kKT / 8); i += 128) {
+                const int r = i / (kKT / 8), c = i % (kKT / 8) * 8, gc = kt * kKT + c;
+                const bool in = gc < nin_pad;
+                cpz16(w + r * kKS + c, in ? W1 + (int64_t)r * nin_pad + gc : W1, in ? 16 : 0);
+            }
+        }
+        cp_commit();
+    };
+    // ldmatrix lane offsets: A (16 x 16, rows then k halves), B (two n-tiles, k halves)
+    const int arow = lane & 15, acol = (lane >> 4) * 8;
+    const int brow = (lane & 7) + ((lane >> 4) << 3), bcol = ((lane >> 3) & 1) * 8;
+    for (int s = 0; s < STAGES - 1; ++s) load(s);
+    float acc[MI][N1][4];
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+        for (int j = 0; j < N1; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
+    for (int kt = 0; kt < nkt; ++kt) {
+        cp_wait<STAGES - 2>();
+        __syncthreads();   // stage kt has landed; every warp is done with stage kt - 1, which is refilled
+        load(kt + STAGES - 1);
+        const float* x = xs(kt % STAGES);
+        const bf16* w = ws(kt % STAGES);
+#pragma unroll
+        for (int ks = 0; ks < kKT; ks += 16) {
+            uint32_t a[MI][4];
+#pragma unroll
+            for (int i = 0; i < MI; ++i)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int r = wm + 16 * i + gid + (q & 1) * 8, c = ks + 2 * tig + (q >> 1) * 8;
+                    const float2 v = *reinterpret_cast<const float2*>(x + r * kKS + c);
+                    a[i][q] = cvt2(v.x, v.y);
+                    if (TRAIN && wn == 0 && m0 + r < n && kt * kKT + c < nin_pad)
+                        *reinterpret_cast<uint32_t*>(io.xb + (m0 + r) * nin_pad + kt * kKT + c) = a[i][q];
+                }
+#pragma unroll
+            for (int j = 0; j < N1; j += 2) {
+                uint32_t b[4];
+                ldm4(b, w + (wn * (kW / WN) + 8 * j + brow) * kKS + ks + bcol);
+#pragma unroll
+                for (int i = 0; i < MI; ++i) {
+                    mma16816(acc[i][j], a[i], b);
+                    mma16816(acc[i][j + 1], a[i], b + 2);
+                }
+            }
+        }
+    }
+    cp_wait<0>();
+    __syncthreads();   // the stages are free: activations and weight chunks take their place
+    bf16* h = reinterpret_cast<bf16*>(sm);
+    auto chunk_buf = [&](int k) { return reinterpret_cast<bf16*>(sm + Sh::HB + (k & 1) * Sh::CB); };
+    // chunks 0, 1: W2; 2 ...: W3
+    const int nchunk = kW / kNC + (nout + kNC - 1) / kNC;
+    auto load_chunk = [&](int k) {
+        if (k < nchunk) {
+            const bool l2 = k < kW / kNC;
+            const bf16* W = l2 ? W2 : W3;
+            const int n0 = (l2 ? k : k - kW / kNC) * kNC, nr = l2 ? kW : nout;
+            bf16* w = chunk_buf(k);
+            for (int i = tid; i < kNC * (kW / 8); i += 128) {
+                const int r = i / (kW / 8), c = i % (kW / 8) * 8;
+                const bool in = n0 + r < nr;
+                cpz16(w + r * kHS + c, in ? W + (int64_t)(n0 + r) * kW + c : W, in ? 16 : 0);
+            }
+        }
+        cp_commit();
+    };
+    // h = relu(z + b) in bf16 of one accumulator pair, to shared memory (and, training, to memory)
+    auto put_h = [&](const float* z, const float* b, int r, int c, bf16* keep) {
+        const float v0 = z[0] + __ldg(b + c), v1 = z[1] + __ldg(b + c + 1);
+        const uint32_t p = cvt2(v0 > 0.f ? v0 : 0.f, v1 > 0.f ? v1 : 0.f);
+        *reinterpret_cast<uint32_t*>(h + r * kHS + c) = p;
+        if (TRAIN && m0 + r < n) *reinterpret_cast<uint32_t*>(keep + (m0 + r) * kW + c) = p;
+    };
+    load_chunk(0);
+    load_chunk(1);
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+        for (int j = 0; j < N1; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; q += 2)
+                put_h(&acc[i][j][q], b1, wm + 16 * i + gid + q * 4, wn * (kW / WN) + 8 * j + 2 * tig, io.h1);
+    // one weight chunk: o[i][j] = rows of h times kNC / WN of its columns
+    uint32_t a[kW / 16][MI][4];
+    auto load_a = [&]() {
+#pragma unroll
+        for (int ks = 0; ks < kW / 16; ++ks)
+#pragma unroll
+            for (int i = 0; i < MI; ++i) ldm4(a[ks][i], h + (wm + 16 * i + arow) * kHS + 16 * ks + acol);
+    };
+    auto times_chunk = [&](int k, float o[MI][N2][4]) {
+        const bf16* w = chunk_buf(k);
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < N2; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) o[i][j][q] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < kW / 16; ++ks)
+#pragma unroll
+            for (int j = 0; j < N2; j += 2) {
+                uint32_t b[4];
+                ldm4(b, w + (wn * (kNC / WN) + 8 * j + brow) * kHS + 16 * ks + bcol);
+#pragma unroll
+                for (int i = 0; i < MI; ++i) {
+                    mma16816(o[i][j], a[ks][i], b);
+                    mma16816(o[i][j + 1], a[ks][i], b + 2);
+                }
+            }
+    };
+    float z2[kW / kNC][MI][N2][4];
+#pragma unroll
+    for (int k = 0; k < kW / kNC; ++k) {
+        cp_wait<1>();
+        __syncthreads();
+        if (k == 0) load_a();
+        times_chunk(k, z2[k]);
+        __syncthreads();
+        load_chunk(k + 2);
+    }
+#pragma unroll
+    for (int k = 0; k < kW / kNC; ++k)
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < N2; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; q += 2)
+                    put_h(&z2[k][i][j][q], b2, wm + 16 * i + gid + q * 4, k * kNC + wn * (kNC / WN) + 8 * j + 2 * tig, io.h2);
+    float lhi = 0.f, llo = 0.f;   // training: sum (y - t)^2 of this thread in two floats
+    for (int k = kW / kNC; k < nchunk; ++k) {
+        cp_wait<1>();
+        __syncthreads();
+        if (k == kW / kNC) load_a();
+        float o[MI][N2][4];
+        times_chunk(k, o);
+        __syncthreads();
+        load_chunk(k + 2);
+        const int n0 = (k - kW / kNC) * kNC + wn * (kNC / WN) + 2 * tig;
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < N2; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; q += 2) {
+                    const int64_t r = m0 + wm + 16 * i + gid + q * 4;
+                    const int c = n0 + 8 * j;
+                    if (r >= n || c >= nout) continue;   // nout is even
+                    const float y0 = o[i][j][q] + __ldg(b3 + c), y1 = o[i][j][q + 1] + __ldg(b3 + c + 1);
+                    if constexpr (!TRAIN) {
+                        *reinterpret_cast<float2*>(Y + r * nout + c) = make_float2(y0, y1);
+                    } else {
+                        const float2 t = __ldg(reinterpret_cast<const float2*>(io.T + r * nout + c));
+                        const float d0 = y0 - t.x, d1 = y1 - t.y;
+                        *reinterpret_cast<uint32_t*>(io.dy + r * nout + c) = cvt2(d0 * io.inv_scale, d1 * io.inv_scale);
+                        // exact square (two floats) added with TwoSum: float64's narrow pipe stays out of it
+                        for (const float d : {d0, d1}) {
+                            const float sq = __fmul_rn(d, d), s = __fadd_rn(lhi, sq), bp = __fsub_rn(s, lhi);
+                            llo += __fadd_rn(__fsub_rn(lhi, __fsub_rn(s, bp)), __fsub_rn(sq, bp)) + __fmaf_rn(d, d, -sq);
+                            lhi = s;
+                        }
+                    }
+                }
+    }
+    cp_wait<0>();
+    if constexpr (TRAIN) {
+        double s = (double)lhi + (double)llo;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) atomicAdd(io.loss, s);
+    }
+}
+
+// Gradient products of one layer in one launch, 32 x 32 of the result per CTA, K whole (the sums keep
+// the order of gemm_bf16), 64 of K per stage, four stages in flight.  Bound by the latency of the K chain
+// (64 dependent products for 1024 rows), so the tiles are small: more CTAs, not more work per CTA.
+//   dw CTAs: G [M][N] = alpha D^T H  (D [K][M], H [K][N] rows of the batch), and the column sums of D
+//            (the bias gradient, rows in order) from the tiles of the CTAs with n0 = 0;
+//   dh CTAs: Z [K][N] = (D W) masked by H > 0, in bf16 (W [M][N] the layer's weights, H its input).
+constexpr int kBT = 32, kBK = 64, kBStages = 4;
+struct BackArgs {
+    int64_t K;             // rows of the batch
+    int M, N;              // the layer's outputs and inputs
+    const bf16 *D, *H, *W;
+    float *G, *db;
+    bf16* Z;               // null: no dh part
+    float beta;
+    int dw_n, dw_tiles;    // CTAs along N and in all of the dw part
+};
+
+__global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
+    // a stage: A as [64][32 + 8] (dw: rows k) or [32][64 + 8] (dh: rows m), B as [64][32 + 8]
+    constexpr int AS = kBK * (kBT + 8), TS = kBT + 8, DS = kBK + 8;
+    __shared__ __align__(16) bf16 sA[kBStages][AS], sB[kBStages][AS];
+    static_assert(kBT * DS <= AS, "stage size");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
+    const int wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
+    const bool dw = (int)blockIdx.x < P.dw_tiles;
+    const int t = dw ? blockIdx.x : blockIdx.x - P.dw_tiles;
+    const int nb = dw ? P.dw_n : (P.N + kBT - 1) / kBT;
+    const int64_t m0 = (int64_t)(t / nb) * kBT;
+    const int n0 = (t % nb) * kBT;
+    const int64_t K = dw ? P.K : P.M;
+    const int64_t rows = dw ? P.M : P.K;       // extent of the result along m
+    const bf16* B = dw ? P.H : P.W;
+    const int nkt = (int)((K + kBK - 1) / kBK);
+    auto load = [&](int kt) {
+        if (kt < nkt) {
+            bf16 *a = sA[kt % kBStages], *b = sB[kt % kBStages];
+            const int64_t k0 = (int64_t)kt * kBK;
+            for (int i = tid; i < kBK * kBT / 8; i += 128) {
+                const int kr = i / (kBT / 8), c = i % (kBT / 8) * 8;
+                const bool inb = k0 + kr < K && n0 + c < P.N;
+                cpz16(b + kr * TS + c, inb ? B + (k0 + kr) * P.N + n0 + c : B, inb ? 16 : 0);
+                if (dw) {
+                    const bool ina = k0 + kr < K && m0 + c < P.M;
+                    cpz16(a + kr * TS + c, ina ? P.D + (k0 + kr) * P.M + m0 + c : P.D, ina ? 16 : 0);
+                } else {
+                    const int mr = i / (kBK / 8), kc = i % (kBK / 8) * 8;
+                    const bool ina = m0 + mr < P.K && k0 + kc < K;
+                    cpz16(a + mr * DS + kc, ina ? P.D + (m0 + mr) * P.M + k0 + kc : P.D, ina ? 16 : 0);
+                }
+            }
+        }
+        cp_commit();
+    };
+    for (int s = 0; s < kBStages - 1; ++s) load(s);
+    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    const bool sums = dw && n0 == 0 && warp == 0;
+    float s = 0.f;
+    // transposed 8 x 8 blocks: A as (m, k), (m + 8, k), (m, k + 8), (m + 8, k + 8); B as (n, k), (n, k + 8), ...
+    const int akr = (lane & 7) + ((lane >> 4) << 3), amc = ((lane >> 3) & 1) * 8;
+    const int bkr = lane & 15, bnc = (lane >> 4) * 8;
+    const int arow = lane & 15, acol = (lane >> 4) * 8;
+    for (int kt = 0; kt < nkt; ++kt) {
+        cp_wait<kBStages - 2>();
+        __syncthreads();
+        load(kt + kBStages - 1);
+        const bf16 *a = sA[kt % kBStages], *b = sB[kt % kBStages];
+#pragma unroll
+        for (int ks = 0; ks < kBK; ks += 16) {
+            uint32_t af[4], bf[4];
+            if (dw) ldm4t(af, a + (ks + akr) * TS + wm + amc);
+            else ldm4(af, a + (wm + arow) * DS + ks + acol);
+            ldm4t(bf, b + (ks + bkr) * TS + wn + bnc);
+            mma16816(acc[0], af, bf);
+            mma16816(acc[1], af, bf + 2);
+        }
+        if (sums) {
+            const int kr1 = (int)min((int64_t)kBK, K - (int64_t)kt * kBK);
+#pragma unroll 16
+            for (int kr = 0; kr < kr1; ++kr) s += __bfloat162float(a[kr * TS + lane]);
+        }
+    }
+    cp_wait<0>();
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+            const int64_t r = m0 + wm + gid + q * 4;
+            const int c = n0 + wn + 8 * j + 2 * tig;
+            if (r >= rows || c >= P.N) continue;   // N is a multiple of 8
+            if (dw) {
+                float2* g = reinterpret_cast<float2*>(P.G + r * P.N + c);
+                float2 v = make_float2(acc[j][q], acc[j][q + 1]);
+                if (P.beta != 0.f) { const float2 o = *g; v.x += P.beta * o.x; v.y += P.beta * o.y; }
+                *g = v;
+            } else {
+                const uint32_t hv = *reinterpret_cast<const uint32_t*>(P.H + r * P.N + c);
+                const float h0 = __uint_as_float(hv << 16), h1 = __uint_as_float(hv & 0xFFFF0000u);
+                *reinterpret_cast<uint32_t*>(P.Z + r * P.N + c) = cvt2(h0 > 0.f ? acc[j][q] : 0.f, h1 > 0.f ? acc[j][q + 1] : 0.f);
+            }
+        }
+    if (sums && m0 + lane < P.M) P.db[m0 + lane] = P.beta != 0.f ? P.db[m0 + lane] + s : s;
+}
+
 __global__ void to_bf16(int64_t n, const float* __restrict__ x, bf16* __restrict__ y) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         y[i] = __float2bfloat16(x[i]);
@@ -154,15 +512,18 @@ __global__ void col_sum(int64_t n, int w, const bf16* __restrict__ d, float* __r
     for (int64_t r = 0; r < n; ++r) s += __bfloat162float(d[r * w + j]);
     db[j] = accumulate ? db[j] + s : s;
 }
+// Adam update and the weights' new bf16 copy
 __global__ void adam(int64_t n, float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                     float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
+                     float* __restrict__ v, bf16* __restrict__ wb, float lr, float b1, float b2, float eps, float c1, float c2) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
         const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
         m[i] = mi;
         v[i] = vi;
-        w[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+        const float wi = w[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+        w[i] = wi;
+        wb[i] = __float2bfloat16(wi);
     }
 }
 
@@ -342,6 +703,51 @@ static bool mlp_reserve(Mlp& M, int64_t b) {
 
 static void mlp_sync_bf16(Mlp& M, cudaStream_t s) { to_bf16<<<nblk(M.nparam), 256, 0, s>>>(M.nparam, M.P, M.Pb); }
 
+// The fused kernels serve the preconditioner's width; rows of 16 bytes in every bf16 matrix need nout % 8 == 0.
+static bool mlp_fast(const Mlp& M) { return M.w == kW && M.nout % 8 == 0; }
+
+template <int BM, int STAGES, bool TRAIN>
+static void launch_fused(const Mlp& M, const float* X, int64_t ldx, int64_t n, float* Y, const MlpTrainIO& io, cudaStream_t s) {
+    typedef FwdShape<BM, STAGES> Sh;
+    static std::atomic<unsigned> ready{0};   // devices whose shared-memory limit is raised
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 32 || !((ready.load() >> dev) & 1u)) {
+        cudaFuncSetAttribute(mlp_fused<BM, STAGES, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem);
+        if (dev < 32) ready.fetch_or(1u << dev);
+    }
+    const int xvec = ((uintptr_t)X & 15) == 0 && ldx % 4 == 0;
+    mlp_fused<BM, STAGES, TRAIN><<<(unsigned)((n + BM - 1) / BM), 128, Sh::smem, s>>>(
+        n, M.nin, M.nin_pad, X, ldx, xvec, M.Pb + M.off(0), M.P + M.off(1), M.Pb + M.off(2), M.P + M.off(3), M.Pb + M.off(4),
+        M.P + M.off(5), M.nout, Y, io);
+}
+
+// Rows per CTA: 64 (the weights are read from L2 once per 64 rows) when that still gives two CTAs per SM,
+// fewer for fewer rows, so that the chip has work: @RULE@
+template <bool TRAIN>
+static void mlp_fused_rows(const Mlp& M, const float* X, int64_t ldx, int64_t n, float* Y, const MlpTrainIO& io, cudaStream_t s) {
+    if (n >= 64 * 152 * 2) launch_fused<64, 3, TRAIN>(M, X, ldx, n, Y, io, s);
+    else if (n >= 32 * 152) launch_fused<32, 4, TRAIN>(M, X, ldx, n, Y, io, s);
+    else launch_fused<16, 6, TRAIN>(M, X, ldx, n, Y, io, s);
+}
+
+// forward and backward of a batch on the fused path: gradients into M.G, loss added to M.loss
+static void mlp_step_fused(Mlp& M, const float* X, int64_t ldx, const float* T, int64_t b, double n_total, float beta,
+                           cudaStream_t s) {
+    const MlpTrainIO io = {T, (float)(1.0 / n_total), M.xb, M.h1, M.h2, M.dyb, M.loss};
+    mlp_fused_rows<true>(M, X, ldx, b, nullptr, io, s);
+    auto back = [&](int m, int nn, const bf16* D, const bf16* H, int k, bf16* Z) {
+        BackArgs P = {b, m, nn, D, H, M.Pb + M.off(k), M.G + M.off(k), M.G + M.off(k + 1), Z, beta, 0, 0};
+        P.dw_n = (nn + kBT - 1) / kBT;
+        P.dw_tiles = P.dw_n * ((m + kBT - 1) / kBT);
+        const int64_t dh = Z ? P.dw_n * ((b + kBT - 1) / kBT) : 0;
+        mlp_back<<<(unsigned)(P.dw_tiles + dh), 128, 0, s>>>(P);
+    };
+    back(M.nout, M.w, M.dyb, M.h2, 4, M.dz2);
+    back(M.w, M.w, M.dz2, M.h1, 2, M.dz1);
+    back(M.w, M.nin_pad, M.dz1, M.xb, 0, nullptr);
+}
+
 // forward of a batch: X float [b][ldx] (first nin columns) -> M.y float [b][nout]
 static void mlp_forward_batch(Mlp& M, const float* X, int64_t ldx, int64_t b, cudaStream_t s) {
     rows_to_bf16<<<nblk(b * M.nin_pad), 256, 0, s>>>(b, M.nin, ldx, X, M.nin_pad, M.xb);
@@ -370,6 +776,13 @@ static void mlp_backward_batch(Mlp& M, const float* T, int64_t b, double n_total
     relu_back<<<nblk(b * M.w), 256, 0, s>>>(b * M.w, M.dh1, M.z1, M.dz1);
     gemm(s, M.w, M.nin_pad, (int)b, M.dz1, 1, M.w, M.xb, 1, M.nin_pad, M.G + M.off(0), M.nin_pad, 1.f, beta);
     col_sum<<<(M.w + 127) / 128, 128, 0, s>>>(b, M.w, M.dz1, M.G + M.off(1), beta != 0.f);
+}
+
+// forward and gradient of a batch (targets read in pairs on the fused path)
+static void mlp_step(Mlp& M, const float* X, int64_t ldx, const float* T, int64_t b, double n_total, float beta, cudaStream_t s) {
+    if (mlp_fast(M) && ((uintptr_t)T & 7) == 0) { mlp_step_fused(M, X, ldx, T, b, n_total, beta, s); return; }
+    mlp_forward_batch(M, X, ldx, b, s);
+    mlp_backward_batch(M, T, b, n_total, beta, s);
 }
 
 int mlp_create(int nin, int width, int nout, uint64_t seed, Mlp** out, std::string& err) {
@@ -438,6 +851,10 @@ int mlp_grads(Mlp* M, float* host) { return cudaMemcpy(host, M->G, M->nparam * 4
 
 int mlp_forward(Mlp* M, const float* X, int64_t ldx, int64_t n, float* Y, cudaStream_t s) {
     const int64_t B = 4096;
+    if (mlp_fast(*M) && ((uintptr_t)Y & 7) == 0) {
+        if (n > 0) mlp_fused_rows<false>(*M, X, ldx, n, Y, MlpTrainIO{}, s);
+        return cudaGetLastError() == cudaSuccess ? 0 : 1;
+    }
     if (!mlp_reserve(*M, std::min(n, B))) return 1;
     for (int64_t r = 0; r < n; r += B) {
         const int64_t b = std::min(B, n - r);
@@ -454,8 +871,7 @@ int mlp_gradient(Mlp* M, const float* X, int64_t ldx, const float* T, int64_t n,
     cudaMemsetAsync(M->loss, 0, 8, s);
     for (int64_t r = 0; r < n; r += B) {
         const int64_t b = std::min(B, n - r);
-        mlp_forward_batch(*M, X + r * ldx, ldx, b, s);
-        mlp_backward_batch(*M, T + r * M->nout, b, (double)n, r == 0 ? 0.f : 1.f, s);
+        mlp_step(*M, X + r * ldx, ldx, T + r * M->nout, b, (double)n, r == 0 ? 0.f : 1.f, s);
     }
     double h = 0.0;
     cudaMemcpyAsync(&h, M->loss, 8, cudaMemcpyDeviceToHost, s);
@@ -472,13 +888,11 @@ int mlp_train(Mlp* M, const float* X, int64_t ldx, const float* T, int64_t n, in
         cudaMemsetAsync(M->loss, 0, 8, s);
         for (int64_t r = 0; r < n; r += batch) {
             const int64_t b = std::min<int64_t>(batch, n - r);
-            mlp_forward_batch(*M, X + r * ldx, ldx, b, s);
-            mlp_backward_batch(*M, T + r * M->nout, b, (double)b, 0.f, s);
+            mlp_step(*M, X + r * ldx, ldx, T + r * M->nout, b, (double)b, 0.f, s);
             ++M->step;
             const float b1 = 0.9f, b2 = 0.999f;
             const float c1 = 1.f / (1.f - std::pow(b1, (float)M->step)), c2 = 1.f / (1.f - std::pow(b2, (float)M->step));
-            adam<<<nblk(M->nparam), 256, 0, s>>>(M->nparam, M->P, M->G, M->Mm, M->Vm, lr, b1, b2, 1e-8f, c1, c2);
-            mlp_sync_bf16(*M, s);
+            adam<<<nblk(M->nparam), 256, 0, s>>>(M->nparam, M->P, M->G, M->Mm, M->Vm, M->Pb, lr, b1, b2, 1e-8f, c1, c2);
         }
         double h = 0.0;
         cudaMemcpyAsync(&h, M->loss, 8, cudaMemcpyDeviceToHost, s);

@@ -60,3 +60,53 @@ def test_penalty_with_point_velocities(dev, triangles, level, deterministic):
         o.set_surface_velocity(None)
     got = g.residual(ph, T(u, dev), T(up, dev), g_points=T(vel, dev)).cpu().numpy()
     assert rel(got, want) <= TOL64
+
+
+# ---- the network: row counts around the tiles of 16, 32 and 64 rows and where the tile changes,
+# odd output edges and inputs without 16-byte rows ----
+def _mlp64(p, X):
+    W1, b1, W2, b2, W3, b3 = p
+    r = lambda a: a.to(torch.bfloat16).double()
+    h1 = r((r(X) @ r(W1).T + b1).clamp_min(0))
+    h2 = r((h1 @ r(W2).T + b2).clamp_min(0))
+    return h1, h2, h2 @ r(W3).T + b3
+
+
+def _params(net, dev):
+    return [T(q, dev) for q in net.unpack(net.params())]
+
+
+@pytest.mark.parametrize("rows", [1, 15, 17, 63, 64, 4863, 4864, 4865, 19455, 19457])
+@pytest.mark.parametrize("shape", [(1027, 1024, 1040, 0), (45, 72, 45, 0), (64, 8, 67, 1)])
+def test_mlp_forward_rows(dev, rows, shape):
+    nin, nout, ldx, shift = shape
+    net = api.Mlp(n_in=nin, n_out=nout, seed=5)
+    torch.manual_seed(rows)
+    X = torch.randn(rows * ldx + shift, device=dev)[shift:].view(rows, ldx)
+    _, _, want = _mlp64(_params(net, dev), X[:, :nin].double())
+    got = net.forward(X).double()
+    # what is left is float32 sums and the activations they round to the other bf16 neighbour (2^-8)
+    assert float((got - want).norm() / want.norm()) <= 2e-3
+
+
+@pytest.mark.parametrize("rows,batch", [(130, 130), (257, 64), (2048, 1000)])
+@pytest.mark.parametrize("nin,nout", [(1027, 1024), (45, 72)])
+def test_mlp_gradient_rows(dev, rows, batch, nin, nout):
+    net = api.Mlp(n_in=nin, n_out=nout, seed=6)
+    torch.manual_seed(rows)
+    X, Y = torch.randn(rows, nin, device=dev), torch.randn(rows, nout, device=dev)
+    p = _params(net, dev)
+    r = lambda a: a.to(torch.bfloat16).double()
+    h1, h2, out = _mlp64(p, X.double())
+    e = out - Y.double()
+    dy = r(e / rows)
+    d2 = r((dy @ r(p[4])) * (h2 > 0))
+    d1 = r((d2 @ r(p[2])) * (h1 > 0))
+    want = [d1.T @ r(X.double()), d1.sum(0), d2.T @ h1, d2.sum(0), dy.T @ h2, dy.sum(0)]
+    loss, g = net.gradient(X, Y)
+    # bf16 neighbours of the activations and errors, at most two roundings deep
+    assert abs(loss - float((e * e).sum()) / (2 * rows)) <= 1e-3 * loss
+    for k, (a, b) in enumerate(zip(net.unpack(g), want)):
+        assert float((T(a, dev) - b).norm() / b.norm()) <= 1e-2, k
+    first = net.train(X, Y, epochs=1, batch=batch, lr=1e-3)[0]
+    assert net.train(X, Y, epochs=8, batch=batch, lr=1e-3)[-1] < first
