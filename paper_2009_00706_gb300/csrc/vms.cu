@@ -56,6 +56,174 @@ template <class T> struct IntShape {
     static constexpr size_t smem = (size_t)(2 * EPB * ESTR + EPB * 8 * MSTR) * sizeof(T);
 };
 
+// One Out element in float64 on 8 lanes of a warp (c = lane & 7); nd its 8 corner rows, sw the warp's
+// 4 x 272 doubles.  FP64 instructions are the cost (see Const64), so the work goes to lanes by what
+// shares most of them:
+//   1. a lane takes one column (u, v, w, p and, J v, their tangents; R: the du/dt columns) of all 8
+//      corners: Hadamard transform, then the inverse along z, y, x with the Gauss abscissa in its
+//      multiply-adds, whose intermediates are the gradients and mixed derivatives (62 instructions for
+//      8 points; point by point they are 8 + 12 + 4 per point).  du/dt of J v: shuffles (6 per column).
+//   2. a lane takes Gauss point c: pointwise64.
+//   3. a lane takes component c & 3 and the four points of one z side: the transposed sums along x and
+//      y, then z with its partner lane (52 instructions).
+// 283 k elements (sphere wake), one R and one J v with all their kernels: 5.91 -> 3.88 ms.
+template <bool JV>
+__device__ __forceinline__ void interior_element64(const Args& A, const double* nd, double* sw, int lane, int64_t idx,
+                                                   bool valid, int lv, int prob, int32_t id) {
+    constexpr double gam = 1.0 / kInvGauss;
+    const int c = lane & 7;
+    double* E = sw + (lane >> 3) * 272;   // V [8 columns][8], GX | GY | GZ [8][4], XY | XZ | YZ [8][2]
+    __syncwarp();
+    {
+        const int col = JV ? (c & 3) + (c >> 2) * CT : (c < 7 ? c : 6);
+        double a[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) a[t] = nd[t * CS + col];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                if (!(t & (1 << k))) {
+                    const double lo = a[t], hi = a[t | (1 << k)];
+                    a[t] = lo + hi;
+                    a[t | (1 << k)] = hi - lo;
+                }
+        double *V = E + 8 * c, *GX = E + 64 + 4 * c, *GY = E + 96 + 4 * c, *GZ = E + 128 + 4 * c, *XY = E + 160 + 2 * c,
+               *XZ = E + 176 + 2 * c, *YZ = E + 192 + 2 * c;
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+            const double gz = z ? gam : -gam;
+            double b[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) b[t] = fma(gz, a[4 + t], a[t]);
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const double gy = y ? gam : -gam;
+                const double c0 = fma(gy, b[2], b[0]), c1 = fma(gy, b[3], b[1]);
+                V[4 * z + 2 * y] = fma(-gam, c1, c0);
+                V[4 * z + 2 * y + 1] = fma(gam, c1, c0);
+                GX[2 * z + y] = c1;
+            }
+            GY[2 * z] = fma(-gam, b[3], b[2]);
+            GY[2 * z + 1] = fma(gam, b[3], b[2]);
+            XY[z] = b[3];
+        }
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            const double gy = y ? gam : -gam;
+            const double d0 = fma(gy, a[6], a[4]), d1 = fma(gy, a[7], a[5]);
+            GZ[2 * y] = fma(-gam, d1, d0);
+            GZ[2 * y + 1] = fma(gam, d1, d0);
+            XZ[y] = d1;
+        }
+        YZ[0] = fma(-gam, a[7], a[6]);
+        YZ[1] = fma(gam, a[7], a[6]);
+    }
+    // 8 x the value at Gauss point c of a field whose value at corner c this lane holds
+    auto to_point = [&](double x) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) x = fma(1.0 + gam, x, (1.0 - gam) * __shfl_xor_sync(0xffffffffu, x, 1 << k));
+        return x;
+    };
+    Point64 F;
+    if (JV)
+        for (int i = 0; i < 3; ++i) F.a[i] = to_point(nd[c * CS + 4 + i]);
+    if (A.ndf)
+        for (int i = 0; i < 3; ++i) F.f[i] = to_point(nd[c * CS + CF + i]);
+    __syncwarp();
+    const int x = c & 1, y = (c >> 1) & 1, z = c >> 2, yz = c >> 1, xz = x | (z << 1), xy = c & 3;
+    Tangent64 D;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const double v = E[8 * i + c], gx = E[64 + 4 * i + yz], gy = E[96 + 4 * i + xz], gz = E[128 + 4 * i + xy];
+        if (i < 3) { F.u[i] = v; F.G[i][0] = gx; F.G[i][1] = gy; F.G[i][2] = gz; }
+        else { F.p = v; F.gp[0] = gx; F.gp[1] = gy; F.gp[2] = gz; }
+    }
+    if (!JV)
+        for (int i = 0; i < 3; ++i) F.a[i] = E[8 * (4 + i) + c];
+    auto mixed = [&](int b, double H[3]) {   // (grad div u)_i = sum_{j != i} d_i d_j u_j
+        H[0] = E[160 + 2 * (b + 1) + z] + E[176 + 2 * (b + 2) + y];
+        H[1] = E[160 + 2 * b + z] + E[192 + 2 * (b + 2) + x];
+        H[2] = E[176 + 2 * b + y] + E[192 + 2 * (b + 1) + x];
+    };
+    mixed(0, F.H);
+    if (JV) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double v = E[8 * (4 + i) + c], gx = E[64 + 4 * (4 + i) + yz], gy = E[96 + 4 * (4 + i) + xz],
+                         gz = E[128 + 4 * (4 + i) + xy];
+            if (i < 3) { D.u[i] = v; D.G[i][0] = gx; D.G[i][1] = gy; D.G[i][2] = gz; }
+            else { D.p = v; D.gp[0] = gx; D.gp[1] = gy; D.gp[2] = gz; }
+        }
+        mixed(4, D.H);
+    }
+    double W[16];
+    {
+        const Phys<double> P(A, prob);
+        const Const64 C(A, P, lv, A.lc[lv][4], A.lc[lv][5]);
+        pointwise64<JV>(C, A.ndf != nullptr, A.c0th, F, D, W);
+    }
+    __syncwarp();   // every lane has read its fields: the coefficients [16][8] take their place
+#pragma unroll
+    for (int k = 0; k < 16; ++k) E[8 * k + c] = W[k];
+    __syncwarp();
+    // the four points of side z = hz: sums along x, then y, for every S over (x, y): M, and Z the sums of
+    // the z coefficient
+    const int k = c & 3, hz = c >> 2;
+    double M[4], Z[4];
+    {
+        const double *f = E + 8 * k + 4 * hz, *sx = E + 8 * (4 + 3 * k) + 4 * hz, *sy = sx + 8, *sz = sx + 16;
+        double lo[2], hi[2], ylo[2], yhi[2], zlo[2], zhi[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const double f0 = f[2 * q], f1 = f[2 * q + 1];
+            lo[q] = f0 + f1;
+            hi[q] = (f1 + sx[2 * q + 1]) + (sx[2 * q] - f0);
+            ylo[q] = sy[2 * q] + sy[2 * q + 1];
+            yhi[q] = sy[2 * q + 1] - sy[2 * q];
+            zlo[q] = sz[2 * q] + sz[2 * q + 1];
+            zhi[q] = sz[2 * q + 1] - sz[2 * q];
+        }
+        M[0] = lo[0] + lo[1];
+        M[1] = hi[0] + hi[1];
+        M[2] = (lo[1] + ylo[1]) + (ylo[0] - lo[0]);
+        M[3] = (hi[1] + yhi[1]) + (yhi[0] - hi[0]);
+        Z[0] = zlo[0] + zlo[1];
+        Z[1] = zhi[0] + zhi[1];
+        Z[2] = zlo[1] - zlo[0];
+        Z[3] = zhi[1] - zhi[0];
+    }
+    // along z with the lane of the other side: this lane ends with S without z (hz = 0) or with z (1)
+    double r[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const double T = fma(hz ? 1.0 : -1.0, M[t], Z[t]);
+        const double give = hz ? M[t] : T, keep = hz ? T : M[t];
+        r[t] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+    }
+    // back to corners: r_c = sum_S sigma_{c,S} gamma^|S| M_S
+    {
+        const double a0 = fma(-gam, r[1], r[0]), a1 = fma(gam, r[1], r[0]), b0 = fma(-gam, r[3], r[2]), b1 = fma(gam, r[3], r[2]);
+        r[0] = fma(-gam, b0, a0);
+        r[1] = fma(-gam, b1, a1);
+        r[2] = fma(gam, b0, a0);
+        r[3] = fma(gam, b1, a1);
+    }
+    const double wq = A.lc[lv][6];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const double o = __shfl_xor_sync(0xffffffffu, r[t], 4);
+        r[t] = wq * (hz ? fma(gam, r[t], o) : fma(-gam, o, r[t]));
+        const int cr = t | (hz << 2);
+        const int32_t ic = __shfl_sync(0xffffffffu, id, (lane & ~7) | cr);
+        if (valid) {
+            if (A.sv) ((double*)A.sv)[32 * idx + 4 * cr + k] = r[t];
+            else scatter1(A, ic, k, r[t]);
+        }
+    }
+    __syncwarp();   // the rows and the exchange area are rewritten by later elements
+}
+
 // One Out element on 8 lanes of a warp (lane & 7 = corner c): the element's rows `nd` are in
 // shared memory (8 rows of CS, stride CS); the warp's moment rows s_mw [32][MSTR].  Thread c
 // transforms column c of the rows into monomial coefficients, evaluates Gauss point c (monomials m),
@@ -67,7 +235,12 @@ template <class T> struct IntShape {
 template <class T, bool JV, bool IL = (JV && sizeof(T) == 4)>
 __device__ __forceinline__ void interior_element(const Args& A, T* nd, T* s_mw, const T m[8], int lane, int64_t idx,
                                                  bool valid, int lv, int prob, int32_t id) {
-    typedef typename std::conditional<JV, Dual<T, sizeof(T) == 4>, T>::type S;
+    if constexpr (sizeof(T) == 8) {
+        interior_element64<JV>(A, nd, s_mw, lane, idx, valid, lv, prob, id);
+        return;
+    } else {
+    typedef Dual<T, 1> DT;
+    typedef typename std::conditional<JV, DT, T>::type S;
     constexpr int MSTR = IntShape<T>::MSTR;
     const int c = lane & 7;
     T* mrow = s_mw + lane * MSTR;
@@ -105,11 +278,11 @@ __device__ __forceinline__ void interior_element(const Args& A, T* nd, T* s_mw, 
     }
     for (int k = 0; k < 4; ++k) r[k] = hadamard_bwd<1>(r[k], c);
     if (A.sv) {
-        // deterministic scatter: node c's 4 rows into the element's slot (one 16- or 32-byte store)
+        // deterministic scatter: node c's 4 rows into the element's slot (one 16-byte store)
         if (valid) st4s<T>((T*)A.sv + 32 * idx + 4 * c, r[0], r[1], r[2], r[3]);
-    } else if constexpr (sizeof(T) == 4) {
+    } else {
         // corners of this warp's 4 elements that are the same node add their rows in shared memory
-        // first; one lane per node scatters (fewer float64 atomics; float64: the plain scatter is faster)
+        // first; one lane per node scatters (fewer float64 atomics)
         const unsigned grp = __match_any_sync(0xffffffffu, valid ? id : -1 - lane);
         __syncwarp();   // every lane has read its moment columns
         st4s<T>(mrow, r[0], r[1], r[2], r[3]);
@@ -123,10 +296,9 @@ __device__ __forceinline__ void interior_element(const Args& A, T* nd, T* s_mw, 
             }
             scatter_t(A, id, t);
         }
-    } else {
-        if (valid) scatter_t(A, id, r);
     }
     __syncwarp();   // the rows and the moments are rewritten by later elements
+    }
 }
 
 // Gauss point c of the 2x2x2 rule (xi_k = +-1/sqrt(3) by bit k of c) in monomial form

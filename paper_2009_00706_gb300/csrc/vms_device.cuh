@@ -88,6 +88,8 @@ template <class T, int K> __device__ __forceinline__ Dual<T, K> rcp(Dual<T, K> x
     return {r, -r * r * x.d};
 }
 
+constexpr double kInvGauss = 1.73205080756887729353;   // sqrt(3): 1 / Gauss abscissa
+
 template <class T> __device__ __forceinline__ T tiny();
 template <> __device__ __forceinline__ float tiny<float>() { return 1e-37f; }
 template <> __device__ __forceinline__ double tiny<double>() { return 1e-300; }
@@ -103,6 +105,7 @@ struct Args {
     double scale;
     float gf[16], wf[16];                // per level: 2/h and h^3/8 (Jacobian of the cube map)
     double gd[16], wd[16];
+    double lc[16][8];                    // per level, float64 kernels: see Const64
     const void* ndv;                     // node data [n_nodes + n_hang][8] of T: us(3), p, at(3), 0
     const void* ndt;                     // tangents  [n_nodes + n_hang][8] of T: dus(3), dp, dat(3), 0
     const void* ndf;                     // body force [n_nodes + n_hang][4] of T, or null
@@ -113,6 +116,7 @@ struct Args {
     const double* V;
     double* out;
     double rho, mu, theta, c0, c1, c2;   // c_k = time coefficients / dt
+    double c0th;                          // c0 / theta
     int theta1;                           // theta == 1
     const int* skip;                      // non-null and nonzero: return at once (solver steps captured in graphs)
     double K0dt;                         // 4 / dt^2
@@ -285,7 +289,6 @@ template <> __device__ __forceinline__ double to_t<double>(double x) { return x;
 
 // scatter one node's 4 values in the element precision: widened to float64 on the float64 unit,
 // which the element kernels leave idle while their integer pipe is busy
-__device__ __forceinline__ void scatter_t(const Args& A, int32_t id, const double r[4]) { scatter(A, id, r); }
 __device__ __forceinline__ void scatter_t(const Args& A, int32_t id, const float r[4]) {
     const double rd[4] = {(double)r[0], (double)r[1], (double)r[2], (double)r[3]};
     scatter(A, id, rd);
@@ -890,6 +893,150 @@ __device__ __forceinline__ void nitsche_rows(const Args& A, const NitschePoint<S
     t[3] = -(ph * P.dn);
 }
 
+// ------------------------------------------------------------------------------------------
+// Float64 elements.  The FP64 pipe issues a warp instruction about every 19 cycles per SM (measured
+// 1.05 TFLOP/s), so these kernels cost what their FP64 instructions cost: everything else (shared
+// memory, shuffles, integer work) runs beside them.  So:
+//   - fields are interpolated as tensor products, and 8-fold: u8 = sum_S a_S xi^S leaves the 1/8 of
+//     every monomial out of values, gradients and mixed derivatives alike, and the constants below
+//     take it up (fields 8 u, 8 p, ...; results 8 F, 8 S, ...; weights w / 64);
+//   - gradients stay in reference coordinates: g = 2/h enters where products are already formed;
+//   - the tangent of du/dt is c0 / theta times the tangent of u_s: never interpolated;
+//   - tau_C = sqrt(arg) / (3 g^2) takes the root of tau_M: no division.
+// ------------------------------------------------------------------------------------------
+struct Const64 {
+    double g, g8, g264, i3g2;   // 2/h, g/8, g^2/64, 1/(3 g^2)
+    double kap, kap8;           // scale of the gradient coefficients S, H (g, or g sqrt(3) when the test sums leave a gamma out), kap/8
+    double rho, irho, mug2, mgk, K, rhog;   // mu g^2 (0 without the viscous strong term), mu g kap, K0 + C_I nu^2 3 g^4, rho g
+    __device__ Const64(const Args& A, const Phys<double>& P, int lv, double kap_, double kap8_) {
+        g = A.lc[lv][0];
+        g8 = A.lc[lv][1];
+        g264 = A.lc[lv][2];
+        i3g2 = A.lc[lv][3];
+        kap = kap_;
+        kap8 = kap8_;
+        rho = P.rho;
+        irho = P.irho;
+        const double g2 = A.lc[lv][7];
+        mug2 = A.drop_visc ? 0.0 : P.mu * g2;
+        mgk = P.mu * (g * kap_);
+        K = fma(P.CI3, g2 * g2, P.K0);
+        rhog = P.rho * g;
+    }
+};
+
+// eight times the fields of a point (G, gp, H in reference coordinates; f = 8 x body force)
+struct Point64 {
+    double u[3], a[3], p, G[3][3], gp[3], H[3], f[3];
+};
+struct Tangent64 {
+    double u[3], p, G[3][3], gp[3], H[3];
+};
+
+// The 16 coefficients of a point, W = (F0, F1, F2, G, S00 .. S22, H0, H1, H2): 8 F, 8 G, and kap x 8
+// of S and H.  JV: their tangents; ratio = c0 / theta.  The operations of pointwise(), in the order that
+// takes the fewest FP64 instructions (113 for R, 219 for J v).
+template <bool JV>
+__device__ __forceinline__ void pointwise64(const Const64& C, bool force, double ratio, const Point64& F,
+                                            const Tangent64& D, double W[16]) {
+    double acc[3], rM[3], up[3], GU[3], c[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double conv = fma(F.G[i][2], F.u[2], fma(F.G[i][1], F.u[1], F.G[i][0] * F.u[0]));
+        acc[i] = fma(C.g8, conv, F.a[i]);
+        if (force) acc[i] -= F.f[i];
+        rM[i] = fma(C.rho, acc[i], fma(-C.mug2, F.H[i], C.g * F.gp[i]));
+    }
+    const double uu = fma(F.u[2], F.u[2], fma(F.u[1], F.u[1], F.u[0] * F.u[0]));
+    const double arg = fma(C.g264, uu, C.K);
+    const double r = rsqrt(arg);
+    const double tC = (arg * r) * C.i3g2;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) up[i] = -r * rM[i];
+    const double div = F.G[0][0] + F.G[1][1] + F.G[2][2];
+    const double q = C.g264 * fma(up[2], up[2], fma(up[1], up[1], up[0] * up[0]));
+    const double s = q > tiny<double>() ? rsqrt(q) : 0.0;
+    double w[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        GU[i] = C.g8 * fma(F.G[i][2], up[2], fma(F.G[i][1], up[1], F.G[i][0] * up[0]));
+        w[i] = -C.irho * up[i];
+        c[i] = fma(s, GU[i], w[i]);
+    }
+    double A[3];   // kap u'
+#pragma unroll
+    for (int i = 0; i < 3; ++i) A[i] = C.kap8 * up[i];
+    const double mp = tC * C.rhog;
+    if constexpr (!JV) {
+        const double P = C.kap * fma(-mp, div, F.p);   // kap (p + p')
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            W[i] = fma(C.rho, acc[i], GU[i]);
+            W[13 + i] = C.kap * w[i];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const double e = i == j ? fma(2.0 * C.mgk, F.G[i][i], -P) : C.mgk * (F.G[i][j] + F.G[j][i]);
+                W[4 + 3 * i + j] = fma(c[i], A[j], fma(-A[i], F.u[j], e));
+            }
+        }
+        W[3] = C.g * div;
+    } else {
+        double dacc[3], dup[3], dGU[3], dc[3], dA[3], dw[3];
+        const double h = (r * r) * (C.g264 * fma(F.u[2], D.u[2], fma(F.u[1], D.u[1], F.u[0] * D.u[0])));   // -dr / r
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            double dconv = F.G[i][0] * D.u[0];
+            dconv = fma(D.G[i][0], F.u[0], dconv);
+            dconv = fma(F.G[i][1], D.u[1], dconv);
+            dconv = fma(D.G[i][1], F.u[1], dconv);
+            dconv = fma(F.G[i][2], D.u[2], dconv);
+            dconv = fma(D.G[i][2], F.u[2], dconv);
+            dacc[i] = fma(ratio, D.u[i], C.g8 * dconv);
+            const double drM = fma(C.rho, dacc[i], fma(-C.mug2, D.H[i], C.g * D.gp[i]));
+            dup[i] = fma(-h, up[i], -r * drM);
+        }
+        const double ddiv = D.G[0][0] + D.G[1][1] + D.G[2][2];
+        const double hs = (s * s) * (C.g264 * fma(up[2], dup[2], fma(up[1], dup[1], up[0] * dup[0])));       // -ds / s
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            double t = F.G[i][0] * dup[0];
+            t = fma(D.G[i][0], up[0], t);
+            t = fma(F.G[i][1], dup[1], t);
+            t = fma(D.G[i][1], up[1], t);
+            t = fma(F.G[i][2], dup[2], t);
+            t = fma(D.G[i][2], up[2], t);
+            dGU[i] = C.g8 * t;
+            dw[i] = -C.irho * dup[i];
+            dc[i] = fma(s, fma(-hs, GU[i], dGU[i]), dw[i]);
+            dA[i] = C.kap8 * dup[i];
+        }
+        const double dP = C.kap * fma(-mp, fma(h, div, ddiv), D.p);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            W[i] = fma(C.rho, dacc[i], dGU[i]);
+            W[13 + i] = C.kap * dw[i];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                double e = i == j ? fma(2.0 * C.mgk, D.G[i][i], -dP) : C.mgk * (D.G[i][j] + D.G[j][i]);
+                e = fma(-dA[i], F.u[j], e);
+                e = fma(-A[i], D.u[j], e);
+                e = fma(dc[i], A[j], e);
+                W[4 + 3 * i + j] = fma(c[i], dA[j], e);
+            }
+        }
+        W[3] = C.g * ddiv;
+    }
+}
+
+// scatter one component of one node through M_e^T
+__device__ __forceinline__ void scatter1(const Args& A, int32_t id, int k, double r) {
+    if (id < A.n_nodes) { atomicAdd(A.out + 4 * (int64_t)id + k, r); return; }
+    const int32_t* hp = A.hpar + 4 * (int64_t)(id - A.n_nodes);
+    const int np = hp[2] >= 0 ? 4 : 2;
+    const double w = np == 4 ? 0.25 : 0.5;
+    for (int p = 0; p < np; ++p) atomicAdd(A.out + 4 * (int64_t)hp[p] + k, w * r);
+}
+
 // Launch arguments from the mesh and the caller's vectors (host side).
 inline Args make_args(const Mesh& m, const double* u, const double* up, const double* up2, const double* f,
                       const imga_physics& ph, const double* v, double* out) {
@@ -906,6 +1053,9 @@ inline Args make_args(const Mesh& m, const double* u, const double* up, const do
         A.wd[l] = 0.125 * h * h * h;
         A.gf[l] = (float)A.gd[l];
         A.wf[l] = (float)A.wd[l];
+        const double g = A.gd[l];
+        const double lc[8] = {g, 0.125 * g, g * g / 64.0, 1.0 / (3.0 * g * g), g * kInvGauss, 0.125 * g * kInvGauss, A.wd[l] / 64.0, g * g};
+        for (int k = 0; k < 8; ++k) A.lc[l][k] = lc[k];
     }
     A.ndv = A.ndt = A.ndf = nullptr;
     A.skip = nullptr;
@@ -926,6 +1076,7 @@ inline Args make_args(const Mesh& m, const double* u, const double* up, const do
     A.c1 = c[1] / ph.dt;
     A.c2 = c[2] / ph.dt;
     A.theta1 = A.theta == 1.0;
+    A.c0th = A.c0 / A.theta;
     A.K0dt = 4.0 / (ph.dt * ph.dt);
     const double nu = ph.mu / ph.rho;
     A.CInu2 = ph.C_I * nu * nu;
