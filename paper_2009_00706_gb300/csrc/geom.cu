@@ -485,6 +485,23 @@ bool device_cut_quadrature(Mesh& m, std::string& err) {
     return true;
 }
 
+// Intercepted list positions by decreasing number of 32-point rounds (counting sort), the order in which
+// the kernels take the elements by default: a long element that starts last would run on alone
+// (Eq. Wpart's cost model), and the slots make the result independent of the order.  12 spheres, mixed
+// J v (76 k Intercepted elements, 21 M points): 983 -> 815 us.
+static bool upload_cut_order(Mesh& m, std::string& err) {
+    const int64_t nc = (int64_t)m.cut_list.size();
+    auto rounds = [&](int64_t i) { return (m.cut_off[i + 1] - m.cut_off[i] + 31) / 32; };
+    int64_t most = 0;
+    for (int64_t i = 0; i < nc; ++i) most = std::max(most, rounds(i));
+    std::vector<int64_t> at(most + 2, 0);   // at[most - r + 1]: elements with r rounds
+    for (int64_t i = 0; i < nc; ++i) ++at[most - rounds(i) + 1];
+    for (int64_t r = 0; r <= most; ++r) at[r + 1] += at[r];
+    std::vector<int32_t> order((size_t)nc);
+    for (int64_t i = 0; i < nc; ++i) order[at[most - rounds(i)]++] = (int32_t)i;
+    return upload(&m.d.cut_order, order, err);
+}
+
 // Deterministic scatter (o2n of Algorithm 2 in a fixed order).  The element kernels write their
 // 8 x 4 contributions to slots: volume slots, one per Out element (out_list order) then one per
 // Intercepted element (cut_list order), in the element precision; surface slots in float64, one per
@@ -588,6 +605,7 @@ bool device_upload_quadrature(Mesh& m, std::string& err) {
         if (j == m.n_sq_sparse || el[j] != el[j - 1]) { sl.push_back(el[j]); so.push_back(j); }
     so.push_back(ns);
     m.n_sq_elem = (int64_t)sl.size();
+    if (!upload_cut_order(m, err)) return false;
     m.sq_off_h = so;
     m.sq_hosts.assign(el.begin(), el.end());
     std::sort(m.sq_hosts.begin(), m.sq_hosts.end());

@@ -96,7 +96,7 @@ struct DeviceMesh {
     double* sq_w = nullptr;
     double* sq_taub = nullptr;    // 1 / h_b
     int32_t* sq_src = nullptr;    // position of every surface point in the export order (imga_physics.g_points)
-    int32_t* cut_order = nullptr;   // Intercepted list positions by decreasing point count (autotuner)
+    int32_t* cut_order = nullptr;   // Intercepted list positions by decreasing number of 32-point rounds
     int32_t* sq_hosts = nullptr;  // every element hosting a surface point (increasing)
     // float64 Nitsche penalty per surface-hosting element (in device point order): element, point range
     // [pen_q[i], pen_q[i+1]), destination slot, and the packed upper triangle of sum_q (w_q/h_b) phi_a phi_b
@@ -201,7 +201,7 @@ struct Mesh {
     bool use_graphs = false;
     // Intercepted-element bucket: warps per block and element order (0 Morton, 1 longest first),
     // per [float64 0 / mixed 1][residual 0 / J v 1]; set by the autotuner
-    struct CutTune { int wpb = 4, lpt = 0; };
+    struct CutTune { int wpb = 4, lpt = 1; };
     CutTune cut_tune[2][2];
     float cut_tune_ms[2][2][6] = {};   // candidate times of the last tuning (ms per launch)
     bool tune_pending[2][2] = {{false, false}, {false, false}};

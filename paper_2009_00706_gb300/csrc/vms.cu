@@ -446,9 +446,170 @@ __device__ __forceinline__ void cut_element(const Args& A, const int32_t* __rest
     warp_scatter_moments<T>(A, M, s_m, lane, my_id, 0.0, A.sv ? (T*)A.sv + 32 * (A.n_out_slots + idx) : nullptr);
 }
 
+// ------------------------------------------------------------------------------------------
+// Intercepted elements in float64 (see Const64: FP64 instructions are the cost).  Per point the fields
+// come from the Hadamard coefficients by Horner steps along x, y, z, whose intermediates are the
+// gradients and mixed derivatives (11 or 12 multiply-adds per column; monomial by monomial 22), and the
+// 32 moments take the transposed steps (16 per component; 20 before).  An element's points are dealt
+// to four parts (part p: points 32 p + lane, + 128, ...) that different warps take, so the longest
+// element (8^(L_max + 1) points) is not one warp's serial work; each part sums its lanes, the parts are
+// added in order.  The fused kernel runs the same four parts on one warp: the same bits.
+//   7.3 k element sphere (234 k points in 776 elements), one R and one J v: 1.44 -> 0.53 ms.
+// ------------------------------------------------------------------------------------------
+constexpr int kCutParts = 4, kCutCols = 14;   // columns: 7 values, 4 tangents (u_s, p), 3 force
+
+// coefficient columns of element e, [column][8], by a block or warp of nt threads (a multiple of 32)
+template <bool JV>
+__device__ __forceinline__ void cut_columns64(const Args& A, int32_t e, double* s_col, int t0, int nt) {
+    for (int t = t0; t < 8 * kCutCols + 16; t += nt) {   // 4 x 32: whole warps (the shuffles)
+        const int col = t >> 3, c = t & 7;
+        const int64_t id = A.conn[8 * (int64_t)e + c];
+        double x = 0.0;
+        if (col < 7) x = __ldg((const double*)A.ndv + 8 * id + col);
+        else if (col < 11) { if (JV) x = __ldg((const double*)A.ndt + 8 * id + col - 7); }
+        else if (col < 14) { if (A.ndf) x = __ldg((const double*)A.ndf + 4 * id + col - 11); }
+        x = hadamard_fwd(x, c);
+        if (col < kCutCols) s_col[t] = x;
+    }
+}
+
+// lane's sum of moment row `lane` (4 S + k) over part p's points of the element, points [q0, q1)
+template <bool JV>
+__device__ __forceinline__ double cut_part64(const Args& A, const Const64& C, double det, const double* s_col,
+                                             const double* __restrict__ pts, int64_t q0, int64_t q1, int p, double* s_m, int lane) {
+    constexpr int MSTR = 34;
+    const int64_t first = q0 + 32 * p;
+    if (first >= q1) return 0.0;
+    double M[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) M[k] = 0.0;
+    for (int64_t q = first + lane; q < q1; q += 32 * kCutParts) {
+        double pt[4];
+        load_pt<double>(pts, q, pt);
+        const double x = pt[0], y = pt[1], z = pt[2];
+        Point64 F;
+        Tangent64 D;
+        auto value = [&](int col) {
+            const double* a = s_col + 8 * col;
+            const double b0 = fma(x, a[1], a[0]), b1 = fma(x, a[3], a[2]), b2 = fma(x, a[5], a[4]), b3 = fma(x, a[7], a[6]);
+            return fma(z, fma(y, b3, b2), fma(y, b1, b0));
+        };
+        // value, gradient and mixed second derivatives (xy, xz, yz)
+        auto all = [&](int col, double& v, double g[3], double m[3]) {
+            const double* a = s_col + 8 * col;
+            const double b0 = fma(x, a[1], a[0]), b1 = fma(x, a[3], a[2]), b2 = fma(x, a[5], a[4]), b3 = fma(x, a[7], a[6]);
+            const double c1 = fma(y, b3, b2), j = fma(y, a[7], a[5]);
+            v = fma(z, c1, fma(y, b1, b0));
+            g[2] = c1;
+            g[1] = fma(z, b3, b1);
+            g[0] = fma(z, j, fma(y, a[3], a[1]));
+            m[0] = fma(z, a[7], a[3]);
+            m[1] = j;
+            m[2] = b3;
+        };
+        {
+            double m[3][3], unused[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) all(i, F.u[i], F.G[i], m[i]);
+            F.H[0] = m[1][0] + m[2][1];
+            F.H[1] = m[0][0] + m[2][2];
+            F.H[2] = m[0][1] + m[1][2];
+            all(3, F.p, F.gp, unused);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) F.a[i] = value(4 + i);
+            if (A.ndf)
+                for (int i = 0; i < 3; ++i) F.f[i] = value(11 + i);
+            if (JV) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) all(7 + i, D.u[i], D.G[i], m[i]);
+                D.H[0] = m[1][0] + m[2][1];
+                D.H[1] = m[0][0] + m[2][2];
+                D.H[2] = m[0][1] + m[1][2];
+                all(10, D.p, D.gp, unused);
+            }
+        }
+        double W[16];
+        pointwise64<JV>(C, A.ndf != nullptr, A.c0th, F, D, W);
+        const double w = pt[3] * det, yz = y * z;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) W[k] *= w;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double f = W[k], sx = W[4 + 3 * k], sy = W[5 + 3 * k], sz = W[6 + 3 * k];
+            const double c = fma(z, f, sz), b = fma(y, f, sy), d = fma(y, c, z * sy);
+            M[k] += f;
+            M[4 + k] = fma(x, f, M[4 + k] + sx);
+            M[8 + k] += b;
+            M[12 + k] = fma(x, b, fma(y, sx, M[12 + k]));
+            M[16 + k] += c;
+            M[20 + k] = fma(x, c, fma(z, sx, M[20 + k]));
+            M[24 + k] += d;
+            M[28 + k] = fma(x, d, fma(yz, sx, M[28 + k]));
+        }
+    }
+    const int rows = (int)min((int64_t)32, q1 - first);   // lanes that had a point
+    double* mrow = s_m + lane * MSTR;
+#pragma unroll
+    for (int k = 0; k < 32; k += 2) *reinterpret_cast<double2*>(mrow + k) = make_double2(M[k], M[k + 1]);
+    __syncwarp();
+    double acc = s_m[lane];
+    for (int t = 1; t < rows; ++t) acc += s_m[t * MSTR + lane];
+    __syncwarp();
+    return acc;
+}
+
+// rows of the element from the summed moments (lane 4 a + k: node a, component k) to its slot or the nodes
+__device__ __forceinline__ void cut_rows64(const Args& A, int32_t e, int64_t idx, double acc, int lane) {
+    acc = hadamard_bwd<4>(acc, lane >> 2);
+    if (A.sv) ((double*)A.sv)[32 * (A.n_out_slots + idx) + lane] = acc;
+    else scatter1(A, A.conn[8 * (int64_t)e + (lane >> 2)], lane & 3, acc);
+}
+
+__device__ __forceinline__ int cut_parts(int64_t points) { return (int)min((int64_t)kCutParts, (points + 31) / 32); }
+
+// a block of W warps per element (warp w: parts w, w + W, ...)
+template <bool JV, int W>
+__global__ void __launch_bounds__(32 * W, 8 / W) vms_cut64(Args A, const int32_t* __restrict__ list, const int64_t* __restrict__ off,
+                                                          const double* __restrict__ pts, const int32_t* __restrict__ order) {
+    __shared__ __align__(16) double s_col[8 * kCutCols], s_m[W][32 * 34], s_part[kCutParts][32];
+    if (A.skip && *A.skip) return;   // a captured solver step after its cycle ended
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t idx = order ? (int64_t)order[blockIdx.x] : blockIdx.x;
+    const int32_t e = list[idx];
+    cut_columns64<JV>(A, e, s_col, threadIdx.x, 32 * W);
+    const int64_t q0 = off[idx], q1 = off[idx + 1];
+    const int lv = A.lev[e];
+    const Const64 C(A, Phys<double>(A, prob_of(A, e)), lv, A.lc[lv][0], A.lc[lv][1]);
+    __syncthreads();
+    for (int p = w; p < kCutParts; p += W) s_part[p][lane] = cut_part64<JV>(A, C, A.lc[lv][6], s_col, pts, q0, q1, p, s_m[w], lane);
+    __syncthreads();
+    if (w > 0) return;
+    double acc = s_part[0][lane];
+    for (int p = 1, np = cut_parts(q1 - q0); p < np; ++p) acc += s_part[p][lane];
+    cut_rows64(A, e, idx, acc, lane);
+}
+
+// the same element on one warp (fused kernel); s: 8 kCutCols + 32 x 34 doubles of the warp
+template <bool JV>
+__device__ __forceinline__ void cut_element64(const Args& A, const int32_t* __restrict__ list, const int64_t* __restrict__ off,
+                                              const double* __restrict__ pts, int64_t idx, double* s, int lane) {
+    const int32_t e = list[idx];
+    cut_columns64<JV>(A, e, s, lane, 32);
+    const int64_t q0 = off[idx], q1 = off[idx + 1];
+    const int lv = A.lev[e];
+    const Const64 C(A, Phys<double>(A, prob_of(A, e)), lv, A.lc[lv][0], A.lc[lv][1]);
+    __syncwarp();
+    double acc = 0.0;
+    for (int p = 0, np = cut_parts(q1 - q0); p < np; ++p) {
+        const double x = cut_part64<JV>(A, C, A.lc[lv][6], s, pts, q0, q1, p, s + 8 * kCutCols, lane);
+        acc = p == 0 ? x : acc + x;
+    }
+    cut_rows64(A, e, idx, acc, lane);
+}
+
 // W warps per block (a tile shape the autotuner picks); `order` (or null) permutes the list
 template <class T, bool JV, int W>
-__global__ void __launch_bounds__(32 * W, (sizeof(T) == 4 ? 16 : 8) / W) vms_cut(Args A, const int32_t* __restrict__ list,
+__global__ void __launch_bounds__(32 * W, 16 / W) vms_cut(Args A, const int32_t* __restrict__ list,
                                                     const int64_t* __restrict__ off, const void* __restrict__ pts,
                                                     const int32_t* __restrict__ order, int64_t n) {
     constexpr int PAD = 16 / (int)sizeof(T), MSTR = 32 + PAD;
@@ -652,7 +813,7 @@ template <class T> struct FusedShape {
     // per warp: the Out layout (2 buffers x 4 elements of rows, 32 moment rows); the per-element
     // layouts (8 rows, 32 moment rows) fit inside it
     static constexpr int WARP = 2 * 4 * ESTR + 32 * MSTR;
-    static_assert(8 * CS + 32 * MSTR <= WARP, "per-element layout");
+    static_assert(8 * CS + 32 * MSTR <= WARP && 8 * kCutCols + 32 * 34 <= WARP, "per-element layout");
     static_assert((WARP * sizeof(T)) % 16 == 0 && (8 * CS * sizeof(T)) % 16 == 0, "16-byte rows");
     static constexpr size_t smem = (size_t)kFusedWarps * WARP * sizeof(T);
 };
@@ -671,7 +832,10 @@ __global__ void __launch_bounds__(32 * kFusedWarps, sizeof(T) == 4 ? 4 : 2) vms_
             if (lane == 0) h = atomicAdd(Q.cnt, 1ull);
             h = __shfl_sync(0xffffffffu, h, 0);
             if ((int64_t)h >= Q.n_items) break;
-            cut_element<T, JV>(A, Q.cut_list, Q.cut_off, Q.cut_pts, (int64_t)Q.items[h], base, base + 8 * CS, lane);
+            if constexpr (sizeof(T) == 8)
+                cut_element64<JV>(A, Q.cut_list, Q.cut_off, (const double*)Q.cut_pts, (int64_t)Q.items[h], base, lane);
+            else
+                cut_element<T, JV>(A, Q.cut_list, Q.cut_off, Q.cut_pts, (int64_t)Q.items[h], base, base + 8 * CS, lane);
             __syncwarp();   // the shared rows are reused by the next item
         }
     };
@@ -1050,17 +1214,17 @@ struct Timed {
 template <class T, bool JV>
 void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt) {
     const int64_t nc = (int64_t)m.cut_list.size();
-    const void* pts = std::is_same<T, float>::value ? (const void*)m.d.cut_pts_f : (const void*)m.d.cut_pts;
     const int32_t* order = lpt ? m.d.cut_order : nullptr;
-    switch (wpb) {
-        case 2: vms_cut<T, JV, 2><<<(unsigned)((nc + 1) / 2), 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
-        case 8:
-            if constexpr (sizeof(T) == 4) {
-                vms_cut<T, JV, 8><<<(unsigned)((nc + 7) / 8), 256, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc);
-                break;
-            }
-            [[fallthrough]];
-        default: vms_cut<T, JV, 4><<<(unsigned)((nc + 3) / 4), 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc);
+    if constexpr (sizeof(T) == 8) {
+        if (wpb == 2) vms_cut64<JV, 2><<<(unsigned)nc, 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
+        else vms_cut64<JV, 4><<<(unsigned)nc, 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
+    } else {
+        const void* pts = m.d.cut_pts_f;
+        switch (wpb) {
+            case 2: vms_cut<T, JV, 2><<<(unsigned)((nc + 1) / 2), 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
+            case 8: vms_cut<T, JV, 8><<<(unsigned)((nc + 7) / 8), 256, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
+            default: vms_cut<T, JV, 4><<<(unsigned)((nc + 3) / 4), 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc);
+        }
     }
 }
 
@@ -1078,16 +1242,6 @@ int autotune_cut(Mesh& m, Args A, cudaStream_t s) {
     const int64_t nc = (int64_t)m.cut_list.size();
     Mesh::CutTune& ct = m.cut_tune[sizeof(T) == 4][JV];
     m.tune_pending[sizeof(T) == 4][JV] = false;
-    if (nc > 0 && !m.d.cut_order) {   // longest first: positions of the list by decreasing point count
-        std::vector<int32_t> ord(nc);
-        for (int64_t i = 0; i < nc; ++i) ord[i] = (int32_t)i;
-        std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) {
-            return m.cut_off[a + 1] - m.cut_off[a] > m.cut_off[b + 1] - m.cut_off[b];
-        });
-        if (cudaMalloc((void**)&m.d.cut_order, nc * sizeof(int32_t)) != cudaSuccess ||
-            cudaMemcpy(m.d.cut_order, ord.data(), nc * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
-            return 1;
-    }
     const int64_t next = m.n_nodes() + m.n_hang();
     T* ndv = node_workspace<T>(m, nullptr);
     A.ndv = ndv;

@@ -110,3 +110,24 @@ def test_mlp_gradient_rows(dev, rows, batch, nin, nout):
         assert float((T(a, dev) - b).norm() / b.norm()) <= 1e-2, k
     first = net.train(X, Y, epochs=1, batch=batch, lr=1e-3)[0]
     assert net.train(X, Y, epochs=8, batch=batch, lr=1e-3)[-1] < first
+
+
+# ---- float64 Intercepted elements: a block's four parts of 32 points at a time, from elements with a
+# few points (less than one part) to 8^4 of them, slots and atomics, all fields in use ----
+@pytest.mark.parametrize("lmax", [0, 1, 3])
+@pytest.mark.parametrize("scheme", [I.SCHEME_BE, I.SCHEME_CN, I.SCHEME_BDF2])
+def test_float64_cut_elements(dev, lmax, scheme):
+    g, o = pair(I.icosphere(2, 0.2, C, 1e-3, 5), 4, lmax=lmax)
+    off, _ = g.cut_points()
+    per = np.diff(off)[np.diff(off) > 0]
+    assert {0: per.max() <= 8, 1: per.min() < 32 < per.max(), 3: per.max() > 1000}[lmax]
+    ph = I.Physics(mu=0.01, dt=0.02, scheme=scheme, g=(0.1, 0.0, -0.2))
+    u, up, v = I.state(g.n_nodes, 3)
+    up2, f = up + 0.01 * v, 0.3 * v[:, [1, 2, 3, 0]]
+    Ro, Jo = o.residual_jvp(ph, u, up, up2, f, v)
+    a = [T(x, dev) for x in (u, up, v, up2, f)]
+    for det in (True, False):
+        g.deterministic(det)
+        R = g.residual(ph, a[0], a[1], a[3], f=a[4]).cpu().numpy()
+        J = g.jvp(ph, a[0], a[1], a[2], a[3], f=a[4]).cpu().numpy()
+        assert rel(R, Ro) <= TOL64 and rel(J, Jo) <= TOL64
