@@ -7,6 +7,7 @@
 // pointwise VMS coefficients are differentiated exactly (dual numbers), weighted and contracted
 // with the test functions.  No global matrix is ever formed.
 //
+//   float64: jac_out64, jac_cut64, jac_surf64 (lane = column of k_e); float32 element arithmetic:
 //   jac_out     8 threads per Out element (thread c: Gauss point c, then node c's 4 rows)
 //   jac_cut     one warp per Intercepted element, 32 sub-cell points per step, lane = row
 //   jac_nitsche one thread per surface point
@@ -121,7 +122,7 @@ __device__ __forceinline__ void add_diag(const Args& A, int32_t id, const double
         for (int q = 0; q < 16; ++q) atomicAdd(D + 16 * (int64_t)hp[p] + q, w2 * blk[q]);
 }
 
-template <class T> struct JacShape { static constexpr int EPB = sizeof(T) == 8 ? 8 : 16; };
+template <class T> struct JacShape { static constexpr int EPB = 16; };
 
 template <class T, int MODE>
 __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const int32_t* __restrict__ list, int64_t n,
@@ -335,6 +336,474 @@ __global__ void __launch_bounds__(128) jac_nitsche(Args A, const int32_t* __rest
     }
 }
 
+// ------------------------------------------------------------------------------------------
+// Float64: a warp per element part, lane = column (corner b, component k) of k_e.  The FP64 pipe is the
+// bound (see Const64), so what does not depend on the column is formed once per point, with a lane per
+// point (fields by Horner steps, the value part of the pointwise terms: about 165 FP64 instructions for 32
+// points), and kept in shared memory; the columns then differentiate around those values with a seed
+// whose zeros are spelled out (100 per point) and add their 32 test moments in registers (80).  The
+// seed-by-seed dual numbers of the float32 kernels below took about 900 per point.
+//   jac_out64   four Out elements per warp: 4 x 8 Gauss points at once, then the elements in turn
+//   jac_cut64   a block of four warps per Intercepted element, 32 sub-cell points per warp at a time
+//   jac_surf64  a warp per element hosting surface points: no atomics between its points
+// 8,192 of 27 k elements (a ninth of them Intercepted, 288 points each): 35.8 -> 4.5 ms.
+// ------------------------------------------------------------------------------------------
+enum { JX = 0, JU = 3, JG = 6, JUP = 15, JGU = 18, JC = 21, JA = 24, JQ = 27, JDIV = 31, JS = 32, JS2 = 33, JNRR = 34,
+       JNRG = 35, JNRM = 36, JMP = 37, JWM = 38, JN = 46 };
+constexpr int JSTR = 33;             // point stride of a stored quantity
+constexpr int JWARP = JN * JSTR;     // doubles of a warp's point area
+
+// value columns of element e as Hadamard coefficients, [column][8] (columns 7-9: force)
+__device__ __forceinline__ void jac_columns64(const Args& A, int32_t e, double* s_col, int t0, int nt) {
+    for (int t = t0; t < 96; t += nt) {
+        const int col = t >> 3, c = t & 7;
+        const int64_t id = A.conn[8 * (int64_t)e + c];
+        double x = 0.0;
+        if (col < 7) x = __ldg((const double*)A.ndv + 8 * id + col);
+        else if (col < 10 && A.ndf) x = __ldg((const double*)A.ndf + 4 * id + col - 7);
+        s_col[t] = hadamard_fwd(x, c);
+    }
+}
+
+// the column-independent quantities of a point (8-fold fields), stored at s[.. * JSTR]; w: its weight / 64
+__device__ __forceinline__ void jac_point64(const Args& A, const Const64& C, const double* s_col, double x, double y, double z,
+                                            double w, double* s) {
+    auto value = [&](int col) {
+        const double* a = s_col + 8 * col;
+        const double b0 = fma(x, a[1], a[0]), b1 = fma(x, a[3], a[2]), b2 = fma(x, a[5], a[4]), b3 = fma(x, a[7], a[6]);
+        return fma(z, fma(y, b3, b2), fma(y, b1, b0));
+    };
+    double u[3], G[3][3], p, gp[3], H[3], m[3][3], none[3];
+    auto all = [&](int col, double& v, double g[3], double d2[3]) {   // as in the Intercepted J v kernel
+        const double* a = s_col + 8 * col;
+        const double b0 = fma(x, a[1], a[0]), b1 = fma(x, a[3], a[2]), b2 = fma(x, a[5], a[4]), b3 = fma(x, a[7], a[6]);
+        const double c1 = fma(y, b3, b2), j = fma(y, a[7], a[5]);
+        v = fma(z, c1, fma(y, b1, b0));
+        g[2] = c1;
+        g[1] = fma(z, b3, b1);
+        g[0] = fma(z, j, fma(y, a[3], a[1]));
+        d2[0] = fma(z, a[7], a[3]);
+        d2[1] = j;
+        d2[2] = b3;
+    };
+    for (int i = 0; i < 3; ++i) all(i, u[i], G[i], m[i]);
+    H[0] = m[1][0] + m[2][1];
+    H[1] = m[0][0] + m[2][2];
+    H[2] = m[0][1] + m[1][2];
+    all(3, p, gp, none);
+    double Gg[3][3], rM[3], up[3], GU[3];
+    for (int i = 0; i < 3; ++i) {
+        for (int j = 0; j < 3; ++j) Gg[i][j] = C.g8 * G[i][j];
+        double acc = fma(Gg[i][2], u[2], fma(Gg[i][1], u[1], fma(Gg[i][0], u[0], value(4 + i))));
+        if (A.ndf) acc -= value(7 + i);
+        rM[i] = fma(C.rho, acc, fma(-C.mug2, H[i], C.g * gp[i]));
+    }
+    const double arg = fma(C.g264, fma(u[2], u[2], fma(u[1], u[1], u[0] * u[0])), C.K);
+    const double r = rsqrt(arg), tC = (arg * r) * C.i3g2;
+    for (int i = 0; i < 3; ++i) up[i] = -r * rM[i];
+    const double q = C.g264 * fma(up[2], up[2], fma(up[1], up[1], up[0] * up[0]));
+    const double sb = q > tiny<double>() ? rsqrt(q) : 0.0;
+    const double rg = (r * r) * C.g264;
+    s[JX * JSTR] = x;
+    s[(JX + 1) * JSTR] = y;
+    s[(JX + 2) * JSTR] = z;
+    for (int i = 0; i < 3; ++i) {
+        GU[i] = fma(Gg[i][2], up[2], fma(Gg[i][1], up[1], Gg[i][0] * up[0]));
+        s[(JU + i) * JSTR] = u[i];
+        for (int j = 0; j < 3; ++j) s[(JG + 3 * i + j) * JSTR] = Gg[i][j];
+        s[(JUP + i) * JSTR] = up[i];
+        s[(JGU + i) * JSTR] = GU[i];
+        s[(JC + i) * JSTR] = fma(sb, GU[i], -C.irho * up[i]);
+        s[(JA + i) * JSTR] = C.kap8 * up[i];
+        s[(JQ + i) * JSTR] = rg * u[i];
+    }
+    s[(JQ + 3) * JSTR] = 0.0;
+    s[JDIV * JSTR] = G[0][0] + G[1][1] + G[2][2];
+    s[JS * JSTR] = sb;
+    s[JS2 * JSTR] = (sb * sb) * C.g264;
+    s[JNRR * JSTR] = -r * C.rho;
+    s[JNRG * JSTR] = -r * C.g;
+    s[JNRM * JSTR] = r * C.mug2;
+    s[JMP * JSTR] = C.kap * (tC * C.rhog);
+    const double wx = w * x, wy = w * y, wxy = wx * y;
+    const double wm[8] = {w, wx, wy, wxy, w * z, wx * z, wy * z, wxy * z};
+    for (int t = 0; t < 8; ++t) s[(JWM + t) * JSTR] = wm[t];
+}
+
+// 8-fold basis function of corner b at (x, y, z): phi, reference gradient d, mixed second derivatives (xy, xz, yz)
+__device__ __forceinline__ void jac_seed64(int b, double x, double y, double z, double& phi, double d[3], double m[3]) {
+    const double fx = (b & 1) ? 1.0 + x : 1.0 - x, fy = (b & 2) ? 1.0 + y : 1.0 - y, fz = (b & 4) ? 1.0 + z : 1.0 - z;
+    const double fyz = fy * fz, fxz = fx * fz, fxy = fx * fy;
+    phi = fx * fyz;
+    d[0] = (b & 1) ? fyz : -fyz;
+    d[1] = (b & 2) ? fxz : -fxz;
+    d[2] = (b & 4) ? fxy : -fxy;
+    m[0] = (((b >> 1) ^ b) & 1) ? -fz : fz;
+    m[1] = (((b >> 2) ^ b) & 1) ? -fy : fy;
+    m[2] = (((b >> 2) ^ (b >> 1)) & 1) ? -fx : fx;
+}
+
+// moments of one column's coefficients: f, s of component i with weighted monomials m
+__device__ __forceinline__ void jac_moments64(const double m[8], int i, double f, double sx, double sy, double sz, double M[32]) {
+    auto add = [&](int S, double a, double v) { M[4 * S + i] = fma(a, v, M[4 * S + i]); };
+    add(0, m[0], f);
+    add(1, m[1], f); add(1, m[0], sx);
+    add(2, m[2], f); add(2, m[0], sy);
+    add(3, m[3], f); add(3, m[2], sx); add(3, m[1], sy);
+    add(4, m[4], f); add(4, m[0], sz);
+    add(5, m[5], f); add(5, m[4], sx); add(5, m[1], sz);
+    add(6, m[6], f); add(6, m[4], sy); add(6, m[2], sz);
+    add(7, m[7], f); add(7, m[6], sx); add(7, m[5], sy); add(7, m[3], sz);
+}
+
+// Column (b, k) at the stored point s, theta left out (the finished column is scaled): the derivative for
+// the seed du_k = phi, or dp = phi.  DIAG: adds the four rows of corner b itself to M[0 .. 4), else the
+// 32 test moments.
+template <bool DIAGM>
+__device__ __forceinline__ void jac_column64(const Const64& C, double ratio, const double* s, int b, int k, double* M) {
+    auto ld = [&](int f) { return s[f * JSTR]; };
+    double phi, d[3], m[3];
+    jac_seed64(b, ld(JX), ld(JX + 1), ld(JX + 2), phi, d, m);
+    const bool isp = k == 3;
+    const double X = fma(C.g8, fma(d[2], ld(JU + 2), fma(d[1], ld(JU + 1), d[0] * ld(JU))), ratio * phi);
+    const double phiv = isp ? 0.0 : phi;
+    const int kk = isp ? 0 : k;
+    // grad p, or the mixed derivatives of u_k that enter (grad div u)_i, i != k
+    const double v[3] = {k == 1 ? m[0] : k == 2 ? m[1] : isp ? d[0] : 0.0, k == 0 ? m[0] : k == 2 ? m[2] : isp ? d[1] : 0.0,
+                         k == 0 ? m[1] : k == 1 ? m[2] : isp ? d[2] : 0.0};
+    const double coef = s[(isp ? JNRG : JNRM) * JSTR], h = s[(JQ + k) * JSTR] * phi, nrr = ld(JNRR);
+    double dacc[3], dup[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        dacc[i] = fma(s[(JG + 3 * i + kk) * JSTR], phiv, i == k ? X : 0.0);
+        dup[i] = fma(nrr, dacc[i], fma(-h, ld(JUP + i), coef * v[i]));
+    }
+    const double hs = ld(JS2) * fma(ld(JUP + 2), dup[2], fma(ld(JUP + 1), dup[1], ld(JUP) * dup[0]));
+    const double t2 = C.g8 * fma(d[2], ld(JUP + 2), fma(d[1], ld(JUP + 1), d[0] * ld(JUP)));
+    const double ddiv = k == 0 ? d[0] : k == 1 ? d[1] : k == 2 ? d[2] : 0.0;
+    const double kphi = C.kap * phi;
+    const double dP = fma(-ld(JMP), fma(h, ld(JDIV), ddiv), isp ? kphi : 0.0);
+    double F[3], dc[3], dA[3], Hh[3], mj[3], tk[3];
+    const double sb = ld(JS);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double dGU = fma(ld(JG + 3 * i), dup[0], fma(ld(JG + 3 * i + 1), dup[1], fma(ld(JG + 3 * i + 2), dup[2], i == k ? t2 : 0.0)));
+        F[i] = fma(C.rho, dacc[i], dGU);
+        const double dw = -C.irho * dup[i];
+        dc[i] = fma(sb, fma(-hs, ld(JGU + i), dGU), dw);
+        dA[i] = C.kap8 * dup[i];
+        Hh[i] = C.kap * dw;
+        mj[i] = C.mgk * d[i];
+        tk[i] = fma(-ld(JA + i), phi, mj[i]);
+    }
+    double m8[8], ph4 = 0.0, g4[3] = {0.0, 0.0, 0.0};
+    if (DIAGM) {
+        ph4 = ld(JWM) * phi;
+        for (int j = 0; j < 3; ++j) g4[j] = ld(JWM) * d[j];
+    } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) m8[t] = ld(JWM + t);
+    }
+    auto put = [&](int i, double f, double sx, double sy, double sz) {
+        if (DIAGM) M[i] = fma(ph4, f, fma(g4[0], sx, fma(g4[1], sy, fma(g4[2], sz, M[i]))));
+        else jac_moments64(m8, i, f, sx, sy, sz, M);
+    };
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double S[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            // mu (dG_ij + dG_ji) - u'_i du_j, and the pressure on the diagonal
+            double e = j == k ? tk[i] : i == k ? mj[j] : 0.0;
+            if (i == j) e = (i == k ? e + mj[i] : e) - dP;
+            S[j] = fma(-dA[i], ld(JU + j), fma(dc[i], ld(JA + j), fma(ld(JC + i), dA[j], e)));
+        }
+        put(i, F[i], S[0], S[1], S[2]);
+    }
+    put(3, C.g * ddiv, Hh[0], Hh[1], Hh[2]);
+}
+
+// test moments -> rows of the 8 corners (one column per lane), velocity columns times theta
+__device__ __forceinline__ void jac_rows64(const Args& A, int k, double M[32]) {
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+            if (!(t & (1 << ax)))
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double lo = M[4 * t + i], hi = M[4 * (t | (1 << ax)) + i];
+                    M[4 * t + i] = lo - hi;
+                    M[4 * (t | (1 << ax)) + i] = lo + hi;
+                }
+    if (!A.theta1 && k < 3)
+        for (int t = 0; t < 32; ++t) M[t] *= A.theta;
+}
+
+// the warp's finished columns: FULL to K (add: onto what is there), BSR into the assembled blocks through
+// M_e (one search of the row per corner pair, not per entry), DIAG (M[0 .. 4): corner b's own rows) to D
+template <int MODE>
+__device__ __forceinline__ void jac_store64(const Args& A, int32_t e, int64_t sl, double* M, int lane, double* __restrict__ K,
+                                            double* __restrict__ D, bool add) {
+    const int b = lane >> 2, k = lane & 3;
+    if (MODE == FULL) {
+        double* o = K + sl * 1024 + lane;
+#pragma unroll
+        for (int r = 0; r < 32; ++r) o[32 * r] = add ? o[32 * r] + M[r] : M[r];
+        return;
+    }
+    int32_t nb[4];
+    double wb;
+    const int cb = corner_nodes(A, A.conn[8 * (int64_t)e + b], nb, wb);
+    if (MODE == DIAG) {
+        for (int p = 0; p < cb; ++p)
+            for (int i = 0; i < 4; ++i) atomicAdd(D + 16 * (int64_t)nb[p] + 4 * i + k, wb * wb * M[i]);
+        return;
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+        int32_t na[4];
+        double wa;
+        const int ca = corner_nodes(A, A.conn[8 * (int64_t)e + a], na, wa);
+        for (int p = 0; p < ca; ++p)
+            for (int q = 0; q < cb; ++q) {
+                const int64_t pos = bsr_find(A.bptr, A.bidx, na[p], nb[q]);
+                if (pos < 0) continue;
+                double* o = K + 16 * pos + k;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (M[4 * a + i] != 0.0) atomicAdd(o + 4 * i, wa * wb * M[4 * a + i]);
+            }
+    }
+}
+
+template <int MODE> struct JacAcc { static constexpr int n = MODE == DIAG ? 4 : 32; };
+
+constexpr int J64W = 4;   // warps per block
+inline size_t jac64_smem() { return (size_t)J64W * (JWARP + 4 * 96) * sizeof(double); }
+
+// list: the Out elements, or (FULL) the requested elements, of which this kernel takes the Out ones
+template <int MODE>
+__global__ void __launch_bounds__(32 * J64W, 2) jac_out64(Args A, const int32_t* __restrict__ list, int64_t n,
+                                                         const int8_t* __restrict__ marker, const int32_t* __restrict__ slot,
+                                                         double* __restrict__ K, double* __restrict__ D) {
+    extern __shared__ __align__(16) double sm[];
+    const int lane = threadIdx.x & 31, le = lane >> 3, w = threadIdx.x >> 5;
+    double* s = sm + w * (JWARP + 4 * 96);
+    double* s_col = s + JWARP;
+    const int64_t i0 = ((int64_t)blockIdx.x * J64W + w) * 4;
+    if (i0 >= n) return;
+    auto takes = [&](int64_t i) {   // element of position i if it is ours, else -1
+        if (i >= n) return -1;
+        const int32_t e = list[i];
+        return MODE != FULL || (marker[e] == 0 && slot[e] == (int32_t)i) ? e : -1;
+    };
+    const int32_t mine = takes(i0 + le);
+    if (!__any_sync(0xffffffffu, mine >= 0)) return;
+    for (int q = 0; q < 4; ++q) {
+        const int32_t e = __shfl_sync(0xffffffffu, mine, 8 * q);
+        if (e >= 0) jac_columns64(A, e, s_col + 96 * q, lane, 32);
+    }
+    __syncwarp();
+    if (mine >= 0) {
+        const int lv = A.lev[mine];
+        const Const64 C(A, Phys<double>(A, prob_of(A, mine)), lv, A.lc[lv][0], A.lc[lv][1]);
+        const double gam = 1.0 / kInvGauss;
+        jac_point64(A, C, s_col + 96 * le, (lane & 1) ? gam : -gam, (lane & 2) ? gam : -gam, (lane & 4) ? gam : -gam,
+                    A.lc[lv][6], s + lane);
+    }
+    __syncwarp();
+    const int b = lane >> 2, k = lane & 3;
+    for (int q = 0; q < 4; ++q) {
+        const int32_t e = __shfl_sync(0xffffffffu, mine, 8 * q);
+        if (e < 0) continue;
+        const int lv = A.lev[e];
+        const Const64 C(A, Phys<double>(A, prob_of(A, e)), lv, A.lc[lv][0], A.lc[lv][1]);
+        double M[JacAcc<MODE>::n];
+#pragma unroll
+        for (int t = 0; t < JacAcc<MODE>::n; ++t) M[t] = 0.0;
+        for (int j = 0; j < 8; ++j) jac_column64<MODE == DIAG>(C, A.c0th, s + 8 * q + j, b, k, M);
+        if constexpr (MODE == DIAG) {
+            if (!A.theta1 && k < 3)
+                for (int t = 0; t < 4; ++t) M[t] *= A.theta;
+        } else {
+            jac_rows64(A, k, M);
+        }
+        jac_store64<MODE>(A, e, i0 + q, M, lane, K, D, false);
+    }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(32 * J64W, 2) jac_cut64(Args A, const int32_t* __restrict__ list, const int64_t* __restrict__ off,
+                                                         const double* __restrict__ pts, const int32_t* __restrict__ order,
+                                                         const int32_t* __restrict__ slot, double* __restrict__ K,
+                                                         double* __restrict__ D) {
+    extern __shared__ __align__(16) double sm[];
+    constexpr int NA = JacAcc<MODE>::n;
+    static_assert(32 * 32 <= JWARP, "the parts' sums take the point areas");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t idx = order[blockIdx.x];
+    const int32_t e = list[idx];
+    const int64_t sl = MODE == FULL ? slot[e] : 0;
+    if (sl < 0) return;
+    double *s = sm + w * JWARP, *s_col = sm + J64W * JWARP;
+    jac_columns64(A, e, s_col, threadIdx.x, 32 * J64W);
+    const int lv = A.lev[e];
+    const Const64 C(A, Phys<double>(A, prob_of(A, e)), lv, A.lc[lv][0], A.lc[lv][1]);
+    const int64_t q0 = off[idx], q1 = off[idx + 1];
+    const int b = lane >> 2, k = lane & 3;
+    double M[NA];
+#pragma unroll
+    for (int t = 0; t < NA; ++t) M[t] = 0.0;
+    __syncthreads();
+    for (int64_t base = q0 + 32 * w; base < q1; base += 32 * J64W) {
+        const int cnt = (int)min((int64_t)32, q1 - base);
+        if (lane < cnt) {
+            double pt[4];
+            load_pt<double>(pts, base + lane, pt);
+            jac_point64(A, C, s_col, pt[0], pt[1], pt[2], pt[3] * A.lc[lv][6], s + lane);
+        }
+        __syncwarp();
+        for (int j = 0; j < cnt; ++j) jac_column64<MODE == DIAG>(C, A.c0th, s + j, b, k, M);
+        __syncwarp();
+    }
+    // the warps' sums in order (the point areas are free)
+#pragma unroll
+    for (int t = 0; t < NA; ++t) s[32 * t + lane] = M[t];
+    __syncthreads();
+    if (w > 0) return;
+    for (int p = 1; p < J64W && q0 + 32 * p < q1; ++p)
+#pragma unroll
+        for (int t = 0; t < NA; ++t) M[t] += sm[p * JWARP + 32 * t + lane];
+    if constexpr (MODE == DIAG) {
+        if (!A.theta1 && k < 3)
+            for (int t = 0; t < 4; ++t) M[t] *= A.theta;
+    } else {
+        jac_rows64(A, k, M);
+    }
+    jac_store64<MODE>(A, e, sl, M, lane, K, D, false);
+}
+
+// Surface terms (rows of nitsche_rows) of a host element: points [pq[i], pq[i + 1]) of element pe[i]; runs
+// after the volume kernels (FULL: adds to their k_e)
+template <int MODE>
+__global__ void __launch_bounds__(128) jac_surf64(Args A, const int32_t* __restrict__ pe, const int64_t* __restrict__ pq,
+                                                  const double* __restrict__ xr, const double* __restrict__ nr,
+                                                  const double* __restrict__ wr, const double* __restrict__ taub, int64_t n,
+                                                  const int32_t* __restrict__ slot, double* __restrict__ K, double* __restrict__ D) {
+    __shared__ double s_col[4][96], s_pt[4][8][JSTR];   // point: velocity jump (0-2), u.n / |rho, inflow| (3), weight (4), tau_B (5)
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 4 + w;
+    if (i >= n) return;
+    const int32_t e = pe[i];
+    const int64_t sl = MODE == FULL ? slot[e] : 0;
+    if (sl < 0) return;
+    jac_columns64(A, e, s_col[w], lane, 32);
+    const Phys<double> P(A, prob_of(A, e));
+    const double g = A.lc[A.lev[e]][0], mg = P.mu * g;
+    const int b = lane >> 2, k = lane & 3;
+    double M[JacAcc<MODE>::n];
+#pragma unroll
+    for (int t = 0; t < JacAcc<MODE>::n; ++t) M[t] = 0.0;
+    __syncwarp();
+    const int64_t q1 = pq[i + 1];
+    for (int64_t base = pq[i]; base < q1; base += 32) {
+        const int cnt = (int)min((int64_t)32, q1 - base);
+        if (lane < cnt) {
+            const int64_t q = base + lane;
+            const double *x = xr + 3 * q, *nn = nr + 3 * q, *gq = point_g(A, q);
+            double un = 0.0;
+            for (int j = 0; j < 3; ++j) {
+                const double* a = s_col[w] + 8 * j;
+                const double b0 = fma(x[0], a[1], a[0]), b1 = fma(x[0], a[3], a[2]), b2 = fma(x[0], a[5], a[4]), b3 = fma(x[0], a[7], a[6]);
+                const double u = 0.125 * fma(x[2], fma(x[1], b3, b2), fma(x[1], b1, b0));
+                un = fma(u, nn[j], un);
+                s_pt[w][j][lane] = u - gq[j];
+            }
+            s_pt[w][3][lane] = un < 0.0 ? P.rho * un : 0.0;
+            s_pt[w][4][lane] = wr[q] * 0.015625;   // 8-fold seed and test functions
+            s_pt[w][5][lane] = A.Cb * P.mu * taub[q];
+        }
+        __syncwarp();
+        for (int j = 0; j < cnt; ++j) {
+            const int64_t q = base + j;
+            const double x = xr[3 * q], y = xr[3 * q + 1], z = xr[3 * q + 2];
+            const double nn[3] = {nr[3 * q], nr[3 * q + 1], nr[3 * q + 2]};
+            double phi, d[3], m[3];
+            jac_seed64(b, x, y, z, phi, d, m);
+            const double wq = s_pt[w][4][j];
+            const bool isp = k == 3;
+            const double nk = k == 0 ? nn[0] : k == 1 ? nn[1] : k == 2 ? nn[2] : 0.0;
+            const double ph = isp ? 0.0 : phi;
+            const double dn = fma(d[2], nn[2], fma(d[1], nn[1], d[0] * nn[0]));
+            const double run = s_pt[w][3][j];                                     // rho u.n where u.n < 0
+            const double rin = run < 0.0 ? P.rho : 0.0;
+            const double diag = fma(s_pt[w][5][j] - run, ph, isp ? 0.0 : -mg * dn);   // coefficient on i = k
+            double F[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                // -tr_i + tau_B d_i - [u.n < 0] rho ((u.n)' (u - g)_i + u.n d_i)
+                double f = isp ? phi * nn[r] : -mg * (d[r] * nk);
+                f = fma(-(rin * nk) * ph, s_pt[w][r][j], f);
+                F[r] = wq * (r == k ? f + diag : f);
+            }
+            const double wmg = -(wq * mg) * ph, wn = -wq * (nk * ph);
+            if (MODE == DIAG) {
+                for (int r = 0; r < 3; ++r) {
+                    double f = phi * F[r];
+                    // S_rj = -mu (n_j d_r + n_r d_j) in reference gradients
+                    f = fma(wmg, (r == k ? dn : 0.0) + nn[r] * (k == 0 ? d[0] : k == 1 ? d[1] : d[2]), f);
+                    M[r] += f;
+                }
+                M[3] = fma(phi, wn, M[3]);
+            } else {
+                const double xy = x * y;
+                const double m8[8] = {1.0, x, y, xy, z, x * z, y * z, xy * z};
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    double S[3];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) S[c] = wmg * ((r == k ? nn[c] : 0.0) + (c == k ? nn[r] : 0.0));
+                    jac_moments64(m8, r, F[r], S[0], S[1], S[2], M);
+                }
+                jac_moments64(m8, 3, wn, 0.0, 0.0, 0.0, M);
+            }
+        }
+        __syncwarp();
+    }
+    if constexpr (MODE == DIAG) {
+        if (!A.theta1 && k < 3)
+            for (int t = 0; t < 4; ++t) M[t] *= A.theta;
+    } else {
+        jac_rows64(A, k, M);
+    }
+    jac_store64<MODE>(A, e, sl, M, lane, K, D, true);
+}
+
+// every float64 kernel; FULL: elems (n of them) the requested elements and slot their positions
+template <int MODE>
+void launch_jac64(const Mesh& m, Args A, const int32_t* elems, int64_t n, const int32_t* slot, double* K, double* D, cudaStream_t s) {
+    const int64_t next = m.n_nodes() + m.n_hang();
+    double* ndv = node_workspace<double>(m, nullptr);
+    A.ndv = ndv;
+    A.ndt = ndv + 8 * next;
+    A.ndf = A.F ? ndv + 16 * next : nullptr;
+    if (next > 0) launch_node_prep<double, false>(A, ndv, ndv + 8 * next, (double*)A.ndf, s);
+    const int64_t no = MODE == FULL ? n : (int64_t)m.out_list.size(), nc = (int64_t)m.cut_list.size(), np = (int64_t)m.pen_elem.size();
+    const size_t smem = jac64_smem();
+    // (set on every call: the attribute belongs to the current device)
+    cudaFuncSetAttribute(jac_out64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(jac_cut64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (no > 0)
+        jac_out64<MODE><<<(unsigned)((no + 4 * J64W - 1) / (4 * J64W)), 32 * J64W, smem, s>>>(A, MODE == FULL ? elems : m.d.out_list, no,
+                                                                                          m.d.marker, slot, K, D);
+    if (nc > 0)
+        jac_cut64<MODE><<<(unsigned)nc, 32 * J64W, smem, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, m.d.cut_order, slot, K, D);
+    if (np > 0)
+        jac_surf64<MODE><<<(unsigned)((np + 3) / 4), 128, 0, s>>>(A, m.d.pen_elem, m.d.pen_q, m.d.sq_x, m.d.sq_n, m.d.sq_w, m.d.sq_taub,
+                                                                 np, slot, K, D);
+}
+
 // rows of prescribed components become identity rows
 __global__ void jac_strong_rows(int64_t nn, const uint8_t* __restrict__ flag, const uint8_t* __restrict__ umask,
                                 double* __restrict__ D) {
@@ -484,7 +953,7 @@ int bsr_assemble(const Mesh& m, const double* u, const double* up, const double*
     A.bptr = bptr;
     A.bidx = bidx;
     cudaMemsetAsync(val, 0, (size_t)nb * 16 * sizeof(double), s);
-    if (precision == 0) launch_bsr_assembly<double>(m, A, val, Ks, s);
+    if (precision == 0) launch_jac64<BSR>(m, A, nullptr, 0, nullptr, val, nullptr, s);
     else launch_bsr_assembly<float>(m, A, val, Ks, s);
     if (nn > 0)
         bsr_strong_rows<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(nn, bptr, bidx, m.d.bcflag,
@@ -501,7 +970,7 @@ int element_jacobians(const Mesh& m, const double* u, const double* up, const do
     cudaMemsetAsync(slot, 0xff, (size_t)m.n_elem() * sizeof(int32_t), s);
     fill_slots<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, elems, slot);
     cudaMemsetAsync(K, 0, (size_t)n * 1024 * sizeof(double), s);
-    if (precision == 0) launch_jac<double, FULL>(m, A, slot, K, nullptr, s);
+    if (precision == 0) launch_jac64<FULL>(m, A, elems, n, slot, K, nullptr, s);
     else launch_jac<float, FULL>(m, A, slot, K, nullptr, s);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
@@ -512,7 +981,7 @@ int block_jacobi_setup(const Mesh& m, const double* u, const double* up, const d
     const int64_t nn = m.n_nodes();
     Args A = make_args(m, u, up, up2, f, ph, nullptr, nullptr);
     cudaMemsetAsync(D, 0, (size_t)nn * 16 * sizeof(double), s);
-    if (precision == 0) launch_jac<double, DIAG>(m, A, nullptr, nullptr, D, s);
+    if (precision == 0) launch_jac64<DIAG>(m, A, nullptr, 0, nullptr, nullptr, D, s);
     else launch_jac<float, DIAG>(m, A, nullptr, nullptr, D, s);
     if (nn > 0) {
         jac_strong_rows<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(nn, m.d.bcflag, m.user_bc ? m.d.bcmask_user : nullptr, D);

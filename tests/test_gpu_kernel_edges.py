@@ -113,14 +113,14 @@ def test_mlp_gradient_rows(dev, rows, batch, nin, nout):
 
 
 # ---- float64 Intercepted elements: a block's four parts of 32 points at a time, from elements with a
-# few points (less than one part) to 8^4 of them, slots and atomics, all fields in use ----
+# few points (less than one part) to several rounds, slots and atomics, all fields in use ----
 @pytest.mark.parametrize("lmax", [0, 1, 3])
 @pytest.mark.parametrize("scheme", [I.SCHEME_BE, I.SCHEME_CN, I.SCHEME_BDF2])
 def test_float64_cut_elements(dev, lmax, scheme):
     g, o = pair(I.icosphere(2, 0.2, C, 1e-3, 5), 4, lmax=lmax)
     off, _ = g.cut_points()
     per = np.diff(off)[np.diff(off) > 0]
-    assert {0: per.max() <= 8, 1: per.min() < 32 < per.max(), 3: per.max() > 1000}[lmax]
+    assert {0: per.max() <= 8, 1: per.min() < 32 < per.max(), 3: per.max() > 256}[lmax]
     ph = I.Physics(mu=0.01, dt=0.02, scheme=scheme, g=(0.1, 0.0, -0.2))
     u, up, v = I.state(g.n_nodes, 3)
     up2, f = up + 0.01 * v, 0.3 * v[:, [1, 2, 3, 0]]
@@ -131,3 +131,39 @@ def test_float64_cut_elements(dev, lmax, scheme):
         R = g.residual(ph, a[0], a[1], a[3], f=a[4]).cpu().numpy()
         J = g.jvp(ph, a[0], a[1], a[2], a[3], f=a[4]).cpu().numpy()
         assert rel(R, Ro) <= TOL64 and rel(J, Jo) <= TOL64
+
+
+# ---- float64 element Jacobians (a warp per element part, lane = column) ----
+@pytest.mark.parametrize("scheme", [I.SCHEME_BE, I.SCHEME_CN, I.SCHEME_BDF2])
+@pytest.mark.parametrize("lmax", [0, 2])
+def test_float64_element_jacobians(dev, scheme, lmax):
+    g, o = pair(I.icosphere(2, 0.2, C, 1e-3, 6), 4, lmax=lmax)
+    ph = I.Physics(mu=0.02, dt=0.05, scheme=scheme, g=(0.2, -0.1, 0.0), drop_visc=int(lmax == 0))
+    u, up, v = I.state(g.n_nodes, 4)
+    u[:, 0] -= 1.5 * (np.arange(g.n_nodes) % 2)          # inflow and outflow at the surface
+    up2, f = up + 0.01 * v, 0.2 * v[:, [2, 0, 1, 3]]
+    a = [T(x, dev) for x in (u, up, up2, f)]
+    mk, _ = g.markers()
+    pick = np.concatenate([np.flatnonzero(mk == 0)[::37], np.flatnonzero(mk == 2)[::9], np.flatnonzero(mk == 1)[:2]])
+    pick = np.random.RandomState(0).permutation(pick).astype(np.int32)[: 2 * (pick.size // 2) - 1]   # any order, odd count
+    K = g.element_jacobians(ph, a[0], a[1], T(pick, dev), a[2], f=a[3]).cpu().numpy()
+    for i, e in enumerate(pick):
+        want = o.element_matrix(ph, u, up, int(e), up2, f)[0]
+        # float64 throughout; the fine scale's direction u' / |u'| loses what it cancels
+        assert np.linalg.norm(K[i] - want) <= 1e-11 * max(np.linalg.norm(want), 1e-300), (int(e), mk[e])
+    # the assembled matrix (same columns through M_e) is the operator of J v
+    Jv = g.jvp(ph, a[0], a[1], T(v, dev), a[2], f=a[3])
+    Av = g.bsr_spmv(g.bsr_assemble(ph, a[0], a[1], a[2], f=a[3]), T(v, dev))
+    assert float((Av - Jv).norm() / Jv.norm()) <= TOL64
+
+
+def test_float64_block_jacobi_matches_mixed(dev):
+    w = I.small_sphere(3)
+    g = api.Mesh.from_workload(w)
+    u, up, _ = I.state(g.n_nodes, 2)
+    its = []
+    for prec in (api.PRECISION_FP64, api.PRECISION_MIXED):
+        st = g.newton_step(w.physics, T(u, dev), T(up, dev), precision=prec, precond=1, max_newton=2, raise_on_failure=False)
+        its.append(st["krylov_per_newton"])
+    # the same blocks to float32 rounding: the same iterations, give or take one
+    assert np.abs(np.array(its[0]) - np.array(its[1])).max() <= 1
