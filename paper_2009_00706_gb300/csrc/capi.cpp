@@ -365,7 +365,7 @@ static imga_status apply(imga_mesh h, const double* u, const double* up, const d
     if (precision != 0 && precision != 1) return fail(IMGA_ERR_INVALID_ARG, "precision must be 0 (FP64) or 1 (mixed)");
     for (const void* p : {(const void*)u, (const void*)up, (const void*)up2, (const void*)f, (const void*)v, (const void*)out})
         if (p && ((uintptr_t)p & 15)) return fail(IMGA_ERR_INVALID_ARG, "node vectors must be 16-byte aligned");
-    if (imga::vms_apply(h->m, u, up, up2, f, *ph, precision, v, out, stream)) return cuda_status("residual/jvp launch");
+    if (imga::vms_apply(h->m, u, up, up2, f, *ph, precision, v, out, stream, false)) return cuda_status("residual/jvp launch");
     return IMGA_OK;
 }
 

@@ -263,10 +263,12 @@ void device_free(Mesh& m);
 // residual / Jv (vms.cu)
 int conversion_selftest(int64_t n, uint64_t seed, int64_t* mismatches, std::string& err);
 int vms_apply_skip(const Mesh& m, const double* u, const double* up, const double* up2, const double* f,
-                   const imga_physics& ph, int precision, const double* v, double* out, void* stream, const int* skip);
+                   const imga_physics& ph, int precision, const double* v, double* out, void* stream, const int* skip,
+                   bool generic);
 void vms_prepare();
+// generic: float64 elements by the generic kernels (the float64 evaluations of a mixed-precision solve)
 int vms_apply(const Mesh& m, const double* u, const double* up, const double* up2, const double* f,
-              const imga_physics& ph, int precision, const double* v, double* out, void* stream);
+              const imga_physics& ph, int precision, const double* v, double* out, void* stream, bool generic);
 
 constexpr size_t kNoAllocScratchBytes = (size_t)32 << 20;   // fixed scratch of imga_jvp_noalloc
 constexpr int kMaxDevices = 64;

@@ -332,7 +332,7 @@ int partition_apply(Partition* P, const double* u, const double* up, const doubl
     // 3. every part's element kernels
     for (Part& q : P->parts) {
         if (vms_apply(*q.mesh, q.d_vec[0], q.d_vec[1], up2 ? q.d_vec[2] : nullptr, f ? q.d_vec[3] : nullptr, ph, precision,
-                      v ? q.d_vec[4] : nullptr, q.d_vec[5], s))
+                      v ? q.d_vec[4] : nullptr, q.d_vec[5], s, false))
             return 1;
     }
     // 4. halo reduce-add: ghosts' partial rows back to their owners, added in part order

@@ -567,17 +567,20 @@ public:
         scale_copy_kernel<<<(unsigned)std::min<int64_t>(4 * M.n_sm, (n + 255) / 256), 256, 0, st>>>(n, a, x, y);
     }
 
+    // float64 evaluations of a mixed-precision solve: the generic element code (kGeneric64 in vms.cu)
+    bool generic64() const { return O.precision != 0; }
+
     int residual(const double* u, double* R) {
-        return vms_apply(M, u, Up, Up2, F, P, 0, nullptr, R, st);
+        return vms_apply(M, u, Up, Up2, F, P, 0, nullptr, R, st, generic64());
     }
     int jv(const double* u, const double* v, double* out) {
-        return vms_apply(M, u, Up, Up2, F, P, O.precision, v, out, st);
+        return vms_apply(M, u, Up, Up2, F, P, O.precision, v, out, st, false);
     }
     // the true linear residual of a restart in float64: with float32 element arithmetic J v is linear
     // only to rounding (~1e-7 relative), so the restarts form b - J x with the float64 J v and every
     // cycle refines the float64 solution (iterative refinement); the Arnoldi steps keep O.precision
     int jv_true(const double* u, const double* v, double* out) {
-        return vms_apply(M, u, Up, Up2, F, P, 0, v, out, st);
+        return vms_apply(M, u, Up, Up2, F, P, 0, v, out, st, generic64());
     }
     int pmode = 0;   // preconditioner in use for the current linear solve (block-Jacobi fallback)
     static bool learned_mode(int p) { return p == 2 || p == 3; }
@@ -701,7 +704,7 @@ public:
         const int grid2 = (int)std::min<int64_t>(4 * M.n_sm, (n + 255) / 256);
         dg_copy_basis<<<grid2, 256, 0, st>>>(G, n, W.V, vk);
         precond(vk, z);
-        if (vms_apply_skip(M, u, Up, Up2, F, P, O.precision, z, w, st, &G->stop)) return 1;
+        if (vms_apply_skip(M, u, Up, Up2, F, P, O.precision, z, w, st, &G->stop, false)) return 1;
         for (int pass = 0; pass < 2; ++pass) {
             double* c = dev_field(pass ? offsetof(GState, h2) : offsetof(GState, h));
             dg_mdot<<<dim3(grid, (kMaxM + 1 + kDotGroup - 1) / kDotGroup), 256, 0, st>>>(G, n, W.V, w, W.partial);
@@ -996,7 +999,7 @@ public:
                 dg_combine<<<grid2, 256, 0, st>>>(G, n, W.V, w);
                 precond(w, z);
                 axpby(1.0, z, 1.0, du);
-                ok = ok && vms_apply_skip(M, u, Up, Up2, F, P, 0, du, w, st, nullptr) == 0;   // float64: jv_true
+                ok = ok && vms_apply_skip(M, u, Up, Up2, F, P, 0, du, w, st, nullptr, generic64()) == 0;   // float64: jv_true
                 cudaMemcpyAsync(r, b, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
                 axpby(-1.0, w, 1.0, r);
                 norm_dev(r, nfield(offsetof(NState, beta)));
@@ -1013,7 +1016,7 @@ public:
                 st = c[1];
                 ng_trial<<<(unsigned)std::min<int64_t>(4 * M.n_sm, (n + 255) / 256), 256, 0, st>>>(
                     n, u, du, nfield(offsetof(NState, lam)), ut);
-                ok = vms_apply_skip(M, ut, Up, Up2, F, P, 0, nullptr, Rt, st, nullptr) == 0;
+                ok = vms_apply_skip(M, ut, Up, Up2, F, P, 0, nullptr, Rt, st, nullptr, generic64()) == 0;
                 norm_dev(Rt, nfield(offsetof(NState, rt)));
                 ng_ls_decide<<<1, 1, 0, st>>>(N, hL);
                 end(c[1], &bL);

@@ -56,6 +56,13 @@ template <class T> struct IntShape {
     static constexpr size_t smem = (size_t)(2 * EPB * ESTR + EPB * 8 * MSTR) * sizeof(T);
 };
 
+// kGeneric64: the residual and J v of a mixed-precision solve run their float64 evaluations on the generic
+// element code, with the roundings it has always had.  Such a solve turns the last bit of a residual into
+// float32 steps of its preconditioner and matvecs, and those into differences as large as its tolerance
+// (1e-9 to 1e-7 of u at 1e-8), so other roundings there would make other solutions, no nearer and no
+// further from the root.  It costs a solve of the 7.3 k element sphere 4 of 40 ms.  Everything else,
+// float64 solves included, takes the kernels below.
+//
 // One Out element in float64 on 8 lanes of a warp (c = lane & 7); nd its 8 corner rows, sw the warp's
 // 4 x 272 doubles.  FP64 instructions are the cost (see Const64), so the work goes to lanes by what
 // shares most of them:
@@ -235,12 +242,7 @@ __device__ __forceinline__ void interior_element64(const Args& A, const double* 
 template <class T, bool JV, bool IL = (JV && sizeof(T) == 4)>
 __device__ __forceinline__ void interior_element(const Args& A, T* nd, T* s_mw, const T m[8], int lane, int64_t idx,
                                                  bool valid, int lv, int prob, int32_t id) {
-    if constexpr (sizeof(T) == 8) {
-        interior_element64<JV>(A, nd, s_mw, lane, idx, valid, lv, prob, id);
-        return;
-    } else {
-    typedef Dual<T, 1> DT;
-    typedef typename std::conditional<JV, DT, T>::type S;
+    typedef typename std::conditional<JV, Dual<T, sizeof(T) == 4>, T>::type S;
     constexpr int MSTR = IntShape<T>::MSTR;
     const int c = lane & 7;
     T* mrow = s_mw + lane * MSTR;
@@ -278,11 +280,11 @@ __device__ __forceinline__ void interior_element(const Args& A, T* nd, T* s_mw, 
     }
     for (int k = 0; k < 4; ++k) r[k] = hadamard_bwd<1>(r[k], c);
     if (A.sv) {
-        // deterministic scatter: node c's 4 rows into the element's slot (one 16-byte store)
+        // deterministic scatter: node c's 4 rows into the element's slot (one 16- or 32-byte store)
         if (valid) st4s<T>((T*)A.sv + 32 * idx + 4 * c, r[0], r[1], r[2], r[3]);
-    } else {
+    } else if constexpr (sizeof(T) == 4) {
         // corners of this warp's 4 elements that are the same node add their rows in shared memory
-        // first; one lane per node scatters (fewer float64 atomics)
+        // first; one lane per node scatters (fewer float64 atomics; float64: the plain scatter is faster)
         const unsigned grp = __match_any_sync(0xffffffffu, valid ? id : -1 - lane);
         __syncwarp();   // every lane has read its moment columns
         st4s<T>(mrow, r[0], r[1], r[2], r[3]);
@@ -296,9 +298,10 @@ __device__ __forceinline__ void interior_element(const Args& A, T* nd, T* s_mw, 
             }
             scatter_t(A, id, t);
         }
+    } else {
+        if (valid) scatter_t(A, id, r);
     }
     __syncwarp();   // the rows and the moments are rewritten by later elements
-    }
 }
 
 // Gauss point c of the 2x2x2 rule (xi_k = +-1/sqrt(3) by bit k of c) in monomial form
@@ -316,7 +319,8 @@ __device__ __forceinline__ void gauss_monomials(int c, T m[8]) {
 // group's 16 elements (interior_element).
 // MINB: resident blocks per SM the register allocation is made for (4: up to 128 registers per thread;
 // 5: up to 102, a few spills, one more block of warps to hide latency with)
-template <class T, bool JV, int MINB = (sizeof(T) == 4 ? 4 : 2)>
+// GEN: float64 elements by the code of the float32 ones (see kGeneric64)
+template <class T, bool JV, int MINB = (sizeof(T) == 4 ? 4 : 2), bool GEN = false>
 __global__ void __launch_bounds__(IntShape<T>::THREADS, MINB) vms_interior(Args A, const int32_t* __restrict__ oconn,
                                                     const uint8_t* __restrict__ olev,
                                                     const uint16_t* __restrict__ oprob, int64_t n) {
@@ -358,8 +362,11 @@ __global__ void __launch_bounds__(IntShape<T>::THREADS, MINB) vms_interior(Args 
         const int lp_next = gnext < ngroups ? level_prob(gnext) : 0;
         cp_wait<1>();
         const int64_t idx = gi * EPB + le;
-        interior_element<T, JV>(A, s_nd + (buf * EPB + le) * ESTR, s_mw, m, lane, idx, idx < n, lp_cur & 255,
-                                lp_cur >> 8, id_cur);
+        if constexpr (sizeof(T) == 8 && !GEN)
+            interior_element64<JV>(A, s_nd + (buf * EPB + le) * ESTR, s_mw, lane, idx, idx < n, lp_cur & 255, lp_cur >> 8, id_cur);
+        else
+            interior_element<T, JV>(A, s_nd + (buf * EPB + le) * ESTR, s_mw, m, lane, idx, idx < n, lp_cur & 255,
+                                    lp_cur >> 8, id_cur);
         id_cur = id_next;
         id_next = id_after;
         lp_cur = lp_next;
@@ -609,7 +616,7 @@ __device__ __forceinline__ void cut_element64(const Args& A, const int32_t* __re
 
 // W warps per block (a tile shape the autotuner picks); `order` (or null) permutes the list
 template <class T, bool JV, int W>
-__global__ void __launch_bounds__(32 * W, 16 / W) vms_cut(Args A, const int32_t* __restrict__ list,
+__global__ void __launch_bounds__(32 * W, (sizeof(T) == 4 ? 16 : 8) / W) vms_cut(Args A, const int32_t* __restrict__ list,
                                                     const int64_t* __restrict__ off, const void* __restrict__ pts,
                                                     const int32_t* __restrict__ order, int64_t n) {
     constexpr int PAD = 16 / (int)sizeof(T), MSTR = 32 + PAD;
@@ -891,8 +898,12 @@ __global__ void __launch_bounds__(32 * kFusedWarps, sizeof(T) == 4 ? 4 : 2) vms_
                     const int lp_next = nxt >= 0 ? level_prob(nxt) : 0;
                     cp_wait<1>();
                     const int64_t idx = 4 * cur + le;
-                    interior_element<T, JV>(A, base + (buf * 4 + le) * ESTR, s_mw, m, lane, idx, idx < Q.n_out,
-                                            lp_cur & 255, lp_cur >> 8, id_cur);
+                    if constexpr (sizeof(T) == 8)
+                        interior_element64<JV>(A, base + (buf * 4 + le) * ESTR, s_mw, lane, idx, idx < Q.n_out, lp_cur & 255,
+                                               lp_cur >> 8, id_cur);
+                    else
+                        interior_element<T, JV>(A, base + (buf * 4 + le) * ESTR, s_mw, m, lane, idx, idx < Q.n_out,
+                                                lp_cur & 255, lp_cur >> 8, id_cur);
                     cur = nxt;
                     nxt = aft;
                     id_cur = id_next;
@@ -1212,11 +1223,12 @@ struct Timed {
 };
 
 template <class T, bool JV>
-void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt) {
+void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt, bool generic = false) {
     const int64_t nc = (int64_t)m.cut_list.size();
     const int32_t* order = lpt ? m.d.cut_order : nullptr;
     if constexpr (sizeof(T) == 8) {
-        if (wpb == 2) vms_cut64<JV, 2><<<(unsigned)nc, 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
+        if (generic) vms_cut<T, JV, 4><<<(unsigned)((nc + 3) / 4), 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order, nc);
+        else if (wpb == 2) vms_cut64<JV, 2><<<(unsigned)nc, 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
         else vms_cut64<JV, 4><<<(unsigned)nc, 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
     } else {
         const void* pts = m.d.cut_pts_f;
@@ -1228,10 +1240,10 @@ void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt) 
     }
 }
 
-template <class T, bool JV, int MINB = (sizeof(T) == 4 ? 4 : 2)>
+template <class T, bool JV, int MINB = (sizeof(T) == 4 ? 4 : 2), bool GEN = false>
 int interior_blocks_per_sm();
 template <class T, bool JV>
-void launch_interior(const Mesh& m, const Args& A, cudaStream_t s, int bps);
+void launch_interior(const Mesh& m, const Args& A, cudaStream_t s, int bps, bool generic = false);
 
 // Autotuner of the Intercepted-element bucket: with the node data of this call prepared, time every
 // (warps per block, element order) candidate on the call's own inputs (3 launches each after one
@@ -1293,14 +1305,14 @@ int autotune_cut(Mesh& m, Args A, cudaStream_t s) {
 }
 
 // Resident CTAs of the persistent interior kernel per SM (queried once; also sets its dynamic smem opt-in).
-template <class T, bool JV, int MINB>
+template <class T, bool JV, int MINB, bool GEN>
 int interior_blocks_per_sm() {
     static int bps = 0;
     if (bps == 0) {
         const size_t smem = IntShape<T>::smem;
         int b = 0;
-        cudaFuncSetAttribute(vms_interior<T, JV, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, vms_interior<T, JV, MINB>, 8 * Epb<T>::value, smem);
+        cudaFuncSetAttribute(vms_interior<T, JV, MINB, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, vms_interior<T, JV, MINB, GEN>, 8 * Epb<T>::value, smem);
         bps = b < 1 ? 1 : b;
     }
     return bps;
@@ -1309,13 +1321,19 @@ int interior_blocks_per_sm() {
 // The persistent interior kernel at bps resident blocks per SM: the 5-block register allocation for
 // bps = 5 (float only), else the default one.
 template <class T, bool JV>
-void launch_interior(const Mesh& m, const Args& A, cudaStream_t s, int bps) {
+void launch_interior(const Mesh& m, const Args& A, cudaStream_t s, int bps, bool generic) {
     const int64_t no = (int64_t)m.out_list.size();
     constexpr int EPB = Epb<T>::value;
     const int64_t grid = std::min<int64_t>((no + EPB - 1) / EPB, (int64_t)bps * m.n_sm);
     if constexpr (sizeof(T) == 4) {
         if (bps >= 5) {
             vms_interior<T, JV, 5><<<(unsigned)grid, 8 * EPB, IntShape<T>::smem, s>>>(A, m.d.out_conn, m.d.out_lev, m.d.out_prob, no);
+            return;
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (generic) {
+            vms_interior<T, JV, 2, true><<<(unsigned)grid, 8 * EPB, IntShape<T>::smem, s>>>(A, m.d.out_conn, m.d.out_lev, m.d.out_prob, no);
             return;
         }
     }
@@ -1405,7 +1423,7 @@ void launch_fused(const Mesh& m, const Args& A, cudaStream_t s, cudaStream_t ss,
 
 template <class T, bool JV>
 void launch_all(const Mesh& m, Args A, cudaStream_t s, void* ws = nullptr, cudaStream_t s_cut = nullptr,
-                cudaStream_t s_sur = nullptr, cudaEvent_t* ev = nullptr) {
+                cudaStream_t s_sur = nullptr, cudaEvent_t* ev = nullptr, bool generic = false) {
     const int64_t next = m.n_nodes() + m.n_hang();
     T* ndv = node_workspace<T>(m, ws);
     T* ndt = ndv + 8 * next;
@@ -1417,7 +1435,7 @@ void launch_all(const Mesh& m, Args A, cudaStream_t s, void* ws = nullptr, cudaS
         Timed t(m, 4, s, (A.n_nodes > 0) + (A.n_hang > 0), !ws);
         launch_node_prep<T, JV>(A, ndv, ndt, ndf, s);
     }
-    if (m.fused && m.d.fq_cnt) {
+    if (m.fused && m.d.fq_cnt && !generic) {
         launch_fused<T, JV>(m, A, s, s_sur, ev, !ws);
         return;
     }
@@ -1433,12 +1451,12 @@ void launch_all(const Mesh& m, Args A, cudaStream_t s, void* ws = nullptr, cudaS
     if (no > 0) {
         Timed t(m, 0, s, 1, !ws);
         const int tuned = m.out_bps[sizeof(T) == 4][JV];
-        launch_interior<T, JV>(m, A, s, tuned > 0 ? tuned : interior_blocks_per_sm<T, JV>());
+        launch_interior<T, JV>(m, A, s, tuned > 0 ? tuned : interior_blocks_per_sm<T, JV>(), generic);
     }
     if (nc > 0) {
         Timed t(m, 1, sc, 1, !ws);
         const Mesh::CutTune& ct = m.cut_tune[sizeof(T) == 4][JV];
-        launch_cut<T, JV>(m, A, sc, ct.wpb, ct.lpt);
+        launch_cut<T, JV>(m, A, sc, ct.wpb, ct.lpt, generic);
     }
     launch_surface<T, JV>(m, A, ss, !ws);
     if (ev) {   // join
@@ -1522,10 +1540,15 @@ static int side_streams(Mesh& mm) {
 }
 
 static int vms_apply_ws(const Mesh& m, const double* u, const double* up, const double* up2, const double* f,
-                        const imga_physics& ph, int precision, const double* v, double* out, void* stream, void* ws) {
+                        const imga_physics& ph, int precision, const double* v, double* out, void* stream, void* ws,
+                        bool generic) {
     cudaStream_t s = (cudaStream_t)stream;
     Args A = make_args(m, u, up, up2, f, ph, v, out);
     const bool jv = v != nullptr;
+    if (generic) {   // (launch attributes, once)
+        interior_blocks_per_sm<double, true, 2, true>();
+        interior_blocks_per_sm<double, false, 2, true>();
+    }
     if (m.tune_pending[precision != 0][jv] && !ws) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         cudaStreamIsCapturing(s, &cs);
@@ -1545,7 +1568,7 @@ static int vms_apply_ws(const Mesh& m, const double* u, const double* up, const 
         GraphKey key;
         std::memset(&key, 0, sizeof(key));
         key.u = u; key.up = up; key.up2 = up2; key.f = f; key.v = v; key.out = out;
-        key.precision = precision;
+        key.precision = precision | (generic ? 2 : 0);
         key.ph = ph;
         key.user_bc = m.user_bc;
         if (side_streams(mm)) return 1;
@@ -1562,7 +1585,7 @@ static int vms_apply_ws(const Mesh& m, const double* u, const double* up, const 
             cudaStream_t b1 = m.concurrent ? s1 : cs, b2 = m.concurrent ? s2 : cs;
             cudaEvent_t* bev = m.concurrent ? ev : nullptr;
             if (precision == 0) {
-                if (jv) launch_all<double, true>(m, A, cs, nullptr, b1, b2, bev); else launch_all<double, false>(m, A, cs, nullptr, b1, b2, bev);
+                if (jv) launch_all<double, true>(m, A, cs, nullptr, b1, b2, bev, generic); else launch_all<double, false>(m, A, cs, nullptr, b1, b2, bev, generic);
             } else {
                 if (jv) launch_all<float, true>(m, A, cs, nullptr, b1, b2, bev); else launch_all<float, false>(m, A, cs, nullptr, b1, b2, bev);
             }
@@ -1596,7 +1619,7 @@ static int vms_apply_ws(const Mesh& m, const double* u, const double* up, const 
         ev = (cudaEvent_t*)mm.fork_ev;
     }
     if (precision == 0) {
-        if (jv) launch_all<double, true>(m, A, s, ws, s1, s2, ev); else launch_all<double, false>(m, A, s, ws, s1, s2, ev);
+        if (jv) launch_all<double, true>(m, A, s, ws, s1, s2, ev, generic); else launch_all<double, false>(m, A, s, ws, s1, s2, ev, generic);
     } else {
         if (jv) launch_all<float, true>(m, A, s, ws, s1, s2, ev); else launch_all<float, false>(m, A, s, ws, s1, s2, ev);
     }
@@ -1709,14 +1732,14 @@ int conversion_selftest(int64_t n, uint64_t seed, int64_t* mismatches, std::stri
 // nonzero (steps of a solver loop that is itself captured in a graph).
 int vms_apply_skip(const Mesh& m, const double* u, const double* up, const double* up2, const double* f,
                    const imga_physics& ph, int precision, const double* v, double* out, void* stream,
-                   const int* skip) {
+                   const int* skip, bool generic) {
     cudaStream_t s = (cudaStream_t)stream;
     Args A = make_args(m, u, up, up2, f, ph, v, out);
     A.skip = skip;
     const bool jv = v != nullptr;
     if (!A.sv && cudaMemsetAsync(out, 0, (size_t)m.n_nodes() * 4 * sizeof(double), s) != cudaSuccess) return 1;
     if (precision == 0) {
-        if (jv) launch_all<double, true>(m, A, s); else launch_all<double, false>(m, A, s);
+        if (jv) launch_all<double, true>(m, A, s, nullptr, nullptr, nullptr, nullptr, generic); else launch_all<double, false>(m, A, s, nullptr, nullptr, nullptr, nullptr, generic);
     } else {
         if (jv) launch_all<float, true>(m, A, s); else launch_all<float, false>(m, A, s);
     }
@@ -1728,6 +1751,8 @@ int vms_apply_skip(const Mesh& m, const double* u, const double* up, const doubl
 void vms_prepare() {
     interior_blocks_per_sm<double, true>();
     interior_blocks_per_sm<double, false>();
+    interior_blocks_per_sm<double, true, 2, true>();
+    interior_blocks_per_sm<double, false, 2, true>();
     interior_blocks_per_sm<float, true>();
     interior_blocks_per_sm<float, false>();
     interior_blocks_per_sm<float, true, 5>();
@@ -1735,8 +1760,8 @@ void vms_prepare() {
 }
 
 int vms_apply(const Mesh& m, const double* u, const double* up, const double* up2, const double* f,
-              const imga_physics& ph, int precision, const double* v, double* out, void* stream) {
-    return vms_apply_ws(m, u, up, up2, f, ph, precision, v, out, stream, nullptr);
+              const imga_physics& ph, int precision, const double* v, double* out, void* stream, bool generic) {
+    return vms_apply_ws(m, u, up, up2, f, ph, precision, v, out, stream, nullptr, generic);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1774,7 +1799,7 @@ int vms_jvp_noalloc(const Mesh& m, const double* u, const double* up, const doub
         }
         ws = g_noalloc_addr[dev];
     }
-    if (vms_apply_ws(m, u, up, up2, f, ph, precision, v, out, stream, ws)) { err = "launch failed"; return 1; }
+    if (vms_apply_ws(m, u, up, up2, f, ph, precision, v, out, stream, ws, false)) { err = "launch failed"; return 1; }
     return 0;
 }
 

@@ -289,6 +289,7 @@ template <> __device__ __forceinline__ double to_t<double>(double x) { return x;
 
 // scatter one node's 4 values in the element precision: widened to float64 on the float64 unit,
 // which the element kernels leave idle while their integer pipe is busy
+__device__ __forceinline__ void scatter_t(const Args& A, int32_t id, const double r[4]) { scatter(A, id, r); }
 __device__ __forceinline__ void scatter_t(const Args& A, int32_t id, const float r[4]) {
     const double rd[4] = {(double)r[0], (double)r[1], (double)r[2], (double)r[3]};
     scatter(A, id, rd);
