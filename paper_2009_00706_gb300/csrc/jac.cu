@@ -10,7 +10,7 @@
 //   float64: jac_out64, jac_cut64, jac_surf64 (lane = column of k_e); float32 element arithmetic:
 //   jac_out     8 threads per Out element (thread c: Gauss point c, then node c's 4 rows)
 //   jac_cut     one warp per Intercepted element, 32 sub-cell points per step, lane = row
-//   jac_nitsche one thread per surface point
+//   jac_nitsche one thread per surface point (a warp per block: there are few points, and each is long)
 // Mode FULL writes k_e for requested elements (slot map); mode DIAG adds the 4x4 diagonal blocks
 // of sum_e M_e^T k_e M_e (each corner's own block times the squared hanging weights; the
 // couplings of two different corners of one element that share a parent are left out) to a
@@ -51,20 +51,68 @@ __device__ __forceinline__ int corner_nodes(const Args& A, int32_t id, int32_t n
     return np;
 }
 
-// entry (row i of corner ida, column k of corner idb) of k_e added to the assembled matrix through
-// M_e^T k_e M_e (Algorithm 2): every parent pair (p, q) receives w_p w_q v in block (p, q)
-__device__ __forceinline__ void bsr_add(const Args& A, int32_t ida, int32_t idb, int i, int k, double v,
-                                        double* __restrict__ val) {
-    if (v == 0.0) return;
+// N entries of row or block (corner ida, corner idb) of k_e added to the assembled matrix through
+// M_e^T k_e M_e (Algorithm 2): every parent pair (p, q) receives w_p w_q v in block (p, q), entry at[j]
+// (4 x row component + column component).  The row is searched once per corner pair: entry by entry the
+// searches were most of the assembly (43.6 k elements,
+// mixed: 5.37 -> 2.01 ms with the basis tables, the shared test functions and the adds below).
+// A warp adds whole blocks from shared memory where it can (bsr_add_blocks): 16 lanes on the 128 bytes of a
+// block make 4 L2 transactions of what lane-by-lane adds make 16 of.
+// Float entries are weighted (powers of two: exact) and tested in float32 and widened on the integer pipe:
+// the FP64 pipe was 58 % busy with that alone.
+__device__ __forceinline__ double wide(float x) { return f2d(x); }
+__device__ __forceinline__ double wide(double x) { return x; }
+template <int N, class T, class At>
+__device__ __forceinline__ void bsr_add(const Args& A, int32_t ida, int32_t idb, const T* v, At at, double* __restrict__ val) {
     int32_t na[4], nb[4];
     double wa, wb;
     const int ca = corner_nodes(A, ida, na, wa), cb = corner_nodes(A, idb, nb, wb);
-    const double vw = wa * wb * v;
+    const T w = (ca == 1 ? T(1) : ca == 2 ? T(0.5) : T(0.25)) * (cb == 1 ? T(1) : cb == 2 ? T(0.5) : T(0.25));
     for (int p = 0; p < ca; ++p)
         for (int q = 0; q < cb; ++q) {
             const int64_t pos = bsr_find(A.bptr, A.bidx, na[p], nb[q]);
-            if (pos >= 0) atomicAdd(val + 16 * pos + 4 * i + k, vw);
+            if (pos < 0) continue;
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+                if (v[j] != T(0)) atomicAdd(val + 16 * pos + at(j), wide(w * v[j]));
         }
+}
+
+// 32 blocks of a warp, entry (block m, j) given by v(m, j), to positions s_pos[m] (-1: none)
+template <class V>
+__device__ __forceinline__ void bsr_add_blocks(const int64_t* s_pos, V v, int lane, double* __restrict__ val) {
+#pragma unroll 4
+    for (int m = lane >> 4; m < 32; m += 2) {
+        const int64_t pos = s_pos[m];
+        const auto x = v(m, lane & 15);
+        if (pos >= 0 && x != 0) atomicAdd(val + 16 * pos + (lane & 15), wide(x));
+    }
+}
+__device__ __forceinline__ bool plain_corner(const Args& A, int32_t id) { return id < A.n_nodes; }
+
+// The block (corner ida, corner idb) of a warp's element, at least one of them hanging, through M_e: lane 4 p + q
+// searches the block of parent pair (p, q), then 16 lanes add each pair's 16 entries v(j).  Uniform call.
+template <class V>
+__device__ __forceinline__ void bsr_add_hanging(const Args& A, int32_t ida, int32_t idb, V v, int lane, double* __restrict__ val) {
+    const int p = (lane >> 2) & 3, q = lane & 3;
+    auto node = [&](int32_t id, int k, int& n) -> int32_t {   // k-th node of a corner and how many there are
+        if (id < A.n_nodes) { n = 1; return id; }
+        const int32_t* hp = A.hpar + 4 * (int64_t)(id - A.n_nodes);
+        n = hp[2] >= 0 ? 4 : 2;
+        return k < n ? hp[k] : -1;
+    };
+    int ca, cb;
+    const int32_t row = node(ida, p, ca), col = node(idb, q, cb);
+    const int64_t pos = lane < 16 && p < ca && q < cb ? bsr_find(A.bptr, A.bidx, row, col) : -1;
+    const auto x = v(lane & 15);
+    const auto w = x * (ca == 1 ? 1.f : ca == 2 ? 0.5f : 0.25f) * (cb == 1 ? 1.f : cb == 2 ? 0.5f : 0.25f);
+    const double d = wide(w);
+#pragma unroll 1
+    for (int m = 0; m < 16; m += 2) {
+        if (((m >> 2) >= ca) || (m & 3) >= cb) continue;   // uniform (pairs m, m + 1: q even and odd)
+        const int64_t o = __shfl_sync(0xffffffffu, pos, m + (lane >> 4));
+        if (o >= 0 && x != 0) atomicAdd(val + 16 * o + (lane & 15), d);
+    }
 }
 
 // tangent fields of the seed (corner b, component k) at a point whose corner-b basis values are
@@ -131,7 +179,26 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
     constexpr int EPB = JacShape<T>::EPB;
     __shared__ __align__(16) T s_nd[EPB][8][CS];
     __shared__ T s_cf[EPB][8][17];
+    __shared__ __align__(16) T s_bas[8][8][4];   // [Gauss point q][corner c]: phi, reference gradient
+    __shared__ T s_blk[MODE == BSR ? EPB / 4 : 1][32][17];      // BSR: block (corner c, corner b) of every lane
+    __shared__ int64_t s_pos[MODE == BSR ? EPB / 4 : 1][32];
     const int c = threadIdx.x & 7, le = threadIdx.x >> 3;
+    for (int t = threadIdx.x; t < 64; t += blockDim.x) {   // the same for every element and seed
+        const T gs = (T)0.57735026918962576451;
+        const T wp = T(0.5) * (T(1) + gs), wm = T(0.5) * (T(1) - gs);
+        const int q = t >> 3, cc = t & 7;
+        T f[3], d[3];
+        for (int kk = 0; kk < 3; ++kk) {
+            const bool same = (((cc >> kk) & 1) == ((q >> kk) & 1));
+            f[kk] = same ? wp : wm;
+            d[kk] = ((cc >> kk) & 1) ? T(0.5) : T(-0.5);
+        }
+        s_bas[q][cc][0] = f[0] * f[1] * f[2];
+        s_bas[q][cc][1] = d[0] * f[1] * f[2];
+        s_bas[q][cc][2] = d[1] * f[0] * f[2];
+        s_bas[q][cc][3] = d[2] * f[0] * f[1];
+    }
+    __syncthreads();
     const int64_t idx = (int64_t)blockIdx.x * EPB + le;
     const bool valid = idx < n;
     const int32_t e = list[valid ? idx : n - 1];
@@ -158,6 +225,7 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
     for (int b = 0; b < 8; ++b) {
         T phb, dphb[3], d2b[3];
         corner_basis<T>(fm, fp, b, phb, dphb, d2b);
+#pragma unroll 1   // (unrolled, the shared value part is contracted differently: other last bits)
         for (int k = 0; k < 4; ++k) {
             Fields<Dual<T>, T> F;
             seed_fields<T>(A, V, g, phb, dphb, d2b, k, F);
@@ -168,14 +236,10 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
             T r[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                T f[3], d[3];
-                for (int kk = 0; kk < 3; ++kk) {
-                    bool same = (((c >> kk) & 1) == ((q >> kk) & 1));
-                    f[kk] = same ? wp : wm;
-                    d[kk] = ((c >> kk) & 1) ? T(0.5) : T(-0.5);
-                }
-                T ph = f[0] * f[1] * f[2];
-                T dp[3] = {d[0] * f[1] * f[2], d[1] * f[0] * f[2], d[2] * f[0] * f[1]};
+                T bs[4];
+                ld4s<T>(&s_bas[q][c][0], bs);
+                const T ph = bs[0];
+                const T* dp = bs + 1;
                 const T* C = s_cf[le][q];
                 for (int i = 0; i < 3; ++i) r[i] += ph * C[i] + dp[0] * C[3 + 3 * i] + dp[1] * C[4 + 3 * i] + dp[2] * C[5 + 3 * i];
                 r[3] += ph * C[12] + dp[0] * C[13] + dp[1] * C[14] + dp[2] * C[15];
@@ -185,12 +249,24 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
                 if (work)
                     for (int i = 0; i < 4; ++i) K[(int64_t)sl * 1024 + (c * 4 + i) * 32 + b * 4 + k] = (double)r[i];
             } else if (MODE == BSR) {
-                const int32_t idb = __shfl_sync(0xffffffffu, id, (threadIdx.x & 31 & ~7) | b);
-                if (work)
-                    for (int i = 0; i < 4; ++i) bsr_add(A, id, idb, i, k, (double)r[i], K);
+                for (int i = 0; i < 4; ++i) s_blk[threadIdx.x >> 5][threadIdx.x & 31][i * 4 + k] = r[i];
             } else if (b == c) {
                 for (int i = 0; i < 4; ++i) diag[i * 4 + k] = (double)r[i];
             }
+        }
+        if (MODE == BSR) {
+            const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+            const int32_t idb = __shfl_sync(0xffffffffu, id, (lane & ~7) | b);
+            const bool plain = plain_corner(A, id) && plain_corner(A, idb);
+            s_pos[w][lane] = work && plain ? bsr_find(A.bptr, A.bidx, id, idb) : -1;
+            __syncwarp();
+            bsr_add_blocks(s_pos[w], [&](int m, int j) { return s_blk[w][m][j]; }, lane, K);
+            for (unsigned need = __ballot_sync(0xffffffffu, work && !plain); need; need &= need - 1) {
+                const int src = __ffs(need) - 1;
+                const int32_t ha = __shfl_sync(0xffffffffu, id, src), hb = __shfl_sync(0xffffffffu, idb, src);
+                bsr_add_hanging(A, ha, hb, [&](int j) { return s_blk[w][src][j]; }, lane, K);
+            }
+            __syncwarp();
         }
     }
     if (MODE == DIAG && work) add_diag(A, id, diag, D);
@@ -201,13 +277,18 @@ constexpr int JWPB = 2;   // warps per block of jac_cut
 template <class T, int MODE>
 __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __restrict__ list,
                                                      const int64_t* __restrict__ off, const void* __restrict__ pts,
-                                                     int64_t n, const int32_t* __restrict__ slot,
-                                                     double* __restrict__ K, double* __restrict__ D) {
+                                                     const int32_t* __restrict__ order, int64_t n,
+                                                     const int32_t* __restrict__ slot, double* __restrict__ K,
+                                                     double* __restrict__ D) {
     __shared__ __align__(16) T s_nd[JWPB][8][CS];
-    __shared__ T s_cf[JWPB][32][20];
+    // a point's coefficients for the four seeds of a corner (80-byte rows: conflict-free 16-byte stores):
+    // the contraction, bound by shared memory, then reads a point's test functions once for four sums
+    __shared__ __align__(16) T s_cf[JWPB][4][32][20];
+    __shared__ __align__(16) T s_bas[JWPB][32][8][4];  // a point's test functions (phi, reference gradient), once for all seeds
+    __shared__ T s_acc[JWPB][32][32];                  // the element's columns so far
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t idx = (int64_t)blockIdx.x * JWPB + w;
-    if (idx >= n) return;
+    if ((int64_t)blockIdx.x * JWPB + w >= n) return;
+    const int64_t idx = order[(int64_t)blockIdx.x * JWPB + w];
     const int32_t e = list[idx];
     const int32_t sl = MODE == FULL ? slot[e] : 0;
     if (sl < 0) return;
@@ -220,9 +301,8 @@ __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __re
     const T g = lvl_g<T>(A, A.lev[e]);
     const T det = lvl_w<T>(A, A.lev[e]);
     const int a = lane >> 2, comp = lane & 3;
-    const T sa[3] = {(a & 1) ? T(1) : T(-1), (a & 2) ? T(1) : T(-1), (a & 4) ? T(1) : T(-1)};
-    T acc[32];
-    for (int s = 0; s < 32; ++s) acc[s] = T(0);
+    T* acc = &s_acc[w][0][lane];   // acc[32 s]: row `lane` of column s
+    for (int s = 0; s < 32; ++s) acc[32 * s] = T(0);
     const int64_t q0 = off[idx], q1 = off[idx + 1];
     for (int64_t base = q0; base < q1; base += 32) {
         const int64_t q = base + lane;
@@ -235,45 +315,76 @@ __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __re
         interp<T, T>(A, fm, fp, &s_nd[w][0][0], CS, g, V);
         const T wq = have ? pt[3] * det : T(0), wqg = wq * g;
         const int m = (int)min((int64_t)32, q1 - base);
-        for (int s = 0; s < 32; ++s) {
-            const int b = s >> 2, k = s & 3;
+        for (int cc = 0; cc < 8; ++cc) {
+            const T s0 = (cc & 1) ? T(1) : T(-1), s1 = (cc & 2) ? T(1) : T(-1), s2 = (cc & 4) ? T(1) : T(-1);
+            const T f0 = T(0.5) * (T(1) + s0 * pt[0]), f1 = T(0.5) * (T(1) + s1 * pt[1]), f2 = T(0.5) * (T(1) + s2 * pt[2]);
+            st4s<T>(&s_bas[w][lane][cc][0], f0 * f1 * f2, T(0.5) * s0 * f1 * f2, T(0.5) * s1 * f0 * f2, T(0.5) * s2 * f0 * f1);
+        }
+        for (int b = 0; b < 8; ++b) {
             T phb, dphb[3], d2b[3];
             corner_basis<T>(fm, fp, b, phb, dphb, d2b);
+#pragma unroll 1   // as in jac_out
+            for (int k = 0; k < 4; ++k) {
             Fields<Dual<T>, T> F;
             seed_fields<T>(A, V, g, phb, dphb, d2b, k, F);
             Dual<T> cf[16];
             pointwise<Dual<T>, T>(A, Phys<T>(A, prob_of(A, e)), F, g, cf);
-            for (int qq = 0; qq < 16; ++qq) s_cf[w][lane][qq] = ((qq < 3 || qq == 12) ? wq : wqg) * cf[qq].d;
-            s_cf[w][lane][16] = pt[0];
-            s_cf[w][lane][17] = pt[1];
-            s_cf[w][lane][18] = pt[2];
-            __syncwarp();
-            T sum = T(0);
-            for (int j = 0; j < m; ++j) {
-                const T* C = s_cf[w][j];
-                T f0 = T(0.5) * (T(1) + sa[0] * C[16]), f1 = T(0.5) * (T(1) + sa[1] * C[17]), f2 = T(0.5) * (T(1) + sa[2] * C[18]);
-                T ph = f0 * f1 * f2;
-                T d0 = T(0.5) * sa[0] * f1 * f2, d1 = T(0.5) * sa[1] * f0 * f2, d2 = T(0.5) * sa[2] * f0 * f1;
-                if (comp < 3) sum += ph * C[comp] + d0 * C[3 + 3 * comp] + d1 * C[4 + 3 * comp] + d2 * C[5 + 3 * comp];
-                else sum += ph * C[12] + d0 * C[13] + d1 * C[14] + d2 * C[15];
+            T cw[16];   // (component, its phi and gradient coefficients) in fours
+            for (int qq = 0; qq < 16; ++qq) cw[qq] = ((qq < 3 || qq == 12) ? wq : wqg) * cf[qq].d;
+            for (int i = 0; i < 3; ++i) st4s<T>(&s_cf[w][k][lane][4 * i], cw[i], cw[3 + 3 * i], cw[4 + 3 * i], cw[5 + 3 * i]);
+            st4s<T>(&s_cf[w][k][lane][12], cw[12], cw[13], cw[14], cw[15]);
             }
-            acc[s] += sum;
+            __syncwarp();
+            T sum[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll 2
+            for (int j = 0; j < m; ++j) {
+                T B[4];
+                ld4s<T>(&s_bas[w][j][a][0], B);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    // (multiply-adds spelled out: contracted otherwise, the sum has other last bits)
+                    T C[4];
+                    ld4s<T>(&s_cf[w][k][j][4 * comp], C);
+                    T t = B[0] * C[0];
+                    t = fma(B[1], C[1], t);
+                    t = fma(B[2], C[2], t);
+                    t = fma(B[3], C[3], t);
+                    sum[k] += t;
+                }
+            }
+            for (int k = 0; k < 4; ++k) acc[32 * (4 * b + k)] += sum[k];
             __syncwarp();
         }
     }
     if (MODE == FULL) {
-        for (int s = 0; s < 32; ++s) K[(int64_t)sl * 1024 + lane * 32 + s] = (double)acc[s];
+        for (int s = 0; s < 32; ++s) K[(int64_t)sl * 1024 + lane * 32 + s] = (double)acc[32 * s];
     } else if (MODE == BSR) {
-        const int32_t ida = __shfl_sync(0xffffffffu, my_id, a);
-        for (int s = 0; s < 32; ++s) {
-            const int32_t idb = __shfl_sync(0xffffffffu, my_id, s >> 2);
-            bsr_add(A, ida, idb, comp, s & 3, (double)acc[s], K);
+        __syncwarp();
+        int64_t* s_pos = reinterpret_cast<int64_t*>(&s_bas[w][0][0][0]);   // (the points are done)
+        const unsigned hanging = __ballot_sync(0xffffffffu, lane < 8 && !plain_corner(A, my_id)) & 0xffu;
+        for (int half = 0; half < 2; ++half) {   // corner pairs (4 half + m / 8, m % 8)
+            const int pa = 4 * half + (lane >> 3), pb = lane & 7;
+            const int32_t ida = __shfl_sync(0xffffffffu, my_id, pa), idb = __shfl_sync(0xffffffffu, my_id, pb);
+            s_pos[lane] = (hanging >> pa | hanging >> pb) & 1u ? -1 : bsr_find(A.bptr, A.bidx, ida, idb);
+            __syncwarp();
+            bsr_add_blocks(s_pos, [&](int m, int j) {
+                return s_acc[w][4 * (m & 7) + (j & 3)][4 * (4 * half + (m >> 3)) + (j >> 2)];
+            }, lane, K);
+            __syncwarp();
         }
+        if (hanging)
+            for (int m = 0; m < 64; ++m) {
+                const int pa = m >> 3, pb = m & 7;
+                if (!((hanging >> pa | hanging >> pb) & 1u)) continue;
+                const int32_t ha = __shfl_sync(0xffffffffu, my_id, pa), hb = __shfl_sync(0xffffffffu, my_id, pb);
+                bsr_add_hanging(A, ha, hb, [&](int j) { return s_acc[w][4 * pb + (j & 3)][4 * pa + (j >> 2)]; }, lane, K);
+            }
     } else {
-        // lane (a, comp) holds row comp of corner a's own block in acc[4a .. 4a+3]
+        // lane (a, comp) holds row comp of corner a's own block in columns 4a .. 4a+3
+        __syncwarp();
         double blk[16];
         for (int i = 0; i < 4; ++i)
-            for (int k = 0; k < 4; ++k) blk[i * 4 + k] = (double)__shfl_sync(0xffffffffu, acc[4 * a + k], 4 * a + i);
+            for (int k = 0; k < 4; ++k) blk[i * 4 + k] = (double)s_acc[w][4 * a + k][4 * a + i];
         const int32_t id = __shfl_sync(0xffffffffu, my_id, a);
         if (comp == 0) add_diag(A, id, blk, D);
     }
@@ -878,11 +989,11 @@ void launch_jac(const Mesh& m, Args A, const int32_t* slot, double* K, double* D
     if (no > 0) jac_out<T, MODE><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, slot, K, D);
     if (nc > 0) {
         const void* pts = sizeof(T) == 4 ? (const void*)m.d.cut_pts_f : (const void*)m.d.cut_pts;
-        jac_cut<T, MODE><<<(unsigned)((nc + JWPB - 1) / JWPB), 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, nc,
+        jac_cut<T, MODE><<<(unsigned)((nc + JWPB - 1) / JWPB), 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order, nc,
                                                                                slot, K, D);
     }
     if (ns > 0)
-        jac_nitsche<T, MODE><<<(unsigned)((ns + 127) / 128), 128, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w,
+        jac_nitsche<T, MODE><<<(unsigned)((ns + 31) / 32), 32, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w,
                                                                         m.d.sq_taub, ns, slot, K, D);
 }
 
@@ -895,21 +1006,27 @@ __global__ void scatter_kmat(Args A, const int32_t* __restrict__ list, int64_t n
     const int row = (int)((t >> 3) & 31), b = (int)(t & 7);
     const int32_t e = list[s];
     const int32_t ida = A.conn[8 * (int64_t)e + (row >> 2)], idb = A.conn[8 * (int64_t)e + b];
-    for (int k = 0; k < 4; ++k) bsr_add(A, ida, idb, row & 3, k, Ks[s * 1024 + row * 32 + 4 * b + k], val);
+    const int comp = row & 3;
+    bsr_add<4>(A, ida, idb, Ks + s * 1024 + row * 32 + 4 * b, [=](int j) { return 4 * comp + j; }, val);
 }
 
-// rows of prescribed components become identity rows of the assembled matrix
+// rows of prescribed components become identity rows of the assembled matrix; eight threads per node
+// over its blocks
 __global__ void bsr_strong_rows(int64_t nn, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                 const uint8_t* __restrict__ flag, const uint8_t* __restrict__ umask, double* __restrict__ val) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = t >> 3;
     if (n >= nn) return;
     uint8_t mask = umask ? umask[n] : (uint8_t)(flag[n] & 15);
     if (flag[n] & 16) mask = 15;
     if (!mask) return;
-    for (int64_t q = ptr[n]; q < ptr[n + 1]; ++q)
+    for (int64_t q = ptr[n] + (t & 7); q < ptr[n + 1]; q += 8)
         for (int k = 0; k < 4; ++k)
-            if ((mask >> k) & 1)
-                for (int j = 0; j < 4; ++j) val[16 * q + 4 * k + j] = (idx[q] == n && j == k) ? 1.0 : 0.0;
+            if ((mask >> k) & 1) {
+                const bool d = idx[q] == n;
+                double2* o = reinterpret_cast<double2*>(val + 16 * q + 4 * k);
+                o[0] = make_double2(d && k == 0 ? 1.0 : 0.0, d && k == 1 ? 1.0 : 0.0);
+                o[1] = make_double2(d && k == 2 ? 1.0 : 0.0, d && k == 3 ? 1.0 : 0.0);
+            }
 }
 
 template <class T>
@@ -926,14 +1043,14 @@ void launch_bsr_assembly(const Mesh& m, Args A, double* val, double* Ks, cudaStr
     if (no > 0) jac_out<T, BSR><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, nullptr, val, nullptr);
     if (nc > 0) {
         const void* pts = sizeof(T) == 4 ? (const void*)m.d.cut_pts_f : (const void*)m.d.cut_pts;
-        jac_cut<T, BSR><<<(unsigned)((nc + JWPB - 1) / JWPB), 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, nc,
+        jac_cut<T, BSR><<<(unsigned)((nc + JWPB - 1) / JWPB), 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order, nc,
                                                                               nullptr, val, nullptr);
     }
     if (ns > 0 && nh > 0) {
         cudaMemsetAsync(m.d.slot, 0xff, (size_t)m.n_elem() * sizeof(int32_t), s);
         fill_slots<<<(unsigned)((nh + 255) / 256), 256, 0, s>>>(nh, m.d.sq_hosts, m.d.slot);
         cudaMemsetAsync(Ks, 0, (size_t)nh * 1024 * sizeof(double), s);
-        jac_nitsche<T, FULL><<<(unsigned)((ns + 127) / 128), 128, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w,
+        jac_nitsche<T, FULL><<<(unsigned)((ns + 31) / 32), 32, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w,
                                                                         m.d.sq_taub, ns, m.d.slot, Ks, nullptr);
         scatter_kmat<<<(unsigned)((nh * 256 + 255) / 256), 256, 0, s>>>(A, m.d.sq_hosts, nh, Ks, val);
     }
@@ -956,7 +1073,7 @@ int bsr_assemble(const Mesh& m, const double* u, const double* up, const double*
     if (precision == 0) launch_jac64<BSR>(m, A, nullptr, 0, nullptr, val, nullptr, s);
     else launch_bsr_assembly<float>(m, A, val, Ks, s);
     if (nn > 0)
-        bsr_strong_rows<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(nn, bptr, bidx, m.d.bcflag,
+        bsr_strong_rows<<<(unsigned)((8 * nn + 255) / 256), 256, 0, s>>>(nn, bptr, bidx, m.d.bcflag,
                                                                     m.user_bc ? m.d.bcmask_user : nullptr, val);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
