@@ -38,23 +38,188 @@ constexpr int kMaxLevels = 24;
 // ------------------------------------------------------------------------------------------
 // kernels
 // ------------------------------------------------------------------------------------------
-// y = b - A x (b null: y = A x); four threads per block row, thread i forms component i
-template <class T>
-__global__ void __launch_bounds__(256) bsr_resid(int64_t n, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
-                                                 const T* __restrict__ val, const T* __restrict__ x,
-                                                 const T* __restrict__ b, T* __restrict__ y) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = t >> 2;
-    const int i = (int)(t & 3);
-    if (row >= n) return;
-    T acc = T(0);
-    for (int64_t q = ptr[row], q1 = ptr[row + 1]; q < q1; ++q) {
-        const int64_t c = idx[q];
-        const T* v = val + 16 * q + 4 * i;
-        const T* xc = x + 4 * c;
-        acc += v[0] * xc[0] + v[1] * xc[1] + v[2] * xc[2] + v[3] * xc[3];
+// Row products of a block matrix, Q quads of lanes per block row.  The blocks come from HBM or L2 (64 or
+// 128 bytes each for 32 flops), so what counts is bytes in flight: lane 4 j + i of a row's lanes loads row i
+// of block q + j whole (16-byte loads) with the column's vector entry, and kRowAhead steps of Q blocks are
+// loaded before the first sum.  Every block's four products are summed by its lane and the blocks' sums
+// added in column order by every lane: the order, and the bits, of a thread that walks the row.  Q = 8 (a
+// warp per row) shortens the chain where the rows of a level leave the chip idle; from kManyRows on Q = 2,
+// which needs a third of the instructions per block.  V-cycle on 74 k nodes, mixed: 349 -> 181 us (186 with
+// Q = 1 there, 200 with Q = 4).
+constexpr int kRowAhead = 4;
+constexpr int64_t kManyRows = 32768;
+
+template <class T> struct Row4 { T v[4]; };
+template <class T> __device__ __forceinline__ Row4<T> load_row(const T* p) {
+    Row4<T> r;
+    if constexpr (sizeof(T) == 4) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+        r.v[0] = a.x; r.v[1] = a.y; r.v[2] = a.z; r.v[3] = a.w;
+    } else {
+        const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+        r.v[0] = a.x; r.v[1] = a.y; r.v[2] = b.x; r.v[3] = b.y;
     }
-    y[4 * row + i] = b ? b[4 * row + i] - acc : acc;
+    return r;
+}
+// (multiply-adds spelled out in one order: the compiler's own choice would depend on the kernel)
+template <class T> __device__ __forceinline__ T dot4(const T* a, const T* b) {
+    return fma(a[3], b[3], fma(a[2], b[2], fma(a[0], b[0], a[1] * b[1])));
+}
+
+// a vector entry of the cycle: x, or x plus the coarse correction of its aggregate on free unknowns
+template <class T> struct Plain {
+    const T* x;
+    __device__ Row4<T> operator()(int64_t c) const {   // (x is rewritten between launches: no read-only loads)
+        Row4<T> r;
+        if constexpr (sizeof(T) == 4) {
+            const float4 a = reinterpret_cast<const float4*>(x)[c];
+            r.v[0] = a.x; r.v[1] = a.y; r.v[2] = a.z; r.v[3] = a.w;
+        } else {
+            const double2 a = reinterpret_cast<const double2*>(x)[2 * c], b = reinterpret_cast<const double2*>(x)[2 * c + 1];
+            r.v[0] = a.x; r.v[1] = a.y; r.v[2] = b.x; r.v[3] = b.y;
+        }
+        return r;
+    }
+};
+template <class T> struct Corrected {
+    Plain<T> x, xc;
+    const uint8_t* fr;
+    uint32_t agg;
+    __device__ Row4<T> operator()(int64_t c) const {
+        Row4<T> r = x(c);
+        const Row4<T> d = xc((uint32_t)c / agg);
+        const unsigned f = fr[c];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((f >> k) & 1u) r.v[k] += d.v[k];
+        return r;
+    }
+};
+
+// component (lane & 3) of row `row` of A x, on the row's 4 Q lanes (live: this row exists; every lane of the
+// warp calls)
+template <int Q, class T, class X>
+__device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
+                                         const T* __restrict__ val, const X& x) {
+    constexpr int D = kRowAhead * (Q == 8 ? 1 : 2);   // steps in flight
+    const int lane = threadIdx.x & 31, j = (lane >> 2) & (Q - 1), i = lane & 3, first = lane & ~(4 * Q - 1);
+    const int64_t q0 = live ? ptr[row] : 0, q1 = live ? ptr[row + 1] : 0;
+    T acc = T(0);
+    for (int64_t base = q0; __any_sync(0xffffffffu, base < q1); base += Q * D) {
+        T t[D];
+        int32_t c[D];
+#pragma unroll
+        for (int g = 0; g < D; ++g) {
+            const int64_t q = base + Q * g + j;
+            c[g] = q < q1 ? __ldg(idx + q) : -1;
+        }
+#pragma unroll
+        for (int g = 0; g < D; ++g) {
+            t[g] = T(0);
+            if (c[g] >= 0) {
+                const Row4<T> a = load_row(val + 16 * (base + Q * g + j) + 4 * i), b = x(c[g]);
+                t[g] = dot4(a.v, b.v);
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < D; ++g)
+#pragma unroll
+            for (int b = 0; b < Q; ++b) {
+                const T s = Q == 1 ? t[g] : __shfl_sync(0xffffffffu, t[g], first + 4 * b + i);
+                if (base + Q * g + b < q1) acc += s;
+            }
+    }
+    return acc;
+}
+
+// y = A x
+template <class T, int Q>
+__global__ void __launch_bounds__(256) bsr_mul(int64_t n, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
+                                               const T* __restrict__ val, const T* __restrict__ x, T* __restrict__ y) {
+    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (4 * Q);
+    const int l = threadIdx.x & (4 * Q - 1);
+    const T acc = row_product<Q, T>(row < n, row, ptr, idx, val, Plain<T>{x});
+    if (row < n && l < 4) y[4 * row + l] = acc;
+}
+
+// One damped block-Jacobi sweep, out of place: y = x + omega Dinv (b - A x), x with the coarse correction
+// where X is Corrected; z (or null): y once more, in float64.
+template <class T, class X, int Q>
+__global__ void __launch_bounds__(256) ml_sweep(int64_t n, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
+                                                const T* __restrict__ val, X x, const T* __restrict__ b,
+                                                const T* __restrict__ Dinv, T omega, T* __restrict__ y, double* __restrict__ z) {
+    const int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (4 * Q);
+    const bool live = r0 < n;
+    const int64_t row = live ? r0 : n - 1;
+    const int l = threadIdx.x & (4 * Q - 1), i = l & 3;
+    const Row4<T> D = load_row(Dinv + 16 * row + 4 * i), xr = x(row);
+    const T bi = b[4 * row + i];
+    const T res = bi - row_product<Q, T>(live, row, ptr, idx, val, x);
+    T v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xffffffffu, res, (threadIdx.x & 28) | k);
+    const T own = i == 0 ? xr.v[0] : i == 1 ? xr.v[1] : i == 2 ? xr.v[2] : xr.v[3];
+    const T out = fma(omega, dot4(D.v, v), own);
+    if (live && l < 4) {
+        y[4 * row + l] = out;
+        if (z) z[4 * row + l] = (double)out;
+    }
+}
+
+// Residual, its restriction and the first sweep of the next level, a block of 256 threads for `per` whole
+// aggregates (or one, in turns of 64 / Q rows, if it has more rows): rc[I] = sum of F_i (b - A x)_i over
+// the aggregate in row order; xc[I] = omega Dinv_c rc[I] (Dinv_c null: the next level is the dense one,
+// which starts from rc alone).  The residual itself is never stored.
+template <class T, int Q>
+__global__ void __launch_bounds__(256) ml_restrict(int64_t nc, int64_t nf, int agg, int per, const int64_t* __restrict__ ptr,
+                                                   const int32_t* __restrict__ idx, const T* __restrict__ val,
+                                                   const T* __restrict__ x, const T* __restrict__ b,
+                                                   const uint8_t* __restrict__ fr, const T* __restrict__ Dinv_c, T omega,
+                                                   T* __restrict__ rc, T* __restrict__ xc) {
+    constexpr int R = 64 / Q;   // rows at a time
+    __shared__ T s_res[R][4];
+    const int r = threadIdx.x / (4 * Q), i = threadIdx.x & 3;
+    const int64_t I0 = (int64_t)blockIdx.x * per, I1 = I0 + per < nc ? I0 + per : nc;
+    const int64_t i0 = I0 * agg, i1 = I1 * agg < nf ? I1 * agg : nf;
+    const int64_t I = I0 + (threadIdx.x >> 2);   // threads 4 a .. 4 a + 3 sum aggregate I0 + a
+    T s = T(0);
+    for (int64_t a0 = i0; a0 < i1; a0 += R) {
+        const int64_t row = a0 + r;
+        const bool live = row < i1;
+        const T bi = live ? b[4 * row + i] : T(0);
+        const T res = bi - row_product<Q, T>(live, row, ptr, idx, val, Plain<T>{x});
+        if (live && (threadIdx.x & (4 * Q - 1)) < 4) s_res[r][i] = res;
+        __syncthreads();
+        if (I < I1)
+            for (int64_t q = I * agg > a0 ? I * agg : a0; q < (I + 1) * agg && q < a0 + R && q < i1; ++q)
+                if ((fr[q] >> i) & 1) s += s_res[q - a0][i];
+        __syncthreads();
+    }
+    if (I >= I1) return;
+    rc[4 * I + i] = s;
+    if (!Dinv_c) return;
+    T v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xfu << (threadIdx.x & 28), s, (threadIdx.x & 28) | k);
+    const Row4<T> D = load_row(Dinv_c + 16 * I + 4 * i);
+    xc[4 * I + i] = omega * dot4(D.v, v);
+}
+
+// x[i][k] += F_i xc[I(i)][k]: on a level of many rows a pass of its own (the corrected entry at every block,
+// with its division by the aggregate size, costs a sweep of 74 k rows 11 us, this pass 3)
+template <class T>
+__global__ void __launch_bounds__(256) ml_prolong(int64_t nf, uint32_t agg, const uint8_t* __restrict__ fr, const T* __restrict__ xc,
+                                                  T* __restrict__ x) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = t >> 2;
+    if (i >= nf) return;
+    if ((fr[i] >> (t & 3)) & 1) x[t] += xc[4 * ((uint32_t)i / agg) + (t & 3)];
+}
+
+// calls f with the quads per row as a constant
+template <class F> void with_quads(int64_t rows, F&& f) {
+    if (rows >= kManyRows) f(std::integral_constant<int, 2>());
+    else f(std::integral_constant<int, 8>());
 }
 
 // free mask of level 0 from the assembled float64 matrix: bit k set unless row (node, k) is an
@@ -248,62 +413,37 @@ __global__ void __launch_bounds__(512) ml_dense_inverse(int N, const double* __r
     }
 }
 
-// x = omega Dinv r   (first sweep from x = 0)
+// r in the cycle's precision and the first sweep from x = 0: x = omega Dinv r
 template <class T>
-__global__ void ml_smooth0(int64_t n, const T* __restrict__ Dinv, T omega, const T* __restrict__ r, T* __restrict__ x) {
+__global__ void ml_start(int64_t n, const T* __restrict__ Dinv, T omega, const double* __restrict__ rd, T* __restrict__ r,
+                         T* __restrict__ x) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t row = t >> 2;
     const int i = (int)(t & 3);
     if (row >= n) return;
-    const T* M = Dinv + 16 * row + 4 * i;
-    const T* v = r + 4 * row;
-    x[4 * row + i] = omega * (M[0] * v[0] + M[1] * v[1] + M[2] * v[2] + M[3] * v[3]);
+    const T own = (T)rd[t];
+    T v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xfu << (threadIdx.x & 28), own, (threadIdx.x & 28) | k);
+    r[t] = own;
+    const Row4<T> D = load_row(Dinv + 16 * row + 4 * i);
+    x[t] = omega * dot4(D.v, v);
 }
 
-// x += omega Dinv res
+// y = Ainv r for the dense last level (N <= 4 * coarse_max <= 96), one block, a thread per row: r from
+// shared memory, 8 entries of the row loaded before they are added (one serial load per entry was its time)
 template <class T>
-__global__ void ml_smooth(int64_t n, const T* __restrict__ Dinv, T omega, const T* __restrict__ res, T* __restrict__ x) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = t >> 2;
-    const int i = (int)(t & 3);
-    if (row >= n) return;
-    const T* M = Dinv + 16 * row + 4 * i;
-    const T* v = res + 4 * row;
-    x[4 * row + i] += omega * (M[0] * v[0] + M[1] * v[1] + M[2] * v[2] + M[3] * v[3]);
-}
-
-// rc[I][k] = sum over the rows i of aggregate I of F_i res[i][k]
-template <class T>
-__global__ void ml_restrict(int64_t nc, int64_t nf, int agg, const uint8_t* __restrict__ fr, const T* __restrict__ res,
-                            T* __restrict__ rc) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t I = t >> 2;
-    const int k = (int)(t & 3);
-    if (I >= nc) return;
+__global__ void __launch_bounds__(96) ml_dense_apply(int N, const T* __restrict__ Ainv, const T* __restrict__ r, T* __restrict__ y) {
+    __shared__ T s_r[96];
+    const int i = threadIdx.x;
+    if (i < N) s_r[i] = r[i];
+    __syncthreads();
+    if (i >= N) return;
     T s = T(0);
-    for (int64_t i = I * agg, iend = (I * agg + agg < nf ? I * agg + agg : nf); i < iend; ++i)
-        if ((fr[i] >> k) & 1) s += res[4 * i + k];
-    rc[4 * I + k] = s;
-}
-
-// x[i][k] += F_i xc[I(i)][k]
-template <class T>
-__global__ void ml_prolong(int64_t nf, int agg, const uint8_t* __restrict__ fr, const T* __restrict__ xc, T* __restrict__ x) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t i = t >> 2;
-    const int k = (int)(t & 3);
-    if (i >= nf) return;
-    if ((fr[i] >> k) & 1) x[4 * i + k] += xc[4 * (i / agg) + k];
-}
-
-// y = Ainv r for the dense last level (N <= 4 * coarse_max); one block
-template <class T>
-__global__ void ml_dense_apply(int N, const T* __restrict__ Ainv, const T* __restrict__ r, T* __restrict__ y) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        T s = T(0);
-        for (int j = 0; j < N; ++j) s += Ainv[(int64_t)i * N + j] * r[j];
-        y[i] = s;
-    }
+    const T* a = Ainv + (int64_t)i * N;
+#pragma unroll 8
+    for (int j = 0; j < N; ++j) s += a[j] * s_r[j];
+    y[i] = s;
 }
 
 inline unsigned blocks(int64_t threads, int per = 256) { return (unsigned)std::max<int64_t>(1, (threads + per - 1) / per); }
@@ -453,30 +593,59 @@ int setup_values(const Mesh& m, Multilevel& L, cudaStream_t s) {
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
+// V-cycle below the first sweep of level l (x[l] = omega Dinv r[l] is there); the result is in *out, one of
+// the level's two iterates.  z (level 0, or null): the last sweep also writes it there in float64.
 template <class T>
-void vcycle(Multilevel& L, size_t l, cudaStream_t s) {
+void vcycle(Multilevel& L, size_t l, cudaStream_t s, T** out, double* z) {
     MLValues<T>& v = values<T>(L);
     const MLPattern& p = L.lev[l];
-    if (l + 1 == L.lev.size()) {
-        ml_dense_apply<T><<<1, 256, 0, s>>>((int)(4 * p.n), v.Cinv, v.r[l], v.x[l]);
+    const T om = (T)L.omega;
+    T *x = v.x[l], *y = v.res[l];
+    auto sweep = [&](auto in, double* zk) {
+        with_quads(p.n, [&](auto q) {
+            constexpr int Q = decltype(q)::value;
+            ml_sweep<T, decltype(in), Q><<<blocks(4 * Q * p.n), 256, 0, s>>>(p.n, p.dptr, p.didx, v.A[l], in, v.r[l], v.Dinv[l], om, y, zk);
+        });
+        std::swap(x, y);
+    };
+    for (int k = 1; k < L.nu; ++k) sweep(Plain<T>{x}, nullptr);
+    const MLPattern& c = L.lev[l + 1];
+    const bool dense = l + 2 == L.lev.size();
+    with_quads(p.n, [&](auto q) {
+        constexpr int Q = decltype(q)::value;
+        const int per = std::max(1, 64 / Q / L.agg);
+        ml_restrict<T, Q><<<(unsigned)((c.n + per - 1) / per), 256, 0, s>>>(c.n, p.n, L.agg, per, p.dptr, p.didx, v.A[l], x, v.r[l], L.fr[l],
+                                                                        dense ? nullptr : v.Dinv[l + 1], om, v.r[l + 1], v.x[l + 1]);
+    });
+    T* xc = v.x[l + 1];
+    if (dense) ml_dense_apply<T><<<1, 96, 0, s>>>((int)(4 * c.n), v.Cinv, v.r[l + 1], xc);
+    else vcycle<T>(L, l + 1, s, &xc, nullptr);
+    for (int k = 0; k < L.nu; ++k) {
+        double* zk = k + 1 == L.nu ? z : nullptr;
+        if (k == 0 && p.n < kManyRows) {
+            sweep(Corrected<T>{{x}, {xc}, L.fr[l], (uint32_t)L.agg}, zk);
+            continue;
+        }
+        if (k == 0) ml_prolong<T><<<blocks(4 * p.n), 256, 0, s>>>(p.n, (uint32_t)L.agg, L.fr[l], xc, x);
+        sweep(Plain<T>{x}, zk);
+    }
+    *out = x;
+}
+
+// z = V-cycle(r): two launches per level (three where it has many rows) and one for the dense one (six before)
+template <class T>
+void apply(Multilevel& L, const double* r, double* z, cudaStream_t s) {
+    MLValues<T>& v = values<T>(L);
+    const int64_t n = L.lev[0].n;
+    if (L.lev.size() == 1) {   // dense only
+        convert_kernel<double, T><<<blocks(4 * n), 256, 0, s>>>(4 * n, r, v.r[0]);
+        ml_dense_apply<T><<<1, 96, 0, s>>>((int)(4 * n), v.Cinv, v.r[0], v.x[0]);
+        convert_kernel<T, double><<<blocks(4 * n), 256, 0, s>>>(4 * n, v.x[0], z);
         return;
     }
-    const T om = (T)L.omega;
-    const int64_t th = 4 * p.n;
-    ml_smooth0<T><<<blocks(th), 256, 0, s>>>(p.n, v.Dinv[l], om, v.r[l], v.x[l]);
-    for (int k = 1; k < L.nu; ++k) {
-        bsr_resid<T><<<blocks(th), 256, 0, s>>>(p.n, p.dptr, p.didx, v.A[l], v.x[l], v.r[l], v.res[l]);
-        ml_smooth<T><<<blocks(th), 256, 0, s>>>(p.n, v.Dinv[l], om, v.res[l], v.x[l]);
-    }
-    bsr_resid<T><<<blocks(th), 256, 0, s>>>(p.n, p.dptr, p.didx, v.A[l], v.x[l], v.r[l], v.res[l]);
-    const MLPattern& c = L.lev[l + 1];
-    ml_restrict<T><<<blocks(4 * c.n), 256, 0, s>>>(c.n, p.n, L.agg, L.fr[l], v.res[l], v.r[l + 1]);
-    vcycle<T>(L, l + 1, s);
-    ml_prolong<T><<<blocks(th), 256, 0, s>>>(p.n, L.agg, L.fr[l], v.x[l + 1], v.x[l]);
-    for (int k = 0; k < L.nu; ++k) {
-        bsr_resid<T><<<blocks(th), 256, 0, s>>>(p.n, p.dptr, p.didx, v.A[l], v.x[l], v.r[l], v.res[l]);
-        ml_smooth<T><<<blocks(th), 256, 0, s>>>(p.n, v.Dinv[l], om, v.res[l], v.x[l]);
-    }
+    ml_start<T><<<blocks(4 * n), 256, 0, s>>>(n, v.Dinv[0], (T)L.omega, r, v.r[0], v.x[0]);
+    T* x;
+    vcycle<T>(L, 0, s, &x, z);
 }
 
 }  // namespace
@@ -558,17 +727,9 @@ int multilevel_apply(Mesh& m, const double* r, double* z, void* stream) {
     Multilevel* L = (Multilevel*)m.mlev;
     if (!L || L->precision < 0) return 1;
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t n4 = 4 * L->lev[0].n;
-    if (n4 == 0) return 0;
-    if (L->precision == 0) {
-        cudaMemcpyAsync(L->vd.r[0], r, n4 * sizeof(double), cudaMemcpyDeviceToDevice, s);
-        vcycle<double>(*L, 0, s);
-        cudaMemcpyAsync(z, L->vd.x[0], n4 * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    } else {
-        convert_kernel<double, float><<<blocks(n4), 256, 0, s>>>(n4, r, L->vf.r[0]);
-        vcycle<float>(*L, 0, s);
-        convert_kernel<float, double><<<blocks(n4), 256, 0, s>>>(n4, L->vf.x[0], z);
-    }
+    if (L->lev[0].n == 0) return 0;
+    if (L->precision == 0) apply<double>(*L, r, z, s);
+    else apply<float>(*L, r, z, s);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
@@ -594,7 +755,10 @@ int bsr_spmv(Mesh& m, const double* val, const double* x, double* y, void* strea
     if (!L) { err = "the block pattern is not on the device (call the assembly first)"; return 1; }
     const MLPattern& p = L->lev[0];
     if (p.n > 0)
-        bsr_resid<double><<<blocks(4 * p.n), 256, 0, (cudaStream_t)stream>>>(p.n, p.dptr, p.didx, val, x, nullptr, y);
+        with_quads(p.n, [&](auto q) {
+            constexpr int Q = decltype(q)::value;
+            bsr_mul<double, Q><<<blocks(4 * Q * p.n), 256, 0, (cudaStream_t)stream>>>(p.n, p.dptr, p.didx, val, x, y);
+        });
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
