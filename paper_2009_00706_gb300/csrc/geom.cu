@@ -512,49 +512,56 @@ static bool upload_cut_order(Mesh& m, std::string& err) {
 // Entry encoding (32 bits): bits 0-2 corner, bits 3-4 weight (0: 1, 1: 1/2, 2: 1/4), bits 5-31
 // global slot (volume slots first; at most 2^27 slots).
 bool build_incidence(Mesh& m, const std::vector<int32_t>& sq_el, const std::vector<int32_t>& dense, std::string& err) {
-    const int64_t nn = m.n_nodes(), nv = (int64_t)(m.out_list.size() + m.cut_list.size());
+    const int64_t nn = m.n_nodes(), no = (int64_t)m.out_list.size(), nv = no + (int64_t)m.cut_list.size();
     const int64_t ns = m.n_sq_elem + m.n_sq_sparse;
     m.n_vslots = nv;
     m.n_sslots = ns;
     if (nv + ns >= ((int64_t)1 << 27)) { err = "too many element slots for the incidence list (2^27)"; return false; }
-    auto elem_of = [&](int64_t s) -> int64_t {
-        if (s < (int64_t)m.out_list.size()) return m.out_list[s];
-        if (s < nv) return m.cut_list[s - (int64_t)m.out_list.size()];
-        if (s < nv + m.n_sq_elem) return dense[s - nv];
-        return sq_el[s - nv - m.n_sq_elem];
-    };
-    std::vector<int64_t> ptr(nn + 1, 0);
     auto visit = [&](auto&& fn) {
-        for (int64_t s = 0; s < nv + ns; ++s) {
-            const int64_t e = elem_of(s);
+        auto element = [&](int64_t s, int64_t e) {
             for (int c = 0; c < 8; ++c) {
                 const int32_t id = m.conn[8 * e + c];
                 if (id < nn) { fn(id, (uint32_t)(s << 5) | (uint32_t)c); continue; }
                 const int64_t h = id - nn;
-                const int np = m.hnp[h];
-                const uint32_t wc = np == 4 ? 2u : 1u;
-                for (int q = 0; q < np; ++q) fn(m.hpar[4 * h + q], (uint32_t)(s << 5) | (wc << 3) | (uint32_t)c);
+                const int q1 = m.hnp[h];
+                const uint32_t wc = q1 == 4 ? 2u : 1u;
+                for (int q = 0; q < q1; ++q) fn(m.hpar[4 * h + q], (uint32_t)(s << 5) | (wc << 3) | (uint32_t)c);
             }
-        }
+        };
+        for (int64_t s = 0; s < nv; ++s) element(s, s < no ? m.out_list[s] : m.cut_list[s - no]);
+        for (int64_t j = 0; j < m.n_sq_elem; ++j) element(nv + j, dense[j]);
+        for (int64_t j = 0; j < m.n_sq_sparse; ++j) element(nv + m.n_sq_elem + j, sq_el[j]);
     };
-    visit([&](int64_t node, uint32_t) { ptr[node + 1] += 1; });
-    for (int64_t i = 0; i < nn; ++i) ptr[i + 1] += ptr[i];
-    std::vector<uint32_t> inc(std::max<int64_t>(1, ptr[nn]));
-    std::vector<int64_t> fill(ptr.begin(), ptr.end() - 1);
-    visit([&](int64_t node, uint32_t code) { inc[fill[node]++] = code; });
-    // stored as a fixed head of kIncHead entries per node (sentinel-padded: one aligned 32-byte load,
-    // no offset to fetch first) and the rest of each list in CSR form; the list order is kept
-    std::vector<uint32_t> head((size_t)std::max<int64_t>(1, nn) * kIncHead, kIncNone);
-    std::vector<int64_t> optr(nn + 1, 0);
-    for (int64_t i = 0; i < nn; ++i) optr[i + 1] = optr[i] + std::max<int64_t>(0, ptr[i + 1] - ptr[i] - kIncHead);
-    std::vector<uint32_t> oinc(std::max<int64_t>(1, optr[nn]));
+    std::vector<int32_t> count(nn, 0);
+    visit([&](int64_t node, uint32_t) { ++count[node]; });
+    // a node's list at a fixed place (one aligned 32-byte load, padded) if it fits, else in CSR form in whole
+    // batches of kIncHead, longest lists first (counting sort: node order within a length)
+    std::vector<int32_t> heavy;
+    std::vector<int64_t> hptr(1, 0), fill(nn), at;
+    auto batches = [&](int64_t i) { return (count[i] + kIncHead - 1) / kIncHead; };
+    int64_t most = 1, nheavy = 0;
+    for (int64_t i = 0; i < nn; ++i) { most = std::max<int64_t>(most, batches(i)); nheavy += count[i] > kIncHead; }
+    at.assign(most + 2, 0);   // at[most - b + 1]: nodes of b batches
     for (int64_t i = 0; i < nn; ++i)
-        for (int64_t q = ptr[i], k = 0; q < ptr[i + 1]; ++q, ++k) {
-            if (k < kIncHead) head[(size_t)i * kIncHead + k] = inc[q];
-            else oinc[optr[i] + k - kIncHead] = inc[q];
-        }
+        if (count[i] > kIncHead) ++at[most - batches(i) + 1];
+    for (int64_t b = 0; b <= most; ++b) at[b + 1] += at[b];
+    heavy.resize(nheavy);
+    for (int64_t i = 0; i < nn; ++i)
+        if (count[i] > kIncHead) heavy[at[most - batches(i)]++] = (int32_t)i;
+    hptr.reserve(nheavy + 1);
+    for (int64_t i = 0; i < nn; ++i) fill[i] = kIncHead * i;
+    for (int32_t i : heavy) {
+        fill[i] = hptr.back();
+        hptr.push_back(hptr.back() + kIncHead * batches(i));
+    }
+    std::vector<uint32_t> head((size_t)std::max<int64_t>(1, nn) * kIncHead, kIncNone), inc(std::max<int64_t>(1, hptr.back()), kIncNone);
+    for (int32_t i : heavy) head[(size_t)i * kIncHead] = kIncHeavy;
+    visit([&](int64_t node, uint32_t code) { (count[node] <= kIncHead ? head : inc)[fill[node]++] = code; });
+    m.n_heavy = (int64_t)heavy.size();
     const size_t slot_bytes = (size_t)std::max<int64_t>(1, nv) * 32 * sizeof(double);
-    if (!upload(&m.d.inc_head, head, err) || !upload(&m.d.inc_ptr, optr, err) || !upload(&m.d.inc, oinc, err)) return false;
+    if (!upload(&m.d.inc_head, head, err) || !upload(&m.d.inc_heavy, heavy, err) || !upload(&m.d.inc_ptr, hptr, err) ||
+        !upload(&m.d.inc, inc, err))
+        return false;
     if (!check(cudaMalloc((void**)&m.d.sv, slot_bytes), err, "cudaMalloc") ||
         !check(cudaMalloc((void**)&m.d.ss, (size_t)std::max<int64_t>(1, ns) * 32 * sizeof(double)), err, "cudaMalloc"))
         return false;
@@ -714,7 +721,7 @@ void device_free(Mesh& m) {
     DeviceMesh& d = m.d;
     void* ptrs[] = {d.key, d.anc, d.lev, d.conn, d.hpar, d.tv, d.tn, d.tc, d.bt_off, d.bt_idx, d.rg_off, d.rg_idx,
                     d.marker, d.cflags, d.out_list, d.out_conn, d.out_lev, d.out_prob, d.eprob, d.pmu, d.pmuf, d.cut_list, d.cut_off, d.cut_pts, d.cut_pts_f, d.cut_order, d.sq_elem, d.sq_x,
-                    d.sq_n, d.sq_w, d.sq_taub, d.sq_src, d.sq_hosts, d.pen_elem, d.pen_q, d.pen_slot, d.pen, d.inc_head, d.inc_ptr, d.inc, d.sv, d.ss, d.sq_list, d.sq_off, d.bcflag, d.bcmask_user, d.bcval_user, m.scratch, d.nd_f, d.nd_d, d.slot,
+                    d.sq_n, d.sq_w, d.sq_taub, d.sq_src, d.sq_hosts, d.pen_elem, d.pen_q, d.pen_slot, d.pen, d.inc_head, d.inc_heavy, d.inc_ptr, d.inc, d.sv, d.ss, d.sq_list, d.sq_off, d.bcflag, d.bcmask_user, d.bcval_user, m.scratch, d.nd_f, d.nd_d, d.slot,
                     d.counters, d.fq_items, d.fq_cnt};
     for (void* p : ptrs)
         if (p) cudaFree(p);

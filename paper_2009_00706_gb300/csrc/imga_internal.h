@@ -105,8 +105,9 @@ struct DeviceMesh {
     int64_t* pen_slot = nullptr;
     double* pen = nullptr;
     // deterministic scatter: node -> (slot, corner, weight) incidence and the element-contribution slots
-    uint32_t* inc_head = nullptr; // [n_nodes][kIncHead] first entries of each node's list (kIncNone pads)
-    int64_t* inc_ptr = nullptr;   // [n_nodes + 1] the rest of each list (CSR)
+    uint32_t* inc_head = nullptr; // [n_nodes][kIncHead] each node's list (kIncNone pads), or kIncHeavy first
+    int32_t* inc_heavy = nullptr; // [n_heavy] nodes with more than kIncHead entries
+    int64_t* inc_ptr = nullptr;   // [n_heavy + 1] their lists (CSR, padded to multiples of kIncHead)
     uint32_t* inc = nullptr;      // bits 0-2 corner, 3-4 weight code, 5-31 global slot
     void* sv = nullptr;           // volume slots [n_vslots][8][4] of the element precision (sized for float64)
     double* ss = nullptr;         // surface slots [n_sslots][8][4] float64
@@ -130,7 +131,7 @@ struct DeviceMesh {
 
 // node incidence lists of the deterministic scatter: fixed head length and its padding code
 constexpr int kIncHead = 8;
-constexpr uint32_t kIncNone = 0xFFFFFFFFu;
+constexpr uint32_t kIncNone = 0xFFFFFFFFu, kIncHeavy = 0xFFFFFFFEu;   // (no slot reaches either: at most 2^27 - 1)
 
 // elements hosting at least this many surface points take the warp-per-element surface kernel
 constexpr int kNitscheDenseMin = 8;
@@ -180,6 +181,7 @@ struct Mesh {
     std::vector<int32_t> sq_hosts;       // every element hosting a surface point (increasing)
     std::vector<int32_t> pen_elem;       // surface-hosting elements in device point order (nitsche_penalty)
     std::vector<int64_t> sq_off_h;       // host copy of DeviceMesh::sq_off
+    int64_t n_heavy = 0;                 // nodes with more than kIncHead incidence entries
     int64_t n_vslots = 0, n_sslots = 0;  // deterministic scatter: volume slots (active elements), surface slots
     bool deterministic = true;           // IMGA_OPT_DETERMINISTIC: slots + ordered node sums (1) or atomics (0)
     std::vector<uint8_t> bcflag;
