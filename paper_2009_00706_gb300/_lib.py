@@ -23,7 +23,7 @@ SOURCES = [
     ("mesh_host.cpp", ["-Xcompiler", "-ffp-contract=off", "-Xcompiler", "-fopenmp"]),
     ("capi.cpp", []),
     ("batch.cpp", []),
-    ("geom.cu", ["-fmad=false"]),
+    ("geom.cu", ["-fmad=false", "-Xcompiler", "-fopenmp"]),
     ("vms.cu", []),
     ("jac.cu", []),
     ("solver.cu", []),

@@ -73,6 +73,9 @@ struct DeviceMesh {
     double* tc = nullptr;         // [n_tri][3]
     int32_t* bt_off = nullptr;    // [n_elem + 1]
     int32_t* bt_idx = nullptr;
+    float* tri_f = nullptr;       // [n_tri][8] centroid, its 1-norm, unit normal in float32 (filter of the normal test)
+    float* tri_box = nullptr;     // [n_tri][8] widened bounding box, valid ray directions (filter of the ray test)
+    int32_t* leaf_lut = nullptr;  // [2^leaf_lut_bits + 1] leaf table over leading Morton bits
     int32_t* rg_off = nullptr;    // ray grid
     int32_t* rg_idx = nullptr;
     // classification results
@@ -169,6 +172,7 @@ struct Mesh {
     TriHost tri;
     std::vector<int32_t> bt_off, bt_idx;
     RayGridHost grid;
+    int leaf_lut_bits = 0;               // see DeviceMesh::leaf_lut
     std::vector<int8_t> marker;
     std::vector<uint8_t> cflags;
     std::vector<int32_t> out_list, cut_list;

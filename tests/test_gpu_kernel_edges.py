@@ -167,3 +167,37 @@ def test_float64_block_jacobi_matches_mixed(dev):
         its.append(st["krylov_per_newton"])
     # the same blocks to float32 rounding: the same iterations, give or take one
     assert np.abs(np.array(its[0]) - np.array(its[1])).max() <= 1
+
+
+# ---- in/out: the float32 filters leave every flag to float64 where they cannot decide ----
+@pytest.mark.parametrize("lo", [(0.0, 0.0, 0.0), (1000.0, -2000.0, 500.0)])
+@pytest.mark.parametrize("body", ["sphere", "box", "truck"])
+def test_classify_near_the_surface(dev, body, lo):
+    lo = np.array(lo)
+    if body == "sphere":
+        tri, edge, lev = I.icosphere(3, 0.2, C, 1e-4, 2), 1.0, 5
+    elif body == "box":      # faces on element planes, edge-on to the rays
+        tri, edge, lev = I.grid_box((0.25, 0.25, 0.375), (0.75, 0.5, 0.625), 1 / 16), 1.0, 4
+    else:
+        tri, edge, lev = I.truck(0.7, 3.2, 2.7, 8, 1e-5, 3), 6.4, 5
+    tri = tri + lo
+    args = (tuple(lo), tuple(lo + edge), lev, [], tri, 1)
+    g, o = api.Mesh(*args), OracleMesh(*args)
+    rs = np.random.RandomState(1)
+    t = tri[rs.randint(0, tri.shape[0], 4000)]
+    bary = rs.dirichlet((1, 1, 1), 4000)
+    bary[:1000, 0] = 0                      # on edges, and at vertices
+    bary[:500, 1] = 0
+    bary /= bary.sum(1, keepdims=True)
+    n = np.cross(t[:, 1] - t[:, 0], t[:, 2] - t[:, 0])
+    n /= np.linalg.norm(n, axis=1, keepdims=True)
+    off = np.concatenate([[0.0], 10.0 ** np.arange(-15, -1)])
+    off = np.concatenate([off, -off])[rs.randint(0, 30, 4000)] * edge
+    far = lo + edge * rs.rand(4000, 3)
+    pts = np.concatenate([np.einsum("ni,nij->nj", bary, t) + off[:, None] * n, far, np.vstack([lo, lo + edge, lo - 1, np.full(3, np.nan)])])
+    want = o.classify(np.nan_to_num(pts, nan=-1e9))
+    assert np.array_equal(g.classify(T(pts, dev)).cpu().numpy(), want)
+    # every ray by itself: +x rays through edge-on faces, grazes re-cast along +y and +z
+    g.classify_rays_only(True)
+    rays = g.classify(T(pts[4000:8000], dev)).cpu().numpy()
+    assert np.array_equal(rays, want[4000:8000])
