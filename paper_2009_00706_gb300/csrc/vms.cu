@@ -1754,6 +1754,8 @@ int conversion_selftest(int64_t n, uint64_t seed, int64_t* mismatches, std::stri
     return 0;
 }
 
+constexpr int64_t kForkOut = 65536;
+
 // Residual / J v on `stream` without the graph path, every kernel returning at once while *skip is
 // nonzero (steps of a solver loop that is itself captured in a graph).
 int vms_apply_skip(const Mesh& m, const double* u, const double* up, const double* up2, const double* f,
@@ -1764,10 +1766,21 @@ int vms_apply_skip(const Mesh& m, const double* u, const double* up, const doubl
     A.skip = skip;
     const bool jv = v != nullptr;
     if (!A.sv && cudaMemsetAsync(out, 0, (size_t)m.n_nodes() * 4 * sizeof(double), s) != cudaSuccess) return 1;
+    // a small mesh's Out kernel is a few microseconds, so its latency-bound neighbours run beside it here
+    // too; from kForkOut Out elements on they gain less than the fork and join cost the captured step
+    // (2.0 M elements: 1.96 s a Newton step in one stream, 2.00 s forked; 7.3 k elements: a Newton
+    // solve 3 % faster forked)
+    cudaStream_t s1 = nullptr, s2 = nullptr;
+    cudaEvent_t* ev = nullptr;
+    if (m.concurrent && m.side[0] && (int64_t)m.out_list.size() < kForkOut) {
+        s1 = (cudaStream_t)m.side[0];
+        s2 = (cudaStream_t)m.side[1];
+        ev = (cudaEvent_t*)const_cast<Mesh&>(m).fork_ev;
+    }
     if (precision == 0) {
-        if (jv) launch_all<double, true>(m, A, s, nullptr, nullptr, nullptr, nullptr, generic); else launch_all<double, false>(m, A, s, nullptr, nullptr, nullptr, nullptr, generic);
+        if (jv) launch_all<double, true>(m, A, s, nullptr, s1, s2, ev, generic); else launch_all<double, false>(m, A, s, nullptr, s1, s2, ev, generic);
     } else {
-        if (jv) launch_all<float, true>(m, A, s); else launch_all<float, false>(m, A, s);
+        if (jv) launch_all<float, true>(m, A, s, nullptr, s1, s2, ev); else launch_all<float, false>(m, A, s, nullptr, s1, s2, ev);
     }
     launch_strong_rows(m, A, ph, jv, s, true, precision);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
