@@ -113,10 +113,7 @@ void gemm(cudaStream_t s, int M, int N, int K, const bf16* A, int64_t sam, int64
 //   50,003 rows: 2,625 -> 161 us (2.55 TB/s of X and Y).
 // ------------------------------------------------------------------------------------------
 constexpr int kW = 128;            // width of the fused path
-constexpr int kKT = 32;            // k per stage of the first layer
-constexpr int kKS = kKT + 8;       // row stride of a stage (floats of X, bf16 of W1): conflict-free fragment reads
-constexpr int kHS = kW + 8;        // row stride of activations and of a weight chunk
-constexpr int kNC = 64;            // output columns per weight chunk of the second and third layer
+constexpr int kHS = kW + 8;        // row stride of activations and of a weight chunk: conflict-free fragment reads
 
 __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // asynchronous copies of 16 or 4 bytes, the first `valid` of them from src, the rest zeros
@@ -143,24 +140,26 @@ struct MlpTrainIO {           // what a training step keeps of the forward pass
     double* loss;             // += sum (y - t)^2
 };
 
-// BM rows per CTA, 4 warps: for BM = 64 two by two over (rows, columns), otherwise all four over the
-// columns.  STAGES k-tiles of X (fp32) and W1 in flight; the same shared memory then holds the
-// activations and two chunks of W2 / W3.
-template <int BM, int STAGES> struct FwdShape {
-    static constexpr int WM = BM == 64 ? 2 : 1, WN = 4 / WM, MI = BM / (16 * WM);
-    static constexpr int XS = BM * kKS * 4, WS = kW * kKS * 2;         // bytes of a stage
-    static constexpr int HB = BM * kHS * 2, CB = kNC * kHS * 2;        // bytes of the activations, of a weight chunk
+// BM rows per CTA of NT threads: for BM = 64 two rows of warps, otherwise one, the others over the columns.
+// STAGES k-tiles of KT columns of X (fp32) and W1 in flight; the same shared memory then holds the
+// activations and two chunks of NC rows of W2 / W3.
+template <int BM, int NT, int KT, int NC, int STAGES> struct FwdShape {
+    static constexpr int WM = BM == 64 ? 2 : 1, WN = NT / 32 / WM, MI = BM / (16 * WM);
+    static constexpr int KS = KT + 8;                                  // row stride of a stage (floats of X, bf16 of W1)
+    static constexpr int XS = BM * KS * 4, WS = kW * KS * 2;           // bytes of a stage
+    static constexpr int HB = BM * kHS * 2, CB = NC * kHS * 2;         // bytes of the activations, of a weight chunk
     static constexpr int smem = STAGES * (XS + WS) > HB + 2 * CB ? STAGES * (XS + WS) : HB + 2 * CB;
+    static_assert(kW / WN % 16 == 0 && NC / WN % 16 == 0 && KT % 16 == 0 && kW % NC == 0, "tiles of pairs of 8 columns");
 };
 
-template <int BM, int STAGES, bool TRAIN>
-__global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad, const float* __restrict__ X, int64_t ldx,
-                                                 int xvec, const bf16* __restrict__ W1, const float* __restrict__ b1,
-                                                 const bf16* __restrict__ W2, const float* __restrict__ b2,
-                                                 const bf16* __restrict__ W3, const float* __restrict__ b3, int nout,
-                                                 float* __restrict__ Y, MlpTrainIO io) {
-    typedef FwdShape<BM, STAGES> Sh;
-    constexpr int WN = Sh::WN, MI = Sh::MI, N1 = kW / WN / 8, N2 = kNC / WN / 8;
+template <int BM, int NT, int KT, int NC, int STAGES, bool TRAIN>
+__global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad, const float* __restrict__ X, int64_t ldx,
+                                                int xvec, const bf16* __restrict__ W1, const float* __restrict__ b1,
+                                                const bf16* __restrict__ W2, const float* __restrict__ b2,
+                                                const bf16* __restrict__ W3, const float* __restrict__ b3, int nout,
+                                                float* __restrict__ Y, MlpTrainIO io) {
+    typedef FwdShape<BM, NT, KT, NC, STAGES> Sh;
+    constexpr int WN = Sh::WN, MI = Sh::MI, N1 = kW / WN / 8, N2 = NC / WN / 8, kKT = KT, kKS = Sh::KS, kNC = NC;
     extern __shared__ __align__(16) unsigned char sm[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
     const int wm = (warp / WN) * 16 * MI, wn = warp % WN;
@@ -172,7 +171,7 @@ __global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad
         if (kt < nkt) {
             float* x = xs(kt % STAGES);
             bf16* w = ws(kt % STAGES);
-            for (int i = tid; i < BM * (kKT / 4); i += 128) {
+            for (int i = tid; i < BM * (kKT / 4); i += NT) {
                 const int r = i / (kKT / 4), c = i % (kKT / 4) * 4, gc = kt * kKT + c;
                 const int64_t gr = m0 + r;
                 const int left = gr < n ? max(0, min(4, nin - gc)) : 0;
@@ -181,7 +180,7 @@ __global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad
                 else
                     for (int j = 0; j < 4; ++j) cpz4(x + r * kKS + c + j, j < left ? src + j : X, j < left ? 4 : 0);
             }
-            for (int i = tid; i < kW * (kKT / 8); i += 128) {
+            for (int i = tid; i < kW * (kKT / 8); i += NT) {
                 const int r = i / (kKT / 8), c = i % (kKT / 8) * 8, gc = kt * kKT + c;
                 const bool in = gc < nin_pad;
                 cpz16(w + r * kKS + c, in ? W1 + (int64_t)r * nin_pad + gc : W1, in ? 16 : 0);
@@ -243,7 +242,7 @@ __global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad
             const bf16* W = l2 ? W2 : W3;
             const int n0 = (l2 ? k : k - kW / kNC) * kNC, nr = l2 ? kW : nout;
             bf16* w = chunk_buf(k);
-            for (int i = tid; i < kNC * (kW / 8); i += 128) {
+            for (int i = tid; i < kNC * (kW / 8); i += NT) {
                 const int r = i / (kW / 8), c = i % (kW / 8) * 8;
                 const bool in = n0 + r < nr;
                 cpz16(w + r * kHS + c, in ? W + (int64_t)(n0 + r) * kW + c : W, in ? 16 : 0);
@@ -317,6 +316,20 @@ __global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad
                     put_h(&z2[k][i][j][q], b2, wm + 16 * i + gid + q * 4, k * kNC + wn * (kNC / WN) + 8 * j + 2 * tig, io.h2);
     float lhi = 0.f, llo = 0.f;   // training: sum (y - t)^2 of this thread in two floats
     for (int k = kW / kNC; k < nchunk; ++k) {
+        const int n0 = (k - kW / kNC) * kNC + wn * (kNC / WN) + 2 * tig;
+        float2 tg[TRAIN ? MI : 1][TRAIN ? N2 : 1][2];
+        if constexpr (TRAIN) {   // the chunk's targets come in beside its weights
+#pragma unroll
+            for (int i = 0; i < MI; ++i)
+#pragma unroll
+                for (int j = 0; j < N2; ++j)
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int64_t r = m0 + wm + 16 * i + gid + q * 8;
+                        const int c = n0 + 8 * j;
+                        tg[i][j][q] = r < n && c < nout ? __ldg(reinterpret_cast<const float2*>(io.T + r * nout + c)) : make_float2(0.f, 0.f);
+                    }
+        }
         cp_wait<1>();
         __syncthreads();
         if (k == kW / kNC) load_a();
@@ -324,7 +337,6 @@ __global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad
         times_chunk(k, o);
         __syncthreads();
         load_chunk(k + 2);
-        const int n0 = (k - kW / kNC) * kNC + wn * (kNC / WN) + 2 * tig;
 #pragma unroll
         for (int i = 0; i < MI; ++i)
 #pragma unroll
@@ -338,7 +350,7 @@ __global__ void __launch_bounds__(128) mlp_fused(int64_t n, int nin, int nin_pad
                     if constexpr (!TRAIN) {
                         *reinterpret_cast<float2*>(Y + r * nout + c) = make_float2(y0, y1);
                     } else {
-                        const float2 t = __ldg(reinterpret_cast<const float2*>(io.T + r * nout + c));
+                        const float2 t = tg[i][j][q >> 1];
                         const float d0 = y0 - t.x, d1 = y1 - t.y;
                         *reinterpret_cast<uint32_t*>(io.dy + r * nout + c) = cvt2(d0 * io.inv_scale, d1 * io.inv_scale);
                         // exact square (two floats) added with TwoSum: float64's narrow pipe stays out of it
@@ -706,29 +718,30 @@ static void mlp_sync_bf16(Mlp& M, cudaStream_t s) { to_bf16<<<nblk(M.nparam), 25
 // The fused kernels serve the preconditioner's width; rows of 16 bytes in every bf16 matrix need nout % 8 == 0.
 static bool mlp_fast(const Mlp& M) { return M.w == kW && M.nout % 8 == 0; }
 
-template <int BM, int STAGES, bool TRAIN>
+template <int BM, int NT, int KT, int NC, int STAGES, bool TRAIN>
 static void launch_fused(const Mlp& M, const float* X, int64_t ldx, int64_t n, float* Y, const MlpTrainIO& io, cudaStream_t s) {
-    typedef FwdShape<BM, STAGES> Sh;
+    typedef FwdShape<BM, NT, KT, NC, STAGES> Sh;
     static std::atomic<unsigned> ready{0};   // devices whose shared-memory limit is raised
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 32 || !((ready.load() >> dev) & 1u)) {
-        cudaFuncSetAttribute(mlp_fused<BM, STAGES, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem);
+        cudaFuncSetAttribute(mlp_fused<BM, NT, KT, NC, STAGES, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem);
         if (dev < 32) ready.fetch_or(1u << dev);
     }
     const int xvec = ((uintptr_t)X & 15) == 0 && ldx % 4 == 0;
-    mlp_fused<BM, STAGES, TRAIN><<<(unsigned)((n + BM - 1) / BM), 128, Sh::smem, s>>>(
+    mlp_fused<BM, NT, KT, NC, STAGES, TRAIN><<<(unsigned)((n + BM - 1) / BM), NT, Sh::smem, s>>>(
         n, M.nin, M.nin_pad, X, ldx, xvec, M.Pb + M.off(0), M.P + M.off(1), M.Pb + M.off(2), M.P + M.off(3), M.Pb + M.off(4),
         M.P + M.off(5), M.nout, Y, io);
 }
 
 // Rows per CTA: 64 (the weights are read from L2 once per 64 rows) when that still gives two CTAs per SM,
-// fewer for fewer rows, so that the chip has work: @RULE@
+// fewer for fewer rows, so that the chip has work (9,000 rows: 51 us with 32).  From 64 x 2 x 152 rows on 64; the small tile takes 8
+// warps, deep stages and wide chunks because a CTA is alone on its SM (1,024-row training steps: 61 -> 33 us).
 template <bool TRAIN>
 static void mlp_fused_rows(const Mlp& M, const float* X, int64_t ldx, int64_t n, float* Y, const MlpTrainIO& io, cudaStream_t s) {
-    if (n >= 64 * 152 * 2) launch_fused<64, 3, TRAIN>(M, X, ldx, n, Y, io, s);
-    else if (n >= 32 * 152) launch_fused<32, 4, TRAIN>(M, X, ldx, n, Y, io, s);
-    else launch_fused<16, 6, TRAIN>(M, X, ldx, n, Y, io, s);
+    if (n >= 64 * 152 * 2) launch_fused<64, 128, 32, 64, 3, TRAIN>(M, X, ldx, n, Y, io, s);
+    else if (n >= 32 * 152) launch_fused<32, 128, 32, 64, 4, TRAIN>(M, X, ldx, n, Y, io, s);
+    else launch_fused<16, 256, 64, 128, 4, TRAIN>(M, X, ldx, n, Y, io, s);
 }
 
 // forward and backward of a batch on the fused path: gradients into M.G, loss added to M.loss
