@@ -9,7 +9,7 @@
 //
 //   float64: jac_out64, jac_cut64, jac_surf64 (lane = column of k_e); float32 element arithmetic:
 //   jac_out     8 threads per Out element (thread c: Gauss point c, then node c's 4 rows)
-//   jac_cut     one warp per Intercepted element, 32 sub-cell points per step, lane = row
+//   jac_cut     four warps per Intercepted element, 32 sub-cell points per step, lane = point, then row
 //   jac_nitsche one thread per surface point (a warp per block: there are few points, and each is long)
 // Mode FULL writes k_e for requested elements (slot map); mode DIAG adds the 4x4 diagonal blocks
 // of sum_e M_e^T k_e M_e (each corner's own block times the squared hanging weights; the
@@ -55,7 +55,7 @@ __device__ __forceinline__ int corner_nodes(const Args& A, int32_t id, int32_t n
 // M_e^T k_e M_e (Algorithm 2): every parent pair (p, q) receives w_p w_q v in block (p, q), entry at[j]
 // (4 x row component + column component).  The row is searched once per corner pair: entry by entry the
 // searches were most of the assembly (43.6 k elements,
-// mixed: 5.37 -> 2.01 ms with the basis tables, the shared test functions and the adds below).
+// mixed: 5.37 -> 1.86 ms with the basis tables, the shared test functions and the adds below).
 // A warp adds whole blocks from shared memory where it can (bsr_add_blocks): 16 lanes on the 128 bytes of a
 // block make 4 L2 transactions of what lane-by-lane adds make 16 of.
 // Float entries are weighted (powers of two: exact) and tested in float32 and widened on the integer pipe:
@@ -78,11 +78,11 @@ __device__ __forceinline__ void bsr_add(const Args& A, int32_t ida, int32_t idb,
         }
 }
 
-// 32 blocks of a warp, entry (block m, j) given by v(m, j), to positions s_pos[m] (-1: none)
-template <class V>
+// N blocks by a warp, entry (block m, j) given by v(m, j), to positions s_pos[m] (-1: none)
+template <int N, class V>
 __device__ __forceinline__ void bsr_add_blocks(const int64_t* s_pos, V v, int lane, double* __restrict__ val) {
 #pragma unroll 4
-    for (int m = lane >> 4; m < 32; m += 2) {
+    for (int m = lane >> 4; m < N; m += 2) {
         const int64_t pos = s_pos[m];
         const auto x = v(m, lane & 15);
         if (pos >= 0 && x != 0) atomicAdd(val + 16 * pos + (lane & 15), wide(x));
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
             const bool plain = plain_corner(A, id) && plain_corner(A, idb);
             s_pos[w][lane] = work && plain ? bsr_find(A.bptr, A.bidx, id, idb) : -1;
             __syncwarp();
-            bsr_add_blocks(s_pos[w], [&](int m, int j) { return s_blk[w][m][j]; }, lane, K);
+            bsr_add_blocks<32>(s_pos[w], [&](int m, int j) { return s_blk[w][m][j]; }, lane, K);
             for (unsigned need = __ballot_sync(0xffffffffu, work && !plain); need; need &= need - 1) {
                 const int src = __ffs(need) - 1;
                 const int32_t ha = __shfl_sync(0xffffffffu, id, src), hb = __shfl_sync(0xffffffffu, idb, src);
@@ -272,37 +272,40 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
     if (MODE == DIAG && work) add_diag(A, id, diag, D);
 }
 
-constexpr int JWPB = 2;   // warps per block of jac_cut
+constexpr int JWPB = 4;   // warps per element of jac_cut
 
+// An Intercepted element: a block of four warps, lane = sub-cell point (32 at a time), each warp the seeds
+// of two corners.  A warp alone with an element ran its hundreds of points 32 seeds deep while most of the
+// chip had nothing left (7.3 k element sphere, 776 elements: 660 -> 361 us an assembly).
 template <class T, int MODE>
 __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __restrict__ list,
                                                      const int64_t* __restrict__ off, const void* __restrict__ pts,
-                                                     const int32_t* __restrict__ order, int64_t n,
-                                                     const int32_t* __restrict__ slot, double* __restrict__ K,
-                                                     double* __restrict__ D) {
-    __shared__ __align__(16) T s_nd[JWPB][8][CS];
-    // a point's coefficients for the four seeds of a corner (80-byte rows: conflict-free 16-byte stores):
-    // the contraction, bound by shared memory, then reads a point's test functions once for four sums
-    __shared__ __align__(16) T s_cf[JWPB][4][32][20];
-    __shared__ __align__(16) T s_bas[JWPB][32][8][4];  // a point's test functions (phi, reference gradient), once for all seeds
-    __shared__ T s_acc[JWPB][32][32];                  // the element's columns so far
+                                                     const int32_t* __restrict__ order, const int32_t* __restrict__ slot,
+                                                     double* __restrict__ K, double* __restrict__ D) {
+    constexpr int NB = 8 / JWPB;                    // corners (of the seeds) per warp
+    __shared__ __align__(16) T s_nd[8][CS];
+    // a point's coefficients for the four seeds of a corner, in fours (component c: phi and gradient
+    // coefficients) at place c ^ (point / 2 & 3): conflict-free 16-byte stores.  The contraction, bound by shared
+    // memory, reads a point's test functions once for four sums.
+    __shared__ __align__(16) T s_cf[JWPB][4][32][16];
+    __shared__ __align__(16) T s_bas[32][8][4];     // a point's test functions (phi, reference gradient), once for all seeds
+    __shared__ T s_acc[32][32];                     // the element's columns so far
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if ((int64_t)blockIdx.x * JWPB + w >= n) return;
-    const int64_t idx = order[(int64_t)blockIdx.x * JWPB + w];
+    const int64_t idx = order[blockIdx.x];
     const int32_t e = list[idx];
     const int32_t sl = MODE == FULL ? slot[e] : 0;
     if (sl < 0) return;
     int32_t my_id = 0;
     if (lane < 8) {
         my_id = A.conn[8 * (int64_t)e + lane];
-        corner_data<T, false>(A, my_id, &s_nd[w][lane][0]);
+        if (w == 0) corner_data<T, false>(A, my_id, &s_nd[lane][0]);
     }
-    __syncwarp();
+    __syncthreads();
     const T g = lvl_g<T>(A, A.lev[e]);
     const T det = lvl_w<T>(A, A.lev[e]);
     const int a = lane >> 2, comp = lane & 3;
-    T* acc = &s_acc[w][0][lane];   // acc[32 s]: row `lane` of column s
-    for (int s = 0; s < 32; ++s) acc[32 * s] = T(0);
+    T* acc = &s_acc[0][lane];   // acc[32 s]: row `lane` of column s
+    for (int s = 4 * NB * w; s < 4 * NB * (w + 1); ++s) acc[32 * s] = T(0);
     const int64_t q0 = off[idx], q1 = off[idx + 1];
     for (int64_t base = q0; base < q1; base += 32) {
         const int64_t q = base + lane;
@@ -312,39 +315,42 @@ __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __re
         T fm[3], fp[3];
         for (int k = 0; k < 3; ++k) { fm[k] = T(0.5) * (T(1) - pt[k]); fp[k] = T(0.5) * (T(1) + pt[k]); }
         Fields<T, T> V;
-        interp<T, T>(A, fm, fp, &s_nd[w][0][0], CS, g, V);
+        interp<T, T>(A, fm, fp, &s_nd[0][0], CS, g, V);
         const T wq = have ? pt[3] * det : T(0), wqg = wq * g;
         const int m = (int)min((int64_t)32, q1 - base);
-        for (int cc = 0; cc < 8; ++cc) {
+        for (int cc = NB * w; cc < NB * (w + 1); ++cc) {
             const T s0 = (cc & 1) ? T(1) : T(-1), s1 = (cc & 2) ? T(1) : T(-1), s2 = (cc & 4) ? T(1) : T(-1);
             const T f0 = T(0.5) * (T(1) + s0 * pt[0]), f1 = T(0.5) * (T(1) + s1 * pt[1]), f2 = T(0.5) * (T(1) + s2 * pt[2]);
-            st4s<T>(&s_bas[w][lane][cc][0], f0 * f1 * f2, T(0.5) * s0 * f1 * f2, T(0.5) * s1 * f0 * f2, T(0.5) * s2 * f0 * f1);
+            st4s<T>(&s_bas[lane][cc][0], f0 * f1 * f2, T(0.5) * s0 * f1 * f2, T(0.5) * s1 * f0 * f2, T(0.5) * s2 * f0 * f1);
         }
-        for (int b = 0; b < 8; ++b) {
+        __syncthreads();
+        for (int b = NB * w; b < NB * (w + 1); ++b) {
             T phb, dphb[3], d2b[3];
             corner_basis<T>(fm, fp, b, phb, dphb, d2b);
 #pragma unroll 1   // as in jac_out
             for (int k = 0; k < 4; ++k) {
-            Fields<Dual<T>, T> F;
-            seed_fields<T>(A, V, g, phb, dphb, d2b, k, F);
-            Dual<T> cf[16];
-            pointwise<Dual<T>, T>(A, Phys<T>(A, prob_of(A, e)), F, g, cf);
-            T cw[16];   // (component, its phi and gradient coefficients) in fours
-            for (int qq = 0; qq < 16; ++qq) cw[qq] = ((qq < 3 || qq == 12) ? wq : wqg) * cf[qq].d;
-            for (int i = 0; i < 3; ++i) st4s<T>(&s_cf[w][k][lane][4 * i], cw[i], cw[3 + 3 * i], cw[4 + 3 * i], cw[5 + 3 * i]);
-            st4s<T>(&s_cf[w][k][lane][12], cw[12], cw[13], cw[14], cw[15]);
+                Fields<Dual<T>, T> F;
+                seed_fields<T>(A, V, g, phb, dphb, d2b, k, F);
+                Dual<T> cf[16];
+                pointwise<Dual<T>, T>(A, Phys<T>(A, prob_of(A, e)), F, g, cf);
+                T cw[16];
+                for (int qq = 0; qq < 16; ++qq) cw[qq] = ((qq < 3 || qq == 12) ? wq : wqg) * cf[qq].d;
+                T* dst = &s_cf[w][k][lane][0];
+                const int x = (lane >> 1) & 3;
+                for (int i = 0; i < 3; ++i) st4s<T>(dst + 4 * (i ^ x), cw[i], cw[3 + 3 * i], cw[4 + 3 * i], cw[5 + 3 * i]);
+                st4s<T>(dst + 4 * (3 ^ x), cw[12], cw[13], cw[14], cw[15]);
             }
             __syncwarp();
             T sum[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll 2
             for (int j = 0; j < m; ++j) {
                 T B[4];
-                ld4s<T>(&s_bas[w][j][a][0], B);
+                ld4s<T>(&s_bas[j][a][0], B);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     // (multiply-adds spelled out: contracted otherwise, the sum has other last bits)
                     T C[4];
-                    ld4s<T>(&s_cf[w][k][j][4 * comp], C);
+                    ld4s<T>(&s_cf[w][k][j][4 * (comp ^ ((j >> 1) & 3))], C);
                     T t = B[0] * C[0];
                     t = fma(B[1], C[1], t);
                     t = fma(B[2], C[2], t);
@@ -355,36 +361,37 @@ __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __re
             for (int k = 0; k < 4; ++k) acc[32 * (4 * b + k)] += sum[k];
             __syncwarp();
         }
+        __syncthreads();   // the test functions are replaced
     }
     if (MODE == FULL) {
-        for (int s = 0; s < 32; ++s) K[(int64_t)sl * 1024 + lane * 32 + s] = (double)acc[32 * s];
-    } else if (MODE == BSR) {
-        __syncwarp();
-        int64_t* s_pos = reinterpret_cast<int64_t*>(&s_bas[w][0][0][0]);   // (the points are done)
+        for (int s = 4 * NB * w; s < 4 * NB * (w + 1); ++s) K[(int64_t)sl * 1024 + lane * 32 + s] = (double)acc[32 * s];
+        return;
+    }
+    __syncthreads();
+    if (MODE == BSR) {
+        constexpr int NP = 64 / JWPB;   // corner pairs per warp: pair (m / 8, m % 8), m = NP w ...
+        int64_t* s_pos = reinterpret_cast<int64_t*>(&s_cf[w][0][0][0]);   // (the points are done)
         const unsigned hanging = __ballot_sync(0xffffffffu, lane < 8 && !plain_corner(A, my_id)) & 0xffu;
-        for (int half = 0; half < 2; ++half) {   // corner pairs (4 half + m / 8, m % 8)
-            const int pa = 4 * half + (lane >> 3), pb = lane & 7;
-            const int32_t ida = __shfl_sync(0xffffffffu, my_id, pa), idb = __shfl_sync(0xffffffffu, my_id, pb);
-            s_pos[lane] = (hanging >> pa | hanging >> pb) & 1u ? -1 : bsr_find(A.bptr, A.bidx, ida, idb);
-            __syncwarp();
-            bsr_add_blocks(s_pos, [&](int m, int j) {
-                return s_acc[w][4 * (m & 7) + (j & 3)][4 * (4 * half + (m >> 3)) + (j >> 2)];
-            }, lane, K);
-            __syncwarp();
-        }
-        if (hanging)
-            for (int m = 0; m < 64; ++m) {
-                const int pa = m >> 3, pb = m & 7;
-                if (!((hanging >> pa | hanging >> pb) & 1u)) continue;
-                const int32_t ha = __shfl_sync(0xffffffffu, my_id, pa), hb = __shfl_sync(0xffffffffu, my_id, pb);
-                bsr_add_hanging(A, ha, hb, [&](int j) { return s_acc[w][4 * pb + (j & 3)][4 * pa + (j >> 2)]; }, lane, K);
-            }
-    } else {
-        // lane (a, comp) holds row comp of corner a's own block in columns 4a .. 4a+3
+        const int pm = NP * w + (lane & (NP - 1)), pa = pm >> 3, pb = pm & 7;
+        const int32_t ida = __shfl_sync(0xffffffffu, my_id, pa), idb = __shfl_sync(0xffffffffu, my_id, pb);
+        if (lane < NP) s_pos[lane] = (hanging >> pa | hanging >> pb) & 1u ? -1 : bsr_find(A.bptr, A.bidx, ida, idb);
         __syncwarp();
+        bsr_add_blocks<NP>(s_pos, [&](int m, int j) {
+            const int q = NP * w + m;
+            return s_acc[4 * (q & 7) + (j & 3)][4 * (q >> 3) + (j >> 2)];
+        }, lane, K);
+        if (hanging)
+            for (int m = NP * w; m < NP * (w + 1); ++m) {
+                const int ha = m >> 3, hb = m & 7;
+                if (!((hanging >> ha | hanging >> hb) & 1u)) continue;
+                const int32_t ia = __shfl_sync(0xffffffffu, my_id, ha), ib = __shfl_sync(0xffffffffu, my_id, hb);
+                bsr_add_hanging(A, ia, ib, [&](int j) { return s_acc[4 * hb + (j & 3)][4 * ha + (j >> 2)]; }, lane, K);
+            }
+    } else if (w == 0) {
+        // lane (a, comp) holds row comp of corner a's own block in columns 4a .. 4a+3
         double blk[16];
         for (int i = 0; i < 4; ++i)
-            for (int k = 0; k < 4; ++k) blk[i * 4 + k] = (double)s_acc[w][4 * a + k][4 * a + i];
+            for (int k = 0; k < 4; ++k) blk[i * 4 + k] = (double)s_acc[4 * a + k][4 * a + i];
         const int32_t id = __shfl_sync(0xffffffffu, my_id, a);
         if (comp == 0) add_diag(A, id, blk, D);
     }
@@ -989,7 +996,7 @@ void launch_jac(const Mesh& m, Args A, const int32_t* slot, double* K, double* D
     if (no > 0) jac_out<T, MODE><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, slot, K, D);
     if (nc > 0) {
         const void* pts = sizeof(T) == 4 ? (const void*)m.d.cut_pts_f : (const void*)m.d.cut_pts;
-        jac_cut<T, MODE><<<(unsigned)((nc + JWPB - 1) / JWPB), 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order, nc,
+        jac_cut<T, MODE><<<(unsigned)nc, 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order,
                                                                                slot, K, D);
     }
     if (ns > 0)
@@ -1043,7 +1050,7 @@ void launch_bsr_assembly(const Mesh& m, Args A, double* val, double* Ks, cudaStr
     if (no > 0) jac_out<T, BSR><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, nullptr, val, nullptr);
     if (nc > 0) {
         const void* pts = sizeof(T) == 4 ? (const void*)m.d.cut_pts_f : (const void*)m.d.cut_pts;
-        jac_cut<T, BSR><<<(unsigned)((nc + JWPB - 1) / JWPB), 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order, nc,
+        jac_cut<T, BSR><<<(unsigned)nc, 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order,
                                                                               nullptr, val, nullptr);
     }
     if (ns > 0 && nh > 0) {
