@@ -44,8 +44,8 @@ constexpr int kMaxLevels = 24;
 // loaded before the first sum.  Every block's four products are summed by its lane and the blocks' sums
 // added in column order by every lane: the order, and the bits, of a thread that walks the row.  Q = 8 (a
 // warp per row) shortens the chain where the rows of a level leave the chip idle; from kManyRows on Q = 2,
-// which needs a third of the instructions per block.  V-cycle on 74 k nodes, mixed: 349 -> 181 us (186 with
-// Q = 1 there, 200 with Q = 4).
+// which needs a third of the instructions per block.  V-cycle on 74 k nodes, mixed: 349 -> 161 us (5 us more
+// with Q = 1 there, 19 with Q = 4, 9 with twice the steps in flight for Q = 2).
 constexpr int kRowAhead = 4;
 constexpr int64_t kManyRows = 32768;
 
@@ -101,25 +101,27 @@ template <class T> struct Corrected {
 template <int Q, class T, class X>
 __device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                          const T* __restrict__ val, const X& x) {
-    constexpr int D = kRowAhead * (Q == 8 ? 1 : 2);   // steps in flight
+    constexpr int D = kRowAhead;   // steps in flight
     const int lane = threadIdx.x & 31, j = (lane >> 2) & (Q - 1), i = lane & 3, first = lane & ~(4 * Q - 1);
     const int64_t q0 = live ? ptr[row] : 0, q1 = live ? ptr[row + 1] : 0;
     T acc = T(0);
     for (int64_t base = q0; __any_sync(0xffffffffu, base < q1); base += Q * D) {
         T t[D];
         int32_t c[D];
+        Row4<T> a[D];
 #pragma unroll
         for (int g = 0; g < D; ++g) {
             const int64_t q = base + Q * g + j;
-            c[g] = q < q1 ? __ldg(idx + q) : -1;
+            c[g] = -1;
+            if (q < q1) {   // (the block does not wait for its column)
+                c[g] = __ldg(idx + q);
+                a[g] = load_row(val + 16 * q + 4 * i);
+            }
         }
 #pragma unroll
         for (int g = 0; g < D; ++g) {
             t[g] = T(0);
-            if (c[g] >= 0) {
-                const Row4<T> a = load_row(val + 16 * (base + Q * g + j) + 4 * i), b = x(c[g]);
-                t[g] = dot4(a.v, b.v);
-            }
+            if (c[g] >= 0) t[g] = dot4(a[g].v, x(c[g]).v);
         }
 #pragma unroll
         for (int g = 0; g < D; ++g)
