@@ -197,25 +197,29 @@ __global__ void __launch_bounds__(256) dg_mdot(GState* G, int64_t n, const doubl
         partial[(int64_t)(k0 + threadIdx.x) * kRedBlocks + blockIdx.x] = v;
     }
     if (!last_block(&G->cnt, gridDim.x * (unsigned)((nk + kDotGroup - 1) / kDotGroup))) return;
-    // per column: a thread's blocks, the warp, then the warps in order (eight columns at a time)
-    double* out = second ? G->h2 : G->h;
-    for (int g = 0; g < nk; g += 8) {
-        double v[8], s8 = 0.0;
+    // per column: the blocks b, b + 256, ... of a lane, the 32 lanes of a segment of blocks, then the segments
+    // in order; a warp takes (eight columns, segment) pairs, their loads not waiting for one another
+    __shared__ double seg[64][9];
+    const int ns = min(8, ((int)gridDim.x + 31) / 32), groups = (nk + 7) / 8;
+#pragma unroll 2
+    for (int t = wid; t < groups * ns; t += 8) {
+        const int g = t / ns, sg = t % ns;
+        double v[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             v[c] = 0.0;
-            if (g + c < nk)
-                for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) v[c] += __ldcg(partial + (int64_t)(g + c) * kRedBlocks + b);
+            if (8 * g + c < nk)
+                for (int b = 32 * sg + lane; b < (int)gridDim.x; b += 256) v[c] += __ldcg(partial + (int64_t)(8 * g + c) * kRedBlocks + b);
         }
-        if (32 * wid < (int)gridDim.x) s8 = warp_sum8(v);
-        __syncthreads();
-        if ((lane & 3) == 0) red[((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)][wid] = s8;
-        __syncthreads();
-        if (threadIdx.x < 8 && g + (int)threadIdx.x < nk) {
-            double t = 0.0;
-            for (int q = 0; q < 8; ++q) t += red[threadIdx.x][q];
-            out[g + threadIdx.x] = t;
-        }
+        const double x = warp_sum8(v);
+        if ((lane & 3) == 0) seg[8 * g + ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)][sg] = x;
+    }
+    __syncthreads();
+    double* out = second ? G->h2 : G->h;
+    if ((int)threadIdx.x < nk) {
+        double t = 0.0;
+        for (int q = 0; q < ns; ++q) t += seg[threadIdx.x][q];
+        out[threadIdx.x] = t;
     }
 }
 
@@ -735,7 +739,7 @@ public:
 
     // precondition V[k] (vec(4) holds it), J v, CGS2 against V[0..k], Givens update, normalise into V[k+1]:
     // five launches beside the preconditioner and J v (11 before).  A Newton solve of the 7.3 k
-    // element sphere to 1e-8, all steps of this file's history together: 84 -> 53 ms
+    // element sphere to 1e-8, with the assembly, the V-cycle and the kernels of J v: 70 -> 35 ms
     int step_launches(const double* u) {
         GState* G = W.G;
         double* vk = vec(4);
