@@ -1112,11 +1112,13 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
 // loads per entry (code, then a 16-byte row), so what counts is loads in flight: the rows of 8 entries go
 // by cp.async to the thread's own places in shared memory, which takes no registers (1,280 nodes in flight
 // per SM instead of 768).  Lists are padded to whole batches of 8 codes, two 16-byte loads.  Most nodes
-// have one batch; the others (parents of hanging nodes) would hold up their warp, so they are taken
-// apart, ordered by length, in blocks of their own that start first.  Writes every row of out: no zeroing
+// have one batch; the others (parents of hanging nodes, nodes at a surface: up to a hundred entries)
+// would hold up their warp, so they are taken apart, longest first, in blocks of their own that start
+// first; where they are few, by four lanes per node with 32 entries in flight.  Writes every row of out: no zeroing
 // before the call.  2.0 M elements, mixed: 137 -> 103 us (376 MB, 3.7 TB/s); 12
 // spheres: 81 -> 50 us.
 constexpr int kGatherThreads = 128;
+constexpr int kQuadLists = 256;   // per SM
 
 // component k of node n after its strong rows
 struct StrongRows {
@@ -1139,14 +1141,71 @@ struct StrongRows {
     }
 };
 
-template <class T>
+template <class T, bool QUADS>
 __global__ void __launch_bounds__(kGatherThreads, sizeof(T) == 4 ? 10 : 6) node_gather(
     Args A, const uint32_t* __restrict__ head, const int32_t* __restrict__ heavy, const int64_t* __restrict__ hptr,
     const uint32_t* __restrict__ inc, int64_t n_heavy, unsigned heavy_blocks, int64_t nv, StrongRows S) {
     static_assert(kIncHead == 8, "batches of two 16-byte loads");
     constexpr int C = sizeof(T) / 4;   // 16-byte chunks of a row
     __shared__ __align__(16) uint4 s_row[8][C][kGatherThreads];
+    __shared__ uint32_t s_code[QUADS ? 8 : 1][kGatherThreads];
     if (A.skip && *A.skip) return;   // a captured solver step after its cycle ended
+    if (QUADS && blockIdx.x < heavy_blocks) {
+        // four lanes per node: each fetches the rows of 8 of the next 32 entries, then sums one component of
+        // all 32 in order
+        const int64_t h = ((int64_t)blockIdx.x * kGatherThreads + threadIdx.x) >> 2;
+        const int k = threadIdx.x & 3, quad = threadIdx.x & ~3;
+        const bool live = h < n_heavy;
+        const int64_t q1 = live ? hptr[h + 1] : 0;
+        int64_t q = live ? hptr[h] : 0;
+        double acc = 0.0;
+        float hi = 0.f, lo = 0.f;
+        for (; __any_sync(0xffffffffu, q < q1); q += 32) {
+            const int64_t mine = q + 8 * k;
+            uint4 c[2] = {{kIncNone, kIncNone, kIncNone, kIncNone}, {kIncNone, kIncNone, kIncNone, kIncNone}};
+            if (mine < q1) {
+                c[0] = __ldg(reinterpret_cast<const uint4*>(inc + mine));
+                c[1] = __ldg(reinterpret_cast<const uint4*>(inc + mine) + 1);
+            }
+            const uint32_t e[8] = {c[0].x, c[0].y, c[0].z, c[0].w, c[1].x, c[1].y, c[1].z, c[1].w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int64_t sl = (int64_t)(e[i] >> 5);
+                s_code[QUADS ? i : 0][threadIdx.x] = e[i];
+                if (sl < nv) {   // (a padding code's slot is past every volume slot)
+                    const char* r = (const char*)A.sv + (32 * sl + 4 * (e[i] & 7)) * sizeof(T);
+#pragma unroll
+                    for (int b = 0; b < C; ++b) cp16(&s_row[i][b][threadIdx.x], r + 16 * b);
+                }
+            }
+            cp_commit();
+            cp_wait<0>();
+            __syncwarp();
+            for (int f = 0; f < 4 && q + 8 * f < q1; ++f)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t code = s_code[QUADS ? i : 0][quad + f];
+                    if (code == kIncNone) continue;
+                    const int wc = (int)((code >> 3) & 3);
+                    const int64_t sl = (int64_t)(code >> 5);
+                    if (sl < nv) {
+                        const T w = wc == 0 ? T(1) : (wc == 1 ? T(0.5) : T(0.25));
+                        const T v = reinterpret_cast<const T*>(&s_row[i][k * sizeof(T) / 16][quad + f])[k & (16 / sizeof(T) - 1)];
+                        if constexpr (sizeof(T) == 4) ff_add(hi, lo, w * v);
+                        else acc += w * v;
+                    } else {   // a float64 surface slot
+                        const double w = wc == 0 ? 1.0 : (wc == 1 ? 0.5 : 0.25);
+                        acc += w * A.ss[32 * (sl - nv) + 4 * (code & 7) + k];
+                    }
+                }
+            __syncwarp();   // the rows and codes are replaced
+        }
+        if (!live) return;
+        const int64_t n = heavy[h];
+        if constexpr (sizeof(T) == 4) acc += f2d(hi) + f2d(lo);
+        A.out[4 * n + k] = (S.mask(n) >> k) & 1 ? S.row(A, n, k) : acc;
+        return;
+    }
     int64_t n;
     const uint4* code;
     int batches = 1;
@@ -1502,12 +1561,16 @@ void launch_strong_rows(const Mesh& m, const Args& A, const imga_physics& ph, bo
         const uint8_t* um = m.user_bc ? m.d.bcmask_user : nullptr;
         const double* uv = m.user_bc ? m.d.bcval_user : nullptr;
         const StrongRows S = {m.d.bcflag, um, uv, ph.u_inf[0], ph.u_inf[1], ph.u_inf[2], jv ? 1 : 0};
-        const unsigned hb = (unsigned)((m.n_heavy + kGatherThreads - 1) / kGatherThreads),
+        // long lists by four lanes per node where that still leaves the chip idle, by a thread per node else
+        // (4 k lists: 17 us against 26; 350 k lists: 58 against 50)
+        const bool quads = m.n_heavy <= (int64_t)kQuadLists * m.n_sm;
+        const unsigned hb = (unsigned)(((quads ? 4 : 1) * m.n_heavy + kGatherThreads - 1) / kGatherThreads),
                        grid = hb + (unsigned)((nn + kGatherThreads - 1) / kGatherThreads);
-        if (precision == 0)
-            node_gather<double><<<grid, kGatherThreads, 0, s>>>(A, m.d.inc_head, m.d.inc_heavy, m.d.inc_ptr, m.d.inc, m.n_heavy, hb, m.n_vslots, S);
-        else
-            node_gather<float><<<grid, kGatherThreads, 0, s>>>(A, m.d.inc_head, m.d.inc_heavy, m.d.inc_ptr, m.d.inc, m.n_heavy, hb, m.n_vslots, S);
+        auto run = [&](auto kernel) {
+            kernel<<<grid, kGatherThreads, 0, s>>>(A, m.d.inc_head, m.d.inc_heavy, m.d.inc_ptr, m.d.inc, m.n_heavy, hb, m.n_vslots, S);
+        };
+        if (precision == 0) { if (quads) run(node_gather<double, true>); else run(node_gather<double, false>); }
+        else { if (quads) run(node_gather<float, true>); else run(node_gather<float, false>); }
         return;
     }
     if (nn > 0)
