@@ -453,6 +453,91 @@ __device__ __forceinline__ void cut_element(const Args& A, const int32_t* __rest
     warp_scatter_moments<T>(A, M, s_m, lane, my_id, 0.0, A.sv ? (T*)A.sv + 32 * (A.n_out_slots + idx) : nullptr);
 }
 
+// The same element, with the same sums, on a block of four warps: each warp evaluates every fourth round of
+// 32 points and leaves the coefficients in shared memory, then takes one component's moments of all four
+// rounds in order (lane l: points l, l + 32, ...).  Where there are few elements, the longest of them (a
+// thousand points and more on one warp) is the kernel's time: 7.3 k element sphere, 776 elements, mixed J v
+// 23 -> 15 us; float64 (the generic code of mixed solves, bound by the FP64 pipe of the SMs that got the long
+// elements) R 480 -> 241, J v 746 -> 368 us.  With many elements the two barriers per 128 points cost more
+// than they give: float32 meshes of more than kSplitCut elements per SM keep a warp per element.
+constexpr int kSplitCut = 16;
+template <class T, bool JV>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) vms_cut_split(Args A, const int32_t* __restrict__ list,
+                                                                            const int64_t* __restrict__ off,
+                                                                            const void* __restrict__ pts,
+                                                                            const int32_t* __restrict__ order) {
+    typedef typename std::conditional<JV, Dual<T>, T>::type S;
+    constexpr int MSTR = 32 + 16 / (int)sizeof(T);
+    __shared__ __align__(16) T s_nd[8 * CS];
+    __shared__ __align__(16) T s_m[32 * MSTR];
+    __shared__ T s_w[4][16][33], s_x[4][3][33];
+    if (A.skip && *A.skip) return;   // a captured solver step after its cycle ended
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t idx = order ? (int64_t)order[blockIdx.x] : blockIdx.x;
+    const int32_t e = list[idx];
+    const int c8 = lane & 7;
+    const int32_t my_id = A.conn[8 * (int64_t)e + c8];
+    if (w == 0) {
+        T rw[CS];
+        corner_data<T, JV>(A, my_id, rw);
+        for (int j = 0; j < 7; ++j) rw[j] = hadamard_fwd(rw[j], c8);
+        if (JV)
+            for (int j = 0; j < 7; ++j) rw[CT + j] = hadamard_fwd(rw[CT + j], c8);
+        if (A.ndf)
+            for (int j = 0; j < 3; ++j) rw[CF + j] = hadamard_fwd(rw[CF + j], c8);
+        if (lane < 8)
+            for (int j = 0; j < CS; ++j) s_nd[lane * CS + j] = rw[j];
+    }
+    __syncthreads();
+    const T g = lvl_g<T>(A, A.lev[e]);
+    const T det = lvl_w<T>(A, A.lev[e]);
+    const Phys<T> P(A, prob_of(A, e));
+    T M[8];   // component w
+    for (int k = 0; k < 8; ++k) M[k] = T(0);
+    const int64_t q0 = off[idx], q1 = off[idx + 1];
+    for (int64_t base = q0; base < q1; base += 128) {
+        const int64_t q = base + 32 * w + lane;
+        if (q < q1) {
+            T pt[4];
+            load_pt<T>(pts, q, pt);
+            T m[8];
+            monomials<T>(pt, m);
+            S cf[16];
+            vms_point_modal<S, T>(A, P, m, s_nd, CS, g, cf);
+            const T wq = pt[3] * det, wqg = wq * g;
+            for (int k = 0; k < 16; ++k) s_w[w][k][lane] = ((k < 3 || k == 12) ? wq : wqg) * Pick<T, JV>::get(cf[k]);
+            for (int k = 0; k < 3; ++k) s_x[w][k][lane] = pt[k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (base + 32 * r + lane < q1) {
+                const T xi[3] = {s_x[r][0][lane], s_x[r][1][lane], s_x[r][2][lane]};
+                T m[8];
+                monomials<T>(xi, m);
+                const T f = s_w[r][w < 3 ? w : 12][lane], sx = s_w[r][w < 3 ? 3 + 3 * w : 13][lane],
+                        sy = s_w[r][w < 3 ? 4 + 3 * w : 14][lane], sz = s_w[r][w < 3 ? 5 + 3 * w : 15][lane];
+                auto add = [&](int Sx, T s, T x) { M[Sx] = fma(s, x, M[Sx]); };   // as add_moments
+                add(0, m[0], f);
+                add(1, m[1], f); add(1, m[0], sx);
+                add(2, m[2], f); add(2, m[0], sy);
+                add(3, m[3], f); add(3, m[2], sx); add(3, m[1], sy);
+                add(4, m[4], f); add(4, m[0], sz);
+                add(5, m[5], f); add(5, m[4], sx); add(5, m[1], sz);
+                add(6, m[6], f); add(6, m[4], sy); add(6, m[2], sz);
+                add(7, m[7], f); add(7, m[6], sx); add(7, m[5], sy); add(7, m[3], sz);
+            }
+        __syncthreads();
+    }
+    for (int k = 0; k < 8; ++k) s_m[lane * MSTR + 4 * k + w] = M[k];
+    __syncthreads();
+    if (w > 0) return;
+    T row[32];
+    for (int k = 0; k < 32; k += 4) ld4s<T>(&s_m[lane * MSTR + k], row + k);
+    __syncwarp();
+    warp_scatter_moments<T>(A, row, s_m, lane, my_id, 0.0, A.sv ? (T*)A.sv + 32 * (A.n_out_slots + idx) : nullptr);
+}
+
 // ------------------------------------------------------------------------------------------
 // Intercepted elements in float64 (see Const64: FP64 instructions are the cost).  Per point the fields
 // come from the Hadamard coefficients by Horner steps along x, y, z, whose intermediates are the
@@ -616,7 +701,7 @@ __device__ __forceinline__ void cut_element64(const Args& A, const int32_t* __re
 
 // W warps per block (a tile shape the autotuner picks); `order` (or null) permutes the list
 template <class T, bool JV, int W>
-__global__ void __launch_bounds__(32 * W, (sizeof(T) == 4 ? 16 : 8) / W) vms_cut(Args A, const int32_t* __restrict__ list,
+__global__ void __launch_bounds__(32 * W, 16 / W) vms_cut(Args A, const int32_t* __restrict__ list,
                                                     const int64_t* __restrict__ off, const void* __restrict__ pts,
                                                     const int32_t* __restrict__ order, int64_t n) {
     constexpr int PAD = 16 / (int)sizeof(T), MSTR = 32 + PAD;
@@ -1312,11 +1397,15 @@ void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt, 
     const int64_t nc = (int64_t)m.cut_list.size();
     const int32_t* order = lpt ? m.d.cut_order : nullptr;
     if constexpr (sizeof(T) == 8) {
-        if (generic) vms_cut<T, JV, 4><<<(unsigned)((nc + 3) / 4), 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order, nc);
+        if (generic) vms_cut_split<T, JV><<<(unsigned)nc, 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
         else if (wpb == 2) vms_cut64<JV, 2><<<(unsigned)nc, 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
         else vms_cut64<JV, 4><<<(unsigned)nc, 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
     } else {
         const void* pts = m.d.cut_pts_f;
+        if (nc <= (int64_t)kSplitCut * m.n_sm) {
+            vms_cut_split<T, JV><<<(unsigned)nc, 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order);
+            return;
+        }
         switch (wpb) {
             case 2: vms_cut<T, JV, 2><<<(unsigned)((nc + 1) / 2), 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
             case 8: vms_cut<T, JV, 8><<<(unsigned)((nc + 7) / 8), 256, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
