@@ -131,7 +131,10 @@ __device__ __forceinline__ void ldm4t(uint32_t r[4], const bf16* p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(saddr(p)) : "memory");
 }
-__device__ __forceinline__ uint32_t cvt2(float lo, float hi) { return pack2(__float2bfloat16(lo), __float2bfloat16(hi)); }
+__device__ __forceinline__ uint32_t cvt2(float lo, float hi) {   // one conversion instruction for the pair
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
 
 struct MlpTrainIO {           // what a training step keeps of the forward pass
     const float* T;           // targets [n][nout]
@@ -167,24 +170,33 @@ __global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad,
     auto xs = [&](int s) { return reinterpret_cast<float*>(sm + s * (Sh::XS + Sh::WS)); };
     auto ws = [&](int s) { return reinterpret_cast<bf16*>(sm + s * (Sh::XS + Sh::WS) + Sh::XS); };
     const int nkt = (nin_pad + kKT - 1) / kKT;
+    // a thread copies the same columns of every stage: its rows' addresses are formed once (they were more than
+    // half of the kernel's instructions)
+    constexpr int XC = KT / 4, XR = NT / XC, XN = BM / XR, WC = KT / 8, WR = NT / WC, WN_ = kW / WR;
+    static_assert(BM % XR == 0 && kW % WR == 0, "whole rows per pass");
+    const int xc = tid % XC * 4, xr = tid / XC, wc = tid % WC * 8, wr = tid / WC;
+    const float* xsrc[XN];
+#pragma unroll
+    for (int i = 0; i < XN; ++i) xsrc[i] = m0 + xr + XR * i < n ? X + (m0 + xr + XR * i) * ldx + xc : nullptr;
+    const bf16* wsrc = W1 + (int64_t)wr * nin_pad + wc;
     auto load = [&](int kt) {
         if (kt < nkt) {
-            float* x = xs(kt % STAGES);
-            bf16* w = ws(kt % STAGES);
-            for (int i = tid; i < BM * (kKT / 4); i += NT) {
-                const int r = i / (kKT / 4), c = i % (kKT / 4) * 4, gc = kt * kKT + c;
-                const int64_t gr = m0 + r;
-                const int left = gr < n ? max(0, min(4, nin - gc)) : 0;
-                const float* src = left ? X + gr * ldx + gc : X;
-                if (xvec) cpz16(x + r * kKS + c, src, 4 * left);
+            float* x = xs(kt % STAGES) + xr * kKS + xc;
+            bf16* w = ws(kt % STAGES) + wr * kKS + wc;
+            const int k0 = kt * kKT, left = max(0, min(4, nin - k0 - xc));
+#pragma unroll
+            for (int i = 0; i < XN; ++i) {
+                const int here = xsrc[i] ? left : 0;
+                const float* src = here ? xsrc[i] + k0 : X;
+                if (xvec) cpz16(x + XR * i * kKS, src, 4 * here);
                 else
-                    for (int j = 0; j < 4; ++j) cpz4(x + r * kKS + c + j, j < left ? src + j : X, j < left ? 4 : 0);
+                    for (int j = 0; j < 4; ++j) cpz4(x + XR * i * kKS + j, j < here ? src + j : X, j < here ? 4 : 0);
             }
-            for (int i = tid; i < kW * (kKT / 8); i += NT) {
-                const int r = i / (kKT / 8), c = i % (kKT / 8) * 8, gc = kt * kKT + c;
-                const bool in = gc < nin_pad;
-                cpz16(w + r * kKS + c, in ? W1 + (int64_t)r * nin_pad + gc : W1, in ? 16 : 0);
-            }
+            const bool in = k0 + wc < nin_pad;
+            const bf16* src = in ? wsrc + k0 : W1;
+            const int64_t step = in ? (int64_t)WR * nin_pad : 0;
+#pragma unroll
+            for (int i = 0; i < WN_; ++i) cpz16(w + WR * i * kKS, src + i * step, in ? 16 : 0);
         }
         cp_commit();
     };
@@ -242,10 +254,15 @@ __global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad,
             const bf16* W = l2 ? W2 : W3;
             const int n0 = (l2 ? k : k - kW / kNC) * kNC, nr = l2 ? kW : nout;
             bf16* w = chunk_buf(k);
-            for (int i = tid; i < kNC * (kW / 8); i += NT) {
-                const int r = i / (kW / 8), c = i % (kW / 8) * 8;
-                const bool in = n0 + r < nr;
-                cpz16(w + r * kHS + c, in ? W + (int64_t)(n0 + r) * kW + c : W, in ? 16 : 0);
+            constexpr int R = NT / (kW / 8);
+            static_assert(kNC % R == 0, "whole rows per pass");
+            const int r0 = tid / (kW / 8), c = tid % (kW / 8) * 8;
+            const bf16* src = W + (int64_t)(n0 + r0) * kW + c;
+            bf16* dst = w + r0 * kHS + c;
+#pragma unroll
+            for (int i = 0; i < kNC / R; ++i) {
+                const bool in = n0 + r0 + R * i < nr;
+                cpz16(dst + R * i * kHS, in ? src + R * i * kW : W, in ? 16 : 0);
             }
         }
         cp_commit();
@@ -373,8 +390,8 @@ __global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad,
 // Gradient products of one layer in one launch, 32 x 32 of the result per CTA, K whole (the sums keep
 // the order of gemm_bf16), 64 of K per stage, four stages in flight.  Bound by the latency of the K chain
 // (64 dependent products for 1024 rows), so the tiles are small: more CTAs, not more work per CTA.
-//   dw CTAs: G [M][N] = alpha D^T H  (D [K][M], H [K][N] rows of the batch), and the column sums of D
-//            (the bias gradient, rows in order) from the tiles of the CTAs with n0 = 0;
+//   dw CTAs: G [M][N] = alpha D^T H  (D [K][M], H [K][N] rows of the batch);
+//   db CTAs: the column sums of D (the bias gradient), rows in order, 32 columns each;
 //   dh CTAs: Z [K][N] = (D W) masked by H > 0, in bf16 (W [M][N] the layer's weights, H its input).
 constexpr int kBT = 32, kBK = 64, kBStages = 4;
 struct BackArgs {
@@ -394,8 +411,10 @@ __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
     static_assert(kBT * DS <= AS, "stage size");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
     const int wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
-    const bool dw = (int)blockIdx.x < P.dw_tiles;
-    const int t = dw ? blockIdx.x : blockIdx.x - P.dw_tiles;
+    // the db CTAs come first (their serial sums are the longest chain), then dw, then dh
+    const int b0 = (int)blockIdx.x - (P.M + kBT - 1) / kBT;
+    const bool db = b0 < 0, dw = b0 < P.dw_tiles;
+    const int t = db ? (int)blockIdx.x * P.dw_n : dw ? b0 : b0 - P.dw_tiles;
     const int nb = dw ? P.dw_n : (P.N + kBT - 1) / kBT;
     const int64_t m0 = (int64_t)(t / nb) * kBT;
     const int n0 = (t % nb) * kBT;
@@ -410,7 +429,7 @@ __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
             for (int i = tid; i < kBK * kBT / 8; i += 128) {
                 const int kr = i / (kBT / 8), c = i % (kBT / 8) * 8;
                 const bool inb = k0 + kr < K && n0 + c < P.N;
-                cpz16(b + kr * TS + c, inb ? B + (k0 + kr) * P.N + n0 + c : B, inb ? 16 : 0);
+                if (!db) cpz16(b + kr * TS + c, inb ? B + (k0 + kr) * P.N + n0 + c : B, inb ? 16 : 0);
                 if (dw) {
                     const bool ina = k0 + kr < K && m0 + c < P.M;
                     cpz16(a + kr * TS + c, ina ? P.D + (k0 + kr) * P.M + m0 + c : P.D, ina ? 16 : 0);
@@ -425,7 +444,6 @@ __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
     };
     for (int s = 0; s < kBStages - 1; ++s) load(s);
     float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-    const bool sums = dw && n0 == 0 && warp == 0;
     float s = 0.f;
     // transposed 8 x 8 blocks: A as (m, k), (m + 8, k), (m, k + 8), (m + 8, k + 8); B as (n, k), (n, k + 8), ...
     const int akr = (lane & 7) + ((lane >> 4) << 3), amc = ((lane >> 3) & 1) * 8;
@@ -436,6 +454,14 @@ __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
         __syncthreads();
         load(kt + kBStages - 1);
         const bf16 *a = sA[kt % kBStages], *b = sB[kt % kBStages];
+        if (db) {
+            const int kr1 = (int)min((int64_t)kBK, K - (int64_t)kt * kBK);
+            if (warp == 0) {
+#pragma unroll 16
+                for (int kr = 0; kr < kr1; ++kr) s += __bfloat162float(a[kr * TS + lane]);
+            }
+            continue;
+        }
 #pragma unroll
         for (int ks = 0; ks < kBK; ks += 16) {
             uint32_t af[4], bf[4];
@@ -445,13 +471,12 @@ __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
             mma16816(acc[0], af, bf);
             mma16816(acc[1], af, bf + 2);
         }
-        if (sums) {
-            const int kr1 = (int)min((int64_t)kBK, K - (int64_t)kt * kBK);
-#pragma unroll 16
-            for (int kr = 0; kr < kr1; ++kr) s += __bfloat162float(a[kr * TS + lane]);
-        }
     }
     cp_wait<0>();
+    if (db) {
+        if (warp == 0 && m0 + lane < P.M) P.db[m0 + lane] = P.beta != 0.f ? P.db[m0 + lane] + s : s;
+        return;
+    }
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -470,7 +495,6 @@ __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
                 *reinterpret_cast<uint32_t*>(P.Z + r * P.N + c) = cvt2(h0 > 0.f ? acc[j][q] : 0.f, h1 > 0.f ? acc[j][q + 1] : 0.f);
             }
         }
-    if (sums && m0 + lane < P.M) P.db[m0 + lane] = P.beta != 0.f ? P.db[m0 + lane] + s : s;
 }
 
 __global__ void to_bf16(int64_t n, const float* __restrict__ x, bf16* __restrict__ y) {
@@ -754,7 +778,7 @@ static void mlp_step_fused(Mlp& M, const float* X, int64_t ldx, const float* T, 
         P.dw_n = (nn + kBT - 1) / kBT;
         P.dw_tiles = P.dw_n * ((m + kBT - 1) / kBT);
         const int64_t dh = Z ? P.dw_n * ((b + kBT - 1) / kBT) : 0;
-        mlp_back<<<(unsigned)(P.dw_tiles + dh), 128, 0, s>>>(P);
+        mlp_back<<<(unsigned)((m + kBT - 1) / kBT + P.dw_tiles + dh), 128, 0, s>>>(P);
     };
     back(M.nout, M.w, M.dyb, M.h2, 4, M.dz2);
     back(M.w, M.w, M.dz2, M.h1, 2, M.dz1);
