@@ -44,8 +44,8 @@ constexpr int kMaxLevels = 24;
 // loaded before the first sum.  Every block's four products are summed by its lane and the blocks' sums
 // added in column order by every lane: the order, and the bits, of a thread that walks the row.  Q = 8 (a
 // warp per row) shortens the chain where the rows of a level leave the chip idle; from kManyRows on Q = 2,
-// which needs a third of the instructions per block.  V-cycle on 74 k nodes, mixed: 349 -> 161 us (5 us more
-// with Q = 1 there, 19 with Q = 4, 9 with twice the steps in flight for Q = 2).
+// which needs a third of the instructions per block.  V-cycle on 74 k nodes, mixed: 349 -> 161 us (137 with
+// overlapping launches, see apply(); 5 us more with Q = 1 there, 19 with Q = 4, 9 with twice the steps in flight for Q = 2).
 constexpr int kRowAhead = 4;
 constexpr int64_t kManyRows = 32768;
 
@@ -97,14 +97,15 @@ template <class T> struct Corrected {
 };
 
 // component (lane & 3) of row `row` of A x, on the row's 4 Q lanes (live: this row exists; every lane of the
-// warp calls)
-template <int Q, class T, class X>
+// warp calls).  begin() runs once, before x is first read: the matrix is loaded ahead of it.
+template <int Q, class T, class X, class B>
 __device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
-                                         const T* __restrict__ val, const X& x) {
+                                         const T* __restrict__ val, const X& x, B&& begin) {
     constexpr int D = kRowAhead;   // steps in flight
     const int lane = threadIdx.x & 31, j = (lane >> 2) & (Q - 1), i = lane & 3, first = lane & ~(4 * Q - 1);
     const int64_t q0 = live ? ptr[row] : 0, q1 = live ? ptr[row + 1] : 0;
     T acc = T(0);
+    bool begun = false;
     for (int64_t base = q0; __any_sync(0xffffffffu, base < q1); base += Q * D) {
         T t[D];
         int32_t c[D];
@@ -118,6 +119,8 @@ __device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* 
                 a[g] = load_row(val + 16 * q + 4 * i);
             }
         }
+        if (!begun) begin();
+        begun = true;
 #pragma unroll
         for (int g = 0; g < D; ++g) {
             t[g] = T(0);
@@ -131,6 +134,7 @@ __device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* 
                 if (base + Q * g + b < q1) acc += s;
             }
     }
+    if (!begun) begin();
     return acc;
 }
 
@@ -140,7 +144,7 @@ __global__ void __launch_bounds__(256) bsr_mul(int64_t n, const int64_t* __restr
                                                const T* __restrict__ val, const T* __restrict__ x, T* __restrict__ y) {
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (4 * Q);
     const int l = threadIdx.x & (4 * Q - 1);
-    const T acc = row_product<Q, T>(row < n, row, ptr, idx, val, Plain<T>{x});
+    const T acc = row_product<Q, T>(row < n, row, ptr, idx, val, Plain<T>{x}, [] {});
     if (row < n && l < 4) y[4 * row + l] = acc;
 }
 
@@ -148,15 +152,22 @@ __global__ void __launch_bounds__(256) bsr_mul(int64_t n, const int64_t* __restr
 // where X is Corrected; z (or null): y once more, in float64.
 template <class T, class X, int Q>
 __global__ void __launch_bounds__(256) ml_sweep(int64_t n, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
-                                                const T* __restrict__ val, X x, const T* __restrict__ b,
-                                                const T* __restrict__ Dinv, T omega, T* __restrict__ y, double* __restrict__ z) {
+                                                const T* __restrict__ val, X x, const T* b,
+                                                const T* __restrict__ Dinv, T omega, T* y, double* z) {
+    next_may_start();
     const int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (4 * Q);
     const bool live = r0 < n;
     const int64_t row = live ? r0 : n - 1;
     const int l = threadIdx.x & (4 * Q - 1), i = l & 3;
-    const Row4<T> D = load_row(Dinv + 16 * row + 4 * i), xr = x(row);
-    const T bi = b[4 * row + i];
-    const T res = bi - row_product<Q, T>(live, row, ptr, idx, val, x);
+    const Row4<T> D = load_row(Dinv + 16 * row + 4 * i);
+    Row4<T> xr;
+    T bi;
+    const T prod = row_product<Q, T>(live, row, ptr, idx, val, x, [&] {
+        after_previous();
+        xr = x(row);
+        bi = b[4 * row + i];
+    });
+    const T res = bi - prod;
     T v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xffffffffu, res, (threadIdx.x & 28) | k);
@@ -175,9 +186,9 @@ __global__ void __launch_bounds__(256) ml_sweep(int64_t n, const int64_t* __rest
 template <class T, int Q>
 __global__ void __launch_bounds__(256) ml_restrict(int64_t nc, int64_t nf, int agg, int per, const int64_t* __restrict__ ptr,
                                                    const int32_t* __restrict__ idx, const T* __restrict__ val,
-                                                   const T* __restrict__ x, const T* __restrict__ b,
-                                                   const uint8_t* __restrict__ fr, const T* __restrict__ Dinv_c, T omega,
-                                                   T* __restrict__ rc, T* __restrict__ xc) {
+                                                   const T* x, const T* b, const uint8_t* __restrict__ fr,
+                                                   const T* __restrict__ Dinv_c, T omega, T* rc, T* xc) {
+    next_may_start();
     constexpr int R = 64 / Q;   // rows at a time
     __shared__ T s_res[R][4];
     const int r = threadIdx.x / (4 * Q), i = threadIdx.x & 3;
@@ -188,8 +199,12 @@ __global__ void __launch_bounds__(256) ml_restrict(int64_t nc, int64_t nf, int a
     for (int64_t a0 = i0; a0 < i1; a0 += R) {
         const int64_t row = a0 + r;
         const bool live = row < i1;
-        const T bi = live ? b[4 * row + i] : T(0);
-        const T res = bi - row_product<Q, T>(live, row, ptr, idx, val, Plain<T>{x});
+        T bi = T(0);
+        const T prod = row_product<Q, T>(live, row, ptr, idx, val, Plain<T>{x}, [&] {
+            after_previous();
+            if (live) bi = b[4 * row + i];
+        });
+        const T res = bi - prod;
         if (live && (threadIdx.x & (4 * Q - 1)) < 4) s_res[r][i] = res;
         __syncthreads();
         if (I < I1)
@@ -197,6 +212,7 @@ __global__ void __launch_bounds__(256) ml_restrict(int64_t nc, int64_t nf, int a
                 if ((fr[q] >> i) & 1) s += s_res[q - a0][i];
         __syncthreads();
     }
+    after_previous();   // (a block without rows waits too)
     if (I >= I1) return;
     rc[4 * I + i] = s;
     if (!Dinv_c) return;
@@ -210,8 +226,9 @@ __global__ void __launch_bounds__(256) ml_restrict(int64_t nc, int64_t nf, int a
 // x[i][k] += F_i xc[I(i)][k]: on a level of many rows a pass of its own (the corrected entry at every block,
 // with its division by the aggregate size, costs a sweep of 74 k rows 11 us, this pass 3)
 template <class T>
-__global__ void __launch_bounds__(256) ml_prolong(int64_t nf, uint32_t agg, const uint8_t* __restrict__ fr, const T* __restrict__ xc,
-                                                  T* __restrict__ x) {
+__global__ void __launch_bounds__(256) ml_prolong(int64_t nf, uint32_t agg, const uint8_t* __restrict__ fr, const T* xc, T* x) {
+    next_may_start();
+    after_previous();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = t >> 2;
     if (i >= nf) return;
@@ -417,8 +434,9 @@ __global__ void __launch_bounds__(512) ml_dense_inverse(int N, const double* __r
 
 // r in the cycle's precision and the first sweep from x = 0: x = omega Dinv r
 template <class T>
-__global__ void ml_start(int64_t n, const T* __restrict__ Dinv, T omega, const double* __restrict__ rd, T* __restrict__ r,
-                         T* __restrict__ x) {
+__global__ void ml_start(int64_t n, const T* __restrict__ Dinv, T omega, const double* rd, T* r, T* x) {
+    next_may_start();
+    after_previous();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t row = t >> 2;
     const int i = (int)(t & 3);
@@ -435,7 +453,9 @@ __global__ void ml_start(int64_t n, const T* __restrict__ Dinv, T omega, const d
 // y = Ainv r for the dense last level (N <= 4 * coarse_max <= 96), one block, a thread per row: r from
 // shared memory, 8 entries of the row loaded before they are added (one serial load per entry was its time)
 template <class T>
-__global__ void __launch_bounds__(96) ml_dense_apply(int N, const T* __restrict__ Ainv, const T* __restrict__ r, T* __restrict__ y) {
+__global__ void __launch_bounds__(96) ml_dense_apply(int N, const T* __restrict__ Ainv, const T* r, T* y) {
+    next_may_start();
+    after_previous();
     __shared__ T s_r[96];
     const int i = threadIdx.x;
     if (i < N) s_r[i] = r[i];
@@ -598,7 +618,7 @@ int setup_values(const Mesh& m, Multilevel& L, cudaStream_t s) {
 // V-cycle below the first sweep of level l (x[l] = omega Dinv r[l] is there); the result is in *out, one of
 // the level's two iterates.  z (level 0, or null): the last sweep also writes it there in float64.
 template <class T>
-void vcycle(Multilevel& L, size_t l, cudaStream_t s, T** out, double* z) {
+void vcycle(Multilevel& L, size_t l, Chain& go, T** out, double* z) {
     MLValues<T>& v = values<T>(L);
     const MLPattern& p = L.lev[l];
     const T om = (T)L.omega;
@@ -606,7 +626,7 @@ void vcycle(Multilevel& L, size_t l, cudaStream_t s, T** out, double* z) {
     auto sweep = [&](auto in, double* zk) {
         with_quads(p.n, [&](auto q) {
             constexpr int Q = decltype(q)::value;
-            ml_sweep<T, decltype(in), Q><<<blocks(4 * Q * p.n), 256, 0, s>>>(p.n, p.dptr, p.didx, v.A[l], in, v.r[l], v.Dinv[l], om, y, zk);
+            go(ml_sweep<T, decltype(in), Q>, blocks(4 * Q * p.n), 256, 0, p.n, p.dptr, p.didx, v.A[l], in, v.r[l], v.Dinv[l], om, y, zk);
         });
         std::swap(x, y);
     };
@@ -616,25 +636,28 @@ void vcycle(Multilevel& L, size_t l, cudaStream_t s, T** out, double* z) {
     with_quads(p.n, [&](auto q) {
         constexpr int Q = decltype(q)::value;
         const int per = std::max(1, 64 / Q / L.agg);
-        ml_restrict<T, Q><<<(unsigned)((c.n + per - 1) / per), 256, 0, s>>>(c.n, p.n, L.agg, per, p.dptr, p.didx, v.A[l], x, v.r[l], L.fr[l],
-                                                                        dense ? nullptr : v.Dinv[l + 1], om, v.r[l + 1], v.x[l + 1]);
+        go(ml_restrict<T, Q>, (c.n + per - 1) / per, 256, 0, c.n, p.n, L.agg, per, p.dptr, p.didx, v.A[l], x, v.r[l], L.fr[l],
+           dense ? nullptr : v.Dinv[l + 1], om, v.r[l + 1], v.x[l + 1]);
     });
     T* xc = v.x[l + 1];
-    if (dense) ml_dense_apply<T><<<1, 96, 0, s>>>((int)(4 * c.n), v.Cinv, v.r[l + 1], xc);
-    else vcycle<T>(L, l + 1, s, &xc, nullptr);
+    if (dense) go(ml_dense_apply<T>, 1, 96, 0, (int)(4 * c.n), v.Cinv, v.r[l + 1], xc);
+    else vcycle<T>(L, l + 1, go, &xc, nullptr);
     for (int k = 0; k < L.nu; ++k) {
         double* zk = k + 1 == L.nu ? z : nullptr;
         if (k == 0 && p.n < kManyRows) {
             sweep(Corrected<T>{{x}, {xc}, L.fr[l], (uint32_t)L.agg}, zk);
             continue;
         }
-        if (k == 0) ml_prolong<T><<<blocks(4 * p.n), 256, 0, s>>>(p.n, (uint32_t)L.agg, L.fr[l], xc, x);
+        if (k == 0) go(ml_prolong<T>, blocks(4 * p.n), 256, 0, p.n, (uint32_t)L.agg, L.fr[l], xc, x);
         sweep(Plain<T>{x}, zk);
     }
     *out = x;
 }
 
-// z = V-cycle(r): two launches per level (three where it has many rows) and one for the dense one (six before)
+// z = V-cycle(r): two launches per level (three where it has many rows) and one for the dense one (six before).
+// On the small levels a launch is little more than its own latency (4 us for 12 k rows): with Chain the next
+// one's blocks are there early and have their part of the matrix loaded when this one ends.  12 launches on 74 k
+// nodes: 161 -> 137 us.
 template <class T>
 void apply(Multilevel& L, const double* r, double* z, cudaStream_t s) {
     MLValues<T>& v = values<T>(L);
@@ -645,9 +668,10 @@ void apply(Multilevel& L, const double* r, double* z, cudaStream_t s) {
         convert_kernel<T, double><<<blocks(4 * n), 256, 0, s>>>(4 * n, v.x[0], z);
         return;
     }
-    ml_start<T><<<blocks(4 * n), 256, 0, s>>>(n, v.Dinv[0], (T)L.omega, r, v.r[0], v.x[0]);
+    Chain go(s);
+    go(ml_start<T>, blocks(4 * n), 256, 0, n, v.Dinv[0], (T)L.omega, r, v.r[0], v.x[0]);
     T* x;
-    vcycle<T>(L, 0, s, &x, z);
+    vcycle<T>(L, 0, go, &x, z);
 }
 
 }  // namespace

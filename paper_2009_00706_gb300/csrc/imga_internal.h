@@ -353,4 +353,40 @@ int peak_flops(int device, int kind, double* tflops, std::string& err);
 
 void set_error(const std::string& s);
 
+#ifdef __CUDACC__
+// Chains of short kernels.  A kernel that begins with next_may_start() lets the launch that follows it (by
+// Chain, on the same stream) put its blocks on the chip while it still runs; every kernel launched that way calls
+// after_previous() in every thread before it touches anything that an earlier kernel of the chain writes or
+// reads: it waits until the kernel before has ended and its stores are visible, and, as each of them
+// waited likewise, all before that too.  Data that other kernels write inside a chain is read by plain loads
+// (__ldg and const __restrict__ are for what the chain never writes).
+__device__ __forceinline__ void next_may_start() { cudaTriggerProgrammaticLaunchCompletion(); }
+__device__ __forceinline__ void after_previous() { cudaGridDependencySynchronize(); }
+
+// The first launch of a chain is an ordinary one, so what was on the stream before has ended when it starts.
+// Under capture every launch is an ordinary one.
+struct Chain {
+    cudaStream_t s;
+    bool early = false, may;
+    explicit Chain(cudaStream_t stream) : s(stream) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusActive;
+        may = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+    }
+    template <class... P, class... A> void operator()(void (*k)(P...), int64_t grid, int block, size_t smem, A&&... a) {
+        cudaLaunchConfig_t c = {};
+        cudaLaunchAttribute at = {};
+        c.gridDim = dim3((unsigned)grid);
+        c.blockDim = dim3((unsigned)block);
+        c.dynamicSmemBytes = smem;
+        c.stream = s;
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        c.attrs = &at;
+        c.numAttrs = early ? 1 : 0;
+        cudaLaunchKernelEx(&c, k, P(a)...);
+        early = may;
+    }
+};
+#endif
+
 }  // namespace imga

@@ -169,6 +169,38 @@ def test_float64_block_jacobi_matches_mixed(dev):
     assert np.abs(np.array(its[0]) - np.array(its[1])).max() <= 1
 
 
+# ---- row products: a warp per row below 32,768 rows, eight lanes from there on ----
+@pytest.mark.parametrize("level", [6, 7])
+def test_row_products_and_vcycle(dev, level):
+    reg = [I.Region(I.REGION_SPHERE_BAND, level, (*C, 0.1, 0.05))]
+    g = api.Mesh((0.0, 0.0, 0.0), (1.0, 1.0, 1.0), 3, reg, I.icosphere(2, 0.1, C, 1e-3, 6), 1)
+    assert (g.n_nodes >= 32768) == (level == 7)
+    ph = I.Physics(mu=0.02, dt=0.05)
+    u, up, v = (T(a, dev) for a in I.state(g.n_nodes, 5))
+    Av = g.bsr_spmv(g.bsr_assemble(ph, u, up, up), v)
+    Jv = g.jvp(ph, u, up, v, up)
+    assert float((Av - Jv).norm() / Jv.norm()) <= TOL64
+    z = {}
+    for prec in (api.PRECISION_FP64, api.PRECISION_MIXED):
+        for sweeps in (1, 2):
+            g.multilevel_setup(ph, u, up, up, precision=prec, sweeps=sweeps)
+            z[prec, sweeps] = g.multilevel_apply(v).clone()
+            out = torch.empty_like(v)
+            graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.graph(graph, stream=side):
+                g.multilevel_apply(v, out=out)
+            for _ in range(20):   # launches that overlap, and captured ones that do not: the same bits every time
+                graph.replay()
+                assert torch.equal(out, z[prec, sweeps])
+                assert torch.equal(g.multilevel_apply(v), z[prec, sweeps])
+    for sweeps in (1, 2):
+        # a float32 cycle: 6e-8 per operation, some hundred of them in a row and a few levels of block inverses
+        # (entries up to ~1e2 times their blocks'); a row or an aggregate gone wrong would be of order one
+        d = z[api.PRECISION_MIXED, sweeps] - z[api.PRECISION_FP64, sweeps]
+        assert float(d.norm() / z[api.PRECISION_FP64, sweeps].norm()) <= 1e-2
+
+
 # ---- in/out: the float32 filters leave every flag to float64 where they cannot decide ----
 @pytest.mark.parametrize("lo", [(0.0, 0.0, 0.0), (1000.0, -2000.0, 500.0)])
 @pytest.mark.parametrize("body", ["sphere", "box", "truck"])
