@@ -17,7 +17,7 @@
 //    bound on its error, and only what that cannot decide is evaluated in float64: the flags are the
 //    float64 ones (normal_test, TriBox).  Leaves are found from a table of leading Morton bits.  445 k points
 //    around a truck (24,576 triangles, 3 % of them cast): 458 -> 142 us.
-//  * sub-cell quadrature: one thread per Intercepted element walks the sub-cell tree depth first
+//  * sub-cell quadrature: one warp per Intercepted element walks the sub-cell tree depth first
 //    in Morton child order (count pass, prefix sum, write pass), so every element's point list
 //    comes out in a fixed order.
 

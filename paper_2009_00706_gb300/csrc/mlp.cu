@@ -110,7 +110,7 @@ void gemm(cudaStream_t s, int M, int N, int K, const bf16* A, int64_t sam, int64
 // that reads X and writes Y once, with the activations of its BM rows in shared memory and registers
 // and the weights (0.56 MB) from L2; mma.sync is far from its rate there.  Every sum runs over k in
 // steps of 16 in increasing order, as in gemm_bf16: the same bits.
-//   50,003 rows: 2,625 -> 161 us (2.55 TB/s of X and Y).
+//   50,003 rows: 2,625 -> 158 us (2.6 TB/s of X and Y).
 // ------------------------------------------------------------------------------------------
 constexpr int kW = 128;            // width of the fused path
 constexpr int kHS = kW + 8;        // row stride of activations and of a weight chunk: conflict-free fragment reads
@@ -760,7 +760,7 @@ static void launch_fused(const Mlp& M, const float* X, int64_t ldx, int64_t n, f
 
 // Rows per CTA: 64 (the weights are read from L2 once per 64 rows) when that still gives two CTAs per SM,
 // fewer for fewer rows, so that the chip has work (9,000 rows: 51 us with 32).  From 64 x 2 x 152 rows on 64; the small tile takes 8
-// warps, deep stages and wide chunks because a CTA is alone on its SM (1,024-row training steps: 61 -> 33 us).
+// warps, deep stages and wide chunks because a CTA is alone on its SM (1,024-row training steps: 61 -> 26 us).
 template <bool TRAIN>
 static void mlp_fused_rows(const Mlp& M, const float* X, int64_t ldx, int64_t n, float* Y, const MlpTrainIO& io, cudaStream_t s) {
     if (n >= 64 * 152 * 2) launch_fused<64, 128, 32, 64, 3, TRAIN>(M, X, ldx, n, Y, io, s);

@@ -14,13 +14,15 @@
 // J v is the forward-mode derivative of the same code (dual numbers value + tangent): the
 // matrix of Algorithms 2/4 applied to v without being formed.
 //
-// Kernels (T = float or double element arithmetic, nodal gathers always float64, scatter by
-// float64 atomics):
+// Kernels (T = float or double element arithmetic, nodal gathers always float64, scatter into slots
+// that node_gather sums, or by float64 atomics):
 //   vms_interior  8 threads per Out element: thread c gathers corner c, evaluates Gauss point c,
 //                 then contracts node c's four rows over the 8 points; interpolation and test
 //                 functions both run in the monomial form of the trilinear basis.
+//                 float64: interior_element64, the same with fewer FP64 instructions.
 //   vms_cut       one warp per Intercepted element; lane l evaluates sub-cell points l, l + 32, ...
-//                 and accumulates their monomial moments, summed over the lanes at the end.
+//                 and accumulates their monomial moments, summed over the lanes at the end;
+//   vms_cut_split four warps per element where elements are few, vms_cut64 in float64.
 //   nitsche       one thread per surface point, for elements hosting few points;
 //   nitsche_el    one warp per element hosting many, lanes over its points (moments).
 //   strong_rows   Dirichlet rows U - g and In-only rows, written after every scatter.
@@ -60,7 +62,7 @@ template <class T> struct IntShape {
 // element code, with the roundings it has always had.  Such a solve turns the last bit of a residual into
 // float32 steps of its preconditioner and matvecs, and those into differences as large as its tolerance
 // (1e-9 to 1e-7 of u at 1e-8), so other roundings there would make other solutions, no nearer and no
-// further from the root.  It costs a solve of the 7.3 k element sphere 4 of 40 ms.  Everything else,
+// further from the root.  It costs a solve of the 7.3 k element sphere 1.5 of 35 ms.  Everything else,
 // float64 solves included, takes the kernels below.
 //
 // One Out element in float64 on 8 lanes of a warp (c = lane & 7); nd its 8 corner rows, sw the warp's
