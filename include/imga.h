@@ -465,8 +465,8 @@ enum { IMGA_OPT_GRAPHS = 1, IMGA_OPT_AUTOTUNE = 2, IMGA_OPT_CLASSIFY_RAYS = 3, I
        IMGA_OPT_FUSED_SPLIT = 6, IMGA_OPT_CONCURRENT = 7 };
 imga_status imga_set_option(imga_mesh mesh, int option, int64_t value);
 
-/* The tile shapes in use.  shape[8] = {warps per block, longest-first order} for
- * [float64, mixed] x [residual, J v].  If ms is non-null, ms[24] receives the per-launch milliseconds
+/* The tuned tile shapes.  shape[8] = {warps per block, 1 if tuned to longest-first order} for
+ * [float64, mixed] x [residual, J v]; {4, 0} where not tuned (4 warps, longest first).  If ms is non-null, ms[24] receives the per-launch milliseconds
  * of the last tuning for the same 4 cases x 6 candidates (warps 2, 4, 8) x (Morton, longest first);
  * an entry is 0 where not measured. */
 imga_status imga_tuning(imga_mesh mesh, int32_t* shape, float* ms);

@@ -207,7 +207,7 @@ struct Mesh {
     bool use_graphs = false;
     // Intercepted-element bucket: warps per block and element order (0 Morton, 1 longest first),
     // per [float64 0 / mixed 1][residual 0 / J v 1]; set by the autotuner
-    struct CutTune { int wpb = 4, lpt = 1; };
+    struct CutTune { int wpb = 4, lpt = 0; bool tuned = false; };   // until tuned: longest first, reported as 0
     CutTune cut_tune[2][2];
     float cut_tune_ms[2][2][6] = {};   // candidate times of the last tuning (ms per launch)
     bool tune_pending[2][2] = {{false, false}, {false, false}};

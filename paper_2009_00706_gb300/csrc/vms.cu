@@ -1453,7 +1453,7 @@ int autotune_cut(Mesh& m, Args A, cudaStream_t s) {
             cudaEventElapsedTime(&ms, e0, e1);
             ms /= 3.f;
             m.cut_tune_ms[sizeof(T) == 4][JV][2 * wi + lpt] = ms;
-            if (ms < best) { best = ms; ct.wpb = wpbs[wi]; ct.lpt = lpt; }
+            if (ms < best) { best = ms; ct = {wpbs[wi], lpt, true}; }
         }
     // the Out-element bucket: the persistent interior kernel with 1 .. (occupancy limit) blocks per SM
     const int64_t no = (int64_t)m.out_list.size();
@@ -1632,7 +1632,7 @@ void launch_all(const Mesh& m, Args A, cudaStream_t s, void* ws = nullptr, cudaS
     if (nc > 0) {
         Timed t(m, 1, sc, 1, !ws);
         const Mesh::CutTune& ct = m.cut_tune[sizeof(T) == 4][JV];
-        launch_cut<T, JV>(m, A, sc, ct.wpb, ct.lpt, generic);
+        launch_cut<T, JV>(m, A, sc, ct.wpb, ct.lpt || !ct.tuned, generic);
     }
     launch_surface<T, JV>(m, A, ss, !ws);
     if (ev) {   // join
