@@ -1710,7 +1710,7 @@ void graphs_free(Mesh& m) {
 }
 
 // the mesh's side streams and fork / join events (created on first use)
-static int side_streams(Mesh& mm) {
+int side_streams(Mesh& mm) {
     if (mm.side[0]) return 0;
     for (int k = 0; k < 3; ++k)
         if (cudaStreamCreateWithFlags((cudaStream_t*)&mm.side[k], cudaStreamNonBlocking) != cudaSuccess) return 1;
