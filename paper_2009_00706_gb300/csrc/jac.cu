@@ -55,7 +55,7 @@ __device__ __forceinline__ int corner_nodes(const Args& A, int32_t id, int32_t n
 // M_e^T k_e M_e (Algorithm 2): every parent pair (p, q) receives w_p w_q v in block (p, q), entry at[j]
 // (4 x row component + column component).  The row is searched once per corner pair: entry by entry the
 // searches were most of the assembly (43.6 k elements,
-// mixed: 5.37 -> 1.86 ms with the basis tables, the shared test functions and the adds below).
+// mixed: 5.37 -> 1.45 ms with the basis tables, the shared test functions, the adds below and selected seeds).
 // A warp adds whole blocks from shared memory where it can (bsr_add_blocks): 16 lanes on the 128 bytes of a
 // block make 4 L2 transactions of what lane-by-lane adds make 16 of.
 // Float entries are weighted (powers of two: exact) and tested in float32 and widened on the integer pipe:
@@ -120,28 +120,27 @@ __device__ __forceinline__ void bsr_add_hanging(const Args& A, int32_t ida, int3
 template <class T>
 __device__ __forceinline__ void seed_fields(const Args& A, const Fields<T, T>& V, T g, T phb, const T dphb[3],
                                             const T d2b[3], int k, Fields<Dual<T>, T>& F) {
+    // (k is known only at run time, so tangents are selected: an indexed store would put F in local memory)
     const T th = (T)A.theta, c0 = (T)A.c0, g2 = g * g;
+    const T tu = th * phb, ta = c0 * phb;
+    T tg[3], tp[3], th2[3];
+    for (int j = 0; j < 3; ++j) { tg[j] = th * g * dphb[j]; tp[j] = g * dphb[j]; th2[j] = th * g2 * d2b[j]; }
+    const bool vel = k < 3;
+#pragma unroll
     for (int i = 0; i < 3; ++i) {
-        F.us[i] = {V.us[i], T(0)};
-        F.at[i] = {V.at[i], T(0)};
-        F.gp[i] = {V.gp[i], T(0)};
-        F.H2[i] = {V.H2[i], T(0)};
+        const bool own = i == k;
+        F.us[i] = {V.us[i], own ? tu : T(0)};
+        F.at[i] = {V.at[i], own ? ta : T(0)};
+        F.gp[i] = {V.gp[i], vel ? T(0) : tp[i]};
+        // (grad div u)_i = sum_{j != i} d_i d_j u_j: a unit u_k at corner b feeds every i != k, by pair (i, k)
+        // (xy, xz, yz: 0, 1, 2)
+        const T h = i == 0 ? (k == 1 ? th2[0] : th2[1]) : i == 1 ? (k == 0 ? th2[0] : th2[2]) : (k == 0 ? th2[1] : th2[2]);
+        F.H2[i] = {V.H2[i], vel && !own ? h : T(0)};
         F.f[i] = V.f[i];
-        for (int j = 0; j < 3; ++j) F.Gu[i][j] = {V.Gu[i][j], T(0)};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) F.Gu[i][j] = {V.Gu[i][j], own ? tg[j] : T(0)};
     }
-    F.p = {V.p, T(0)};
-    if (k < 3) {
-        F.us[k].d = th * phb;
-        F.at[k].d = c0 * phb;
-        for (int j = 0; j < 3; ++j) F.Gu[k][j].d = th * g * dphb[j];
-        // (grad div u)_i = sum_{j != i} d_i d_j u_j: a unit u_k at corner b feeds every i != k
-        const int pair[3][3] = {{-1, 0, 1}, {0, -1, 2}, {1, 2, -1}};
-        for (int i = 0; i < 3; ++i)
-            if (i != k) F.H2[i].d = th * g2 * d2b[pair[i][k]];
-    } else {
-        F.p.d = phb;
-        for (int j = 0; j < 3; ++j) F.gp[j].d = g * dphb[j];
-    }
+    F.p = {V.p, vel ? T(0) : phb};
 }
 
 template <class T>
@@ -172,13 +171,19 @@ __device__ __forceinline__ void add_diag(const Args& A, int32_t id, const double
 
 template <class T> struct JacShape { static constexpr int EPB = 16; };
 
+// Bound by issue and dependent chains, so no indexed local arrays (the seeds are selected, see seed_fields) and
+// registers for five blocks per SM, 2.8 waves instead of 3.5 on 33.7 k Out elements: an assembly of 43.6 k
+// elements 1,858 -> 1,505 us with the selected seeds here and in jac_cut, 1,450 with the fifth block and the
+// 16-byte accesses below.
 template <class T, int MODE>
-__global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const int32_t* __restrict__ list, int64_t n,
+__global__ void __launch_bounds__(8 * JacShape<T>::EPB, sizeof(T) == 4 ? 5 : 1) jac_out(Args A, const int32_t* __restrict__ list, int64_t n,
                                                                 const int32_t* __restrict__ slot, double* __restrict__ K,
                                                                 double* __restrict__ D) {
     constexpr int EPB = JacShape<T>::EPB;
     __shared__ __align__(16) T s_nd[EPB][8][CS];
-    __shared__ T s_cf[EPB][8][17];
+    // a Gauss point's coefficients, in fours (component i: phi and gradient coefficients), for 16-byte accesses;
+    // the strides keep the four elements of a warp, and its points, on different banks
+    __shared__ __align__(16) T s_cf[EPB][8 * 20 + 4];
     __shared__ __align__(16) T s_bas[8][8][4];   // [Gauss point q][corner c]: phi, reference gradient
     __shared__ T s_blk[MODE == BSR ? EPB / 4 : 1][32][17];      // BSR: block (corner c, corner b) of every lane
     __shared__ int64_t s_pos[MODE == BSR ? EPB / 4 : 1][32];
@@ -231,7 +236,10 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
             seed_fields<T>(A, V, g, phb, dphb, d2b, k, F);
             Dual<T> cf[16];
             pointwise<Dual<T>, T>(A, Phys<T>(A, prob_of(A, e)), F, g, cf);
-            for (int q = 0; q < 16; ++q) s_cf[le][c][q] = ((q < 3 || q == 12) ? wq : wqg) * cf[q].d;
+            T cw[16];
+            for (int q = 0; q < 16; ++q) cw[q] = ((q < 3 || q == 12) ? wq : wqg) * cf[q].d;
+            for (int i = 0; i < 3; ++i) st4s<T>(&s_cf[le][20 * c + 4 * i], cw[i], cw[3 + 3 * i], cw[4 + 3 * i], cw[5 + 3 * i]);
+            st4s<T>(&s_cf[le][20 * c + 12], cw[12], cw[13], cw[14], cw[15]);
             __syncwarp();
             T r[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
@@ -240,9 +248,11 @@ __global__ void __launch_bounds__(8 * JacShape<T>::EPB) jac_out(Args A, const in
                 ld4s<T>(&s_bas[q][c][0], bs);
                 const T ph = bs[0];
                 const T* dp = bs + 1;
-                const T* C = s_cf[le][q];
-                for (int i = 0; i < 3; ++i) r[i] += ph * C[i] + dp[0] * C[3 + 3 * i] + dp[1] * C[4 + 3 * i] + dp[2] * C[5 + 3 * i];
-                r[3] += ph * C[12] + dp[0] * C[13] + dp[1] * C[14] + dp[2] * C[15];
+                for (int i = 0; i < 4; ++i) {
+                    T C[4];
+                    ld4s<T>(&s_cf[le][20 * q + 4 * i], C);
+                    r[i] += ph * C[0] + dp[0] * C[1] + dp[1] * C[2] + dp[2] * C[3];
+                }
             }
             __syncwarp();
             if (MODE == FULL) {
