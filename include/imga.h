@@ -241,7 +241,8 @@ imga_status imga_bsr_pattern(imga_mesh mesh, int64_t* n_blocks, int64_t* indptr,
 imga_status imga_bsr_assemble(imga_mesh mesh, const double* u, const double* u_prev, const double* u_prev2,
                               const double* f, const imga_physics* phys, int precision, double* vals, void* stream);
 /* y = K x with an assembled matrix vals of this mesh's block pattern; x, y DEVICE float64 [n_nodes][4].
- * Needs the pattern on the device (any earlier imga_bsr_assemble or imga_multilevel_setup). */
+ * Needs the pattern on the device (any earlier imga_bsr_assemble or imga_multilevel_setup).  vals, x and
+ * y (here and in imga_bsr_assemble) may start at any 8-byte address; vals and x are read faster from 16-byte ones. */
 imga_status imga_bsr_spmv(imga_mesh mesh, const double* vals, const double* x, double* y, void* stream);
 
 /* Multilevel preconditioner by block coarsening of the assembled Jacobian (no counterpart in the

@@ -23,6 +23,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -49,10 +50,15 @@ constexpr int kMaxLevels = 24;
 constexpr int kRowAhead = 4;
 constexpr int64_t kManyRows = 32768;
 
+// WIDE: 16-byte loads.  The caller's float64 arrays of imga_bsr_spmv may start at any 8-byte address (a view into a
+// packed buffer); those that do not start at a 16-byte one are read entry by entry.
 template <class T> struct Row4 { T v[4]; };
-template <class T> __device__ __forceinline__ Row4<T> load_row(const T* p) {
+template <bool WIDE = true, class T> __device__ __forceinline__ Row4<T> load_row(const T* p) {
     Row4<T> r;
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (!WIDE) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) r.v[k] = __ldg(p + k);
+    } else if constexpr (sizeof(T) == 4) {
         const float4 a = __ldg(reinterpret_cast<const float4*>(p));
         r.v[0] = a.x; r.v[1] = a.y; r.v[2] = a.z; r.v[3] = a.w;
     } else {
@@ -67,11 +73,14 @@ template <class T> __device__ __forceinline__ T dot4(const T* a, const T* b) {
 }
 
 // a vector entry of the cycle: x, or x plus the coarse correction of its aggregate on free unknowns
-template <class T> struct Plain {
+template <class T, bool WIDE = true> struct Plain {
     const T* x;
     __device__ Row4<T> operator()(int64_t c) const {   // (x is rewritten between launches: no read-only loads)
         Row4<T> r;
-        if constexpr (sizeof(T) == 4) {
+        if constexpr (!WIDE) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) r.v[k] = x[4 * c + k];
+        } else if constexpr (sizeof(T) == 4) {
             const float4 a = reinterpret_cast<const float4*>(x)[c];
             r.v[0] = a.x; r.v[1] = a.y; r.v[2] = a.z; r.v[3] = a.w;
         } else {
@@ -98,7 +107,7 @@ template <class T> struct Corrected {
 
 // component (lane & 3) of row `row` of A x, on the row's 4 Q lanes (live: this row exists; every lane of the
 // warp calls).  begin() runs once, before x is first read: the matrix is loaded ahead of it.
-template <int Q, class T, class X, class B>
+template <int Q, class T, bool WIDE = true, class X, class B>
 __device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                          const T* __restrict__ val, const X& x, B&& begin) {
     constexpr int D = kRowAhead;   // steps in flight
@@ -116,7 +125,7 @@ __device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* 
             c[g] = -1;
             if (q < q1) {   // (the block does not wait for its column)
                 c[g] = __ldg(idx + q);
-                a[g] = load_row(val + 16 * q + 4 * i);
+                a[g] = load_row<WIDE>(val + 16 * q + 4 * i);
             }
         }
         if (!begun) begin();
@@ -139,12 +148,12 @@ __device__ __forceinline__ T row_product(bool live, int64_t row, const int64_t* 
 }
 
 // y = A x
-template <class T, int Q>
+template <class T, int Q, bool WIDE>
 __global__ void __launch_bounds__(256) bsr_mul(int64_t n, const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                                                const T* __restrict__ val, const T* __restrict__ x, T* __restrict__ y) {
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (4 * Q);
     const int l = threadIdx.x & (4 * Q - 1);
-    const T acc = row_product<Q, T>(row < n, row, ptr, idx, val, Plain<T>{x}, [] {});
+    const T acc = row_product<Q, T, WIDE>(row < n, row, ptr, idx, val, Plain<T, WIDE>{x}, [] {});
     if (row < n && l < 4) y[4 * row + l] = acc;
 }
 
@@ -780,10 +789,13 @@ int bsr_spmv(Mesh& m, const double* val, const double* x, double* y, void* strea
     Multilevel* L = (Multilevel*)m.mlev;
     if (!L) { err = "the block pattern is not on the device (call the assembly first)"; return 1; }
     const MLPattern& p = L->lev[0];
+    const bool wide = (((uintptr_t)val | (uintptr_t)x) & 15) == 0;
     if (p.n > 0)
         with_quads(p.n, [&](auto q) {
             constexpr int Q = decltype(q)::value;
-            bsr_mul<double, Q><<<blocks(4 * Q * p.n), 256, 0, (cudaStream_t)stream>>>(p.n, p.dptr, p.didx, val, x, y);
+            auto run = [&](auto kernel) { kernel<<<blocks(4 * Q * p.n), 256, 0, (cudaStream_t)stream>>>(p.n, p.dptr, p.didx, val, x, y); };
+            if (wide) run(bsr_mul<double, Q, true>);
+            else run(bsr_mul<double, Q, false>);
         });
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }

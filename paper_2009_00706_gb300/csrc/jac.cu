@@ -1067,13 +1067,20 @@ __global__ void bsr_strong_rows(int64_t nn, const int64_t* __restrict__ ptr, con
     uint8_t mask = umask ? umask[n] : (uint8_t)(flag[n] & 15);
     if (flag[n] & 16) mask = 15;
     if (!mask) return;
+    const bool wide = (reinterpret_cast<uintptr_t>(val) & 15) == 0;   // (the caller's matrix may start at any 8-byte address)
     for (int64_t q = ptr[n] + (t & 7); q < ptr[n + 1]; q += 8)
         for (int k = 0; k < 4; ++k)
             if ((mask >> k) & 1) {
                 const bool d = idx[q] == n;
-                double2* o = reinterpret_cast<double2*>(val + 16 * q + 4 * k);
-                o[0] = make_double2(d && k == 0 ? 1.0 : 0.0, d && k == 1 ? 1.0 : 0.0);
-                o[1] = make_double2(d && k == 2 ? 1.0 : 0.0, d && k == 3 ? 1.0 : 0.0);
+                const double r[4] = {d && k == 0 ? 1.0 : 0.0, d && k == 1 ? 1.0 : 0.0, d && k == 2 ? 1.0 : 0.0, d && k == 3 ? 1.0 : 0.0};
+                double* o = val + 16 * q + 4 * k;
+                if (wide) {
+                    reinterpret_cast<double2*>(o)[0] = make_double2(r[0], r[1]);
+                    reinterpret_cast<double2*>(o)[1] = make_double2(r[2], r[3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) o[j] = r[j];
+                }
             }
 }
 

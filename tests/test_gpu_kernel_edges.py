@@ -233,3 +233,36 @@ def test_classify_near_the_surface(dev, body, lo):
     g.classify_rays_only(True)
     rays = g.classify(T(pts[4000:8000], dev)).cpu().numpy()
     assert np.array_equal(rays, want[4000:8000])
+
+
+# ---- the caller's matrix and vectors as float64 views that start at an odd element (8-byte, not 16-byte
+# addresses), on both sides of the size where the row products change shape ----
+@pytest.mark.parametrize("level", [5, 7])
+def test_matrix_in_views_at_odd_elements(dev, level):
+    reg = [I.Region(I.REGION_SPHERE_BAND, level, (*C, 0.1, 0.05))]
+    g = api.Mesh((0.0, 0.0, 0.0), (1.0, 1.0, 1.0), 3, reg, I.icosphere(2, 0.1, C, 1e-3, 6), 1)
+    assert (g.n_nodes >= 32768) == (level == 7)
+    ph = I.Physics(mu=0.02, dt=0.05)
+    u, up, v = (T(a, dev) for a in I.state(g.n_nodes, 5))
+    ptr, idx = g.bsr_pattern()
+
+    def odd(*shape):
+        t = torch.empty(1 + int(np.prod(shape)), dtype=torch.float64, device=dev)[1:].view(*shape)
+        assert t.data_ptr() % 16 == 8
+        return t
+
+    A = g.bsr_assemble(ph, u, up)
+    B = g.bsr_assemble(ph, u, up, out=odd(idx.size, 4, 4))
+    # float64 atomics add at most a few dozen terms per entry, in any order
+    assert float((A - B).abs().max() / A.abs().max()) <= 1e-13
+    rows = torch.from_numpy(np.repeat(np.arange(g.n_nodes), np.diff(ptr))).to(dev)
+    on = rows == torch.from_numpy(idx.astype(np.int64)).to(dev)
+    eye = torch.eye(4, dtype=torch.float64, device=dev)
+    s = torch.zeros(g.n_nodes, 4, dtype=torch.float64, device=dev).index_add_(0, rows, B.abs().sum(2))
+    flat = s == 1.0                                       # identity rows
+    assert flat[:, :3].any() and torch.equal(B[on][flat], eye.expand(g.n_nodes, 4, 4)[flat])
+    B.copy_(A)
+    w = odd(g.n_nodes, 4).copy_(v)
+    want = g.bsr_spmv(A, v)
+    for vals, x in ((B, v), (A, w), (B, w)):
+        assert torch.equal(g.bsr_spmv(vals, x, out=odd(g.n_nodes, 4)), want)
