@@ -136,6 +136,46 @@ __device__ __forceinline__ uint32_t cvt2(float lo, float hi) {   // one conversi
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// A thread's sum of squares, no less exact than a float64 one: the square is exact in two floats, and the sum is
+// kept in three (TwoSum: hi + mid exactly what was added but for mid's own rounding errors, which lo adds up), 72 bits
+// against 53.  Where a value's square or its low part leaves the float32 range (below 2^-51, from 2^58 on, inf, NaN)
+// the N values go to a float64 sum.  One float64 multiply-add per value instead cost a training step of 1,024 rows 6 of 79 us:
+// the FP64 pipe takes a warp's instruction every 19 cycles and 64 of the SMs had all of them.
+struct SquareSum {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    double wide = 0.0;
+    static __device__ __forceinline__ float two_sum(float& s, float x) {   // s += x, the rounding error returned
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s), e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+        s = t;
+        return e;
+    }
+    template <int N> __device__ __forceinline__ void add(const float* d) {
+        constexpr uint32_t least = (127u - 51u) << 23, end = (127u + 58u) << 23;
+        uint32_t lowest = ~0u, highest = 0u;   // magnitudes' bits less one: a zero is above all of them, and harmless
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const uint32_t b = __float_as_uint(d[k]) & 0x7FFFFFFFu;
+            lowest = min(lowest, b - 1u);
+            highest = max(highest, b);
+        }
+        if (lowest >= least - 1u && highest < end) {
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const float p = __fmul_rn(d[k], d[k]), e = __fmaf_rn(d[k], d[k], -p);
+                const float a = two_sum(mid, two_sum(hi, p)), b = two_sum(mid, e);
+                lo = __fadd_rn(lo, __fadd_rn(a, b));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const double x = f2d(d[k]);
+                wide = fma(x, x, wide);
+            }
+        }
+    }
+    __device__ __forceinline__ double total() const { return (double)hi + ((double)mid + ((double)lo + wide)); }
+};
+
 struct MlpTrainIO {           // what a training step keeps of the forward pass
     const float* T;           // targets [n][nout]
     float inv_scale;
@@ -331,7 +371,7 @@ __global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad,
 #pragma unroll
                 for (int q = 0; q < 4; q += 2)
                     put_h(&z2[k][i][j][q], b2, wm + 16 * i + gid + q * 4, k * kNC + wn * (kNC / WN) + 8 * j + 2 * tig, io.h2);
-    float lhi = 0.f, llo = 0.f;   // training: sum (y - t)^2 of this thread in two floats
+    SquareSum sq;   // training: this thread's sum of (y - t)^2
     for (int k = kW / kNC; k < nchunk; ++k) {
         const int n0 = (k - kW / kNC) * kNC + wn * (kNC / WN) + 2 * tig;
         float2 tg[TRAIN ? MI : 1][TRAIN ? N2 : 1][2];
@@ -362,26 +402,27 @@ __global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad,
                 for (int q = 0; q < 4; q += 2) {
                     const int64_t r = m0 + wm + 16 * i + gid + q * 4;
                     const int c = n0 + 8 * j;
-                    if (r >= n || c >= nout) continue;   // nout is even
-                    const float y0 = o[i][j][q] + __ldg(b3 + c), y1 = o[i][j][q + 1] + __ldg(b3 + c + 1);
+                    float &y0 = o[i][j][q], &y1 = o[i][j][q + 1];
+                    if (r >= n || c >= nout) {   // nout is even
+                        y0 = y1 = 0.f;
+                        continue;
+                    }
+                    y0 += __ldg(b3 + c);
+                    y1 += __ldg(b3 + c + 1);
                     if constexpr (!TRAIN) {
                         *reinterpret_cast<float2*>(Y + r * nout + c) = make_float2(y0, y1);
-                    } else {
+                    } else {   // from here on the errors
                         const float2 t = tg[i][j][q >> 1];
-                        const float d0 = y0 - t.x, d1 = y1 - t.y;
-                        *reinterpret_cast<uint32_t*>(io.dy + r * nout + c) = cvt2(d0 * io.inv_scale, d1 * io.inv_scale);
-                        // exact square (two floats) added with TwoSum: float64's narrow pipe stays out of it
-                        for (const float d : {d0, d1}) {
-                            const float sq = __fmul_rn(d, d), s = __fadd_rn(lhi, sq), bp = __fsub_rn(s, lhi);
-                            llo += __fadd_rn(__fsub_rn(lhi, __fsub_rn(s, bp)), __fsub_rn(sq, bp)) + __fmaf_rn(d, d, -sq);
-                            lhi = s;
-                        }
+                        y0 -= t.x;
+                        y1 -= t.y;
+                        *reinterpret_cast<uint32_t*>(io.dy + r * nout + c) = cvt2(y0 * io.inv_scale, y1 * io.inv_scale);
                     }
                 }
+        if constexpr (TRAIN) sq.template add<MI * N2 * 4>(&o[0][0][0]);
     }
     cp_wait<0>();
     if constexpr (TRAIN) {
-        double s = (double)lhi + (double)llo;
+        double s = sq.total();
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) atomicAdd(io.loss, s);
     }

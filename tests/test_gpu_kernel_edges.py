@@ -266,3 +266,22 @@ def test_matrix_in_views_at_odd_elements(dev, level):
     want = g.bsr_spmv(A, v)
     for vals, x in ((B, v), (A, w), (B, w)):
         assert torch.equal(g.bsr_spmv(vals, x, out=odd(g.n_nodes, 4)), want)
+
+
+# ---- the training loss is a float64 sum of float64 squares ----
+@pytest.mark.parametrize("rows", [16, 1000, 5000])
+def test_mlp_loss_is_a_float64_sum(dev, rows):
+    net = api.Mlp(seed=1)
+    net.set_params(np.zeros(net.n_params, np.float32))    # y = 0: the errors are the targets
+    X = torch.zeros(rows, 1027, device=dev)
+    # at most 64 additions in a thread, 5 over its warp, then one of at most rows / 2 warps after another
+    tol = (64 + 5 + rows / 2) * 2.0 ** -53
+    for c in (1.9767611, 1.4614793, 3e-20, 1e20):         # squares below and above the float32 range among them
+        t = torch.full((rows, 1024), c, device=dev)
+        want = 0.5 * 1024 * float(t[0, 0].double()) ** 2
+        assert abs(net.gradient(X, t)[0] / want - 1) <= tol, c
+    t = torch.randn(rows, 1024, device=dev)
+    t[rows // 2, 7] = float("inf")
+    assert net.gradient(X, t)[0] == float("inf")
+    t[0, 0] = float("nan")
+    assert np.isnan(net.gradient(X, t)[0])
