@@ -397,7 +397,8 @@ imga_status imga_mlp_shape(imga_mlp mlp, int64_t* n_params, int* n_in_pad);
 /* FP32 master weights in the order W1 [width][n_in_pad], b1, W2 [width][width], b2, W3 [n_out][width],
  * b3 (host array of n_params floats); set = 1 writes them (and resets Adam), set = 0 reads. */
 imga_status imga_mlp_params(imga_mlp mlp, float* host, int set);
-/* Y [n][n_out] = MLP(X [n][ldx], first n_in columns), float32 device arrays */
+/* Y [n][n_out] = MLP(X [n][ldx], first n_in columns), float32 device arrays.  Y may be X itself where ldx >= n_out
+ * (results overwrite the inputs); arrays that overlap take a slower path through a buffer of the network. */
 imga_status imga_mlp_forward(imga_mlp mlp, const float* X, int64_t ldx, int64_t n, float* Y, void* stream);
 /* loss and gradient (host, n_params floats, same order as the weights) over all n samples */
 imga_status imga_mlp_gradient(imga_mlp mlp, const float* X, int64_t ldx, const float* T, int64_t n, double* loss,

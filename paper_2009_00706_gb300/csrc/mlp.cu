@@ -929,7 +929,9 @@ int mlp_grads(Mlp* M, float* host) { return cudaMemcpy(host, M->G, M->nparam * 4
 
 int mlp_forward(Mlp* M, const float* X, int64_t ldx, int64_t n, float* Y, cudaStream_t s) {
     const int64_t B = 4096;
-    if (mlp_fast(*M) && ((uintptr_t)Y & 7) == 0) {
+    // (in place, or overlapping otherwise: batch by batch, each read whole before its results are written)
+    const bool apart = (uintptr_t)(Y + n * M->nout) <= (uintptr_t)X || (uintptr_t)(X + (n - 1) * ldx + M->nin) <= (uintptr_t)Y;
+    if (mlp_fast(*M) && ((uintptr_t)Y & 7) == 0 && (apart || n == 0)) {
         if (n > 0) mlp_fused_rows<false>(*M, X, ldx, n, Y, MlpTrainIO{}, s);
         return cudaGetLastError() == cudaSuccess ? 0 : 1;
     }

@@ -285,3 +285,15 @@ def test_mlp_loss_is_a_float64_sum(dev, rows):
     assert net.gradient(X, t)[0] == float("inf")
     t[0, 0] = float("nan")
     assert np.isnan(net.gradient(X, t)[0])
+
+
+# ---- results written over the inputs: one thread block's results reach the rows that another reads ----
+@pytest.mark.parametrize("rows", [17, 1000, 5000])
+@pytest.mark.parametrize("nin,nout,ldx", [(1027, 1024, 1040), (45, 72, 72)])
+def test_mlp_forward_in_place(dev, rows, nin, nout, ldx):
+    net = api.Mlp(n_in=nin, n_out=nout, seed=3)
+    torch.manual_seed(rows)
+    X = torch.randn(rows, ldx, device=dev)
+    want = net.forward(X.clone())
+    api.check(_lib.load().imga_mlp_forward(net.h, api._ptr(X), ldx, rows, api._ptr(X), api._stream(None)))
+    assert torch.equal(X.view(-1)[: rows * nout].view(rows, nout), want)   # the same sums in the same order
