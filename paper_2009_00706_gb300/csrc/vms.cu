@@ -912,7 +912,8 @@ template <class T> struct FusedShape {
     static constexpr size_t smem = (size_t)kFusedWarps * WARP * sizeof(T);
 };
 
-template <class T, bool JV>
+// GEN: as in vms_interior
+template <class T, bool JV, bool GEN = false>
 __global__ void __launch_bounds__(32 * kFusedWarps, sizeof(T) == 4 ? 4 : 2) vms_fused(Args A, FusedQueue Q) {
     constexpr int ESTR = FusedShape<T>::ESTR, MSTR = FusedShape<T>::MSTR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -926,7 +927,7 @@ __global__ void __launch_bounds__(32 * kFusedWarps, sizeof(T) == 4 ? 4 : 2) vms_
             if (lane == 0) h = atomicAdd(Q.cnt, 1ull);
             h = __shfl_sync(0xffffffffu, h, 0);
             if ((int64_t)h >= Q.n_items) break;
-            if constexpr (sizeof(T) == 8)
+            if constexpr (sizeof(T) == 8 && !GEN)
                 cut_element64<JV>(A, Q.cut_list, Q.cut_off, (const double*)Q.cut_pts, (int64_t)Q.items[h], base, lane);
             else
                 cut_element<T, JV>(A, Q.cut_list, Q.cut_off, Q.cut_pts, (int64_t)Q.items[h], base, base + 8 * CS, lane);
@@ -985,7 +986,7 @@ __global__ void __launch_bounds__(32 * kFusedWarps, sizeof(T) == 4 ? 4 : 2) vms_
                     const int lp_next = nxt >= 0 ? level_prob(nxt) : 0;
                     cp_wait<1>();
                     const int64_t idx = 4 * cur + le;
-                    if constexpr (sizeof(T) == 8)
+                    if constexpr (sizeof(T) == 8 && !GEN)
                         interior_element64<JV>(A, base + (buf * 4 + le) * ESTR, s_mw, lane, idx, idx < Q.n_out, lp_cur & 255,
                                                lp_cur >> 8, id_cur);
                     else
@@ -1517,14 +1518,14 @@ void launch_interior(const Mesh& m, const Args& A, cudaStream_t s, int bps, bool
 }
 
 // Resident CTAs of the fused kernel per SM (queried once; also sets its dynamic smem opt-in).
-template <class T, bool JV>
+template <class T, bool JV, bool GEN = false>
 int fused_blocks_per_sm() {
     static int bps = 0;
     if (bps == 0) {
         const size_t smem = FusedShape<T>::smem;
         int b = 0;
-        cudaFuncSetAttribute(vms_fused<T, JV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, vms_fused<T, JV>, 32 * kFusedWarps, smem);
+        cudaFuncSetAttribute(vms_fused<T, JV, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, vms_fused<T, JV, GEN>, 32 * kFusedWarps, smem);
         bps = b < 1 ? 1 : b;
     }
     return bps;
@@ -1563,7 +1564,7 @@ void launch_surface(const Mesh& m, const Args& A, cudaStream_t ss, bool timed) {
 // the Out and Intercepted buckets in one persistent launch (vms_fused); the surface kernels beside
 // it on the side stream ss (forked and joined with the events ev), or after it on s
 template <class T, bool JV>
-void launch_fused(const Mesh& m, const Args& A, cudaStream_t s, cudaStream_t ss, cudaEvent_t* ev, bool timed) {
+void launch_fused(const Mesh& m, const Args& A, cudaStream_t s, cudaStream_t ss, cudaEvent_t* ev, bool timed, bool generic) {
     const bool fork = ev && ss && ss != s;
     if (fork) {   // the surface kernels first: their blocks take their SMs, the persistent queue fills the rest
         cudaEventRecord(ev[0], s);
@@ -1586,8 +1587,15 @@ void launch_fused(const Mesh& m, const Args& A, cudaStream_t s, cudaStream_t ss,
         Timed t(m, 5, s, 1, timed);
         const int64_t work = Q.n_items + (Q.n_out + 3) / 4;   // warp items
         const int64_t blocks = (work + kFusedWarps - 1) / kFusedWarps;
-        const int64_t grid = std::min<int64_t>(blocks, (int64_t)fused_blocks_per_sm<T, JV>() * m.n_sm);
-        vms_fused<T, JV><<<(unsigned)grid, 32 * kFusedWarps, FusedShape<T>::smem, s>>>(A, Q);
+        auto run = [&](auto kernel, int bps) {
+            kernel<<<(unsigned)std::min<int64_t>(blocks, (int64_t)bps * m.n_sm), 32 * kFusedWarps, FusedShape<T>::smem, s>>>(A, Q);
+        };
+        if constexpr (sizeof(T) == 8) {
+            if (generic) run(vms_fused<T, JV, true>, fused_blocks_per_sm<T, JV, true>());
+            else run(vms_fused<T, JV>, fused_blocks_per_sm<T, JV>());
+        } else {
+            run(vms_fused<T, JV>, fused_blocks_per_sm<T, JV>());
+        }
     }
     if (fork) {
         cudaEventRecord(ev[2], ss);
@@ -1611,8 +1619,8 @@ void launch_all(const Mesh& m, Args A, cudaStream_t s, void* ws = nullptr, cudaS
         Timed t(m, 4, s, (A.n_nodes > 0) + (A.n_hang > 0), !ws);
         launch_node_prep<T, JV>(A, ndv, ndt, ndf, s);
     }
-    if (m.fused && m.d.fq_cnt && !generic) {
-        launch_fused<T, JV>(m, A, s, s_sur, ev, !ws);
+    if (m.fused && m.d.fq_cnt) {
+        launch_fused<T, JV>(m, A, s, s_sur, ev, !ws, generic);
         return;
     }
     // fork: the Intercepted-element and surface kernels run beside the Out-element kernel
@@ -1697,6 +1705,8 @@ int fused_prepare(Mesh& m, std::string& err) {
     m.fq_counts[2] = m.n_sq_sparse;
     fused_blocks_per_sm<double, true>();
     fused_blocks_per_sm<double, false>();
+    fused_blocks_per_sm<double, true, true>();
+    fused_blocks_per_sm<double, false, true>();
     fused_blocks_per_sm<float, true>();
     fused_blocks_per_sm<float, false>();
     return 0;

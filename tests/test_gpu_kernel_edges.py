@@ -297,3 +297,26 @@ def test_mlp_forward_in_place(dev, rows, nin, nout, ldx):
     want = net.forward(X.clone())
     api.check(_lib.load().imga_mlp_forward(net.h, api._ptr(X), ldx, rows, api._ptr(X), api._stream(None)))
     assert torch.equal(X.view(-1)[: rows * nout].view(rows, nout), want)   # the same sums in the same order
+
+
+# ---- a mixed-precision solve's float64 evaluations take the fused launch too where it is switched on ----
+@pytest.mark.parametrize("graphs", [False, True])
+def test_fused_launch_in_mixed_solves(dev, graphs):
+    w = I.small_sphere(4)
+    g = api.Mesh.from_workload(w)
+    u0, up, _ = I.state(g.n_nodes, 4)
+    kw = dict(precision=api.PRECISION_MIXED, precond=1, max_newton=2, raise_on_failure=False)
+    u = [T(u0, dev) for _ in range(2)]
+    st = [None, None]
+    for fused in (False, True):
+        g.fused(fused)
+        g.use_graphs(graphs)
+        st[fused] = g.newton_step(w.physics, u[fused], T(up, dev), **kw)
+    # the same sums but for the contraction of a last bit, which a solve to 1e-3 per linear step may amplify
+    assert abs(st[0]["krylov_its"] - st[1]["krylov_its"]) <= 2
+    assert float((u[0] - u[1]).norm() / u[0].norm()) <= 1e-5
+    g.profile(True)                                        # (profiled solves are driven from the host)
+    g.newton_step(w.physics, T(u0, dev), T(up, dev), **kw)
+    n = {k: c for k, (_, c) in g.profile_read().items()}
+    g.profile(False)
+    assert n["fused"] > 0 and n["out_elements"] == 0 and n["cut_elements"] == 0
