@@ -432,7 +432,8 @@ imga_status imga_gemm_bf16(int M, int N, int K, const float* A, const float* B, 
  * Eq. (Wpart): the bucket of elements with uneven quadrature counts (8 to 4096 points).  Tuning
  * synchronises the stream, and is skipped inside a stream capture and by imga_jvp_noalloc.  Value 0
  * restores the default shape (4 warps, longest first).  In float64 the warps are those of one element; in
- * mixed precision the kernel for meshes of few Intercepted elements has one shape.  Both values drop the cached graphs. */
+ * mixed precision meshes of at most 16 Intercepted elements per SM have a kernel of one shape (4 warps), timed in
+ * both orders only.  Both values drop the cached graphs. */
 /* IMGA_OPT_CLASSIFY_RAYS (value 1 on, 0 off, default off): imga_classify sends every point to ray
  * parity, skipping the stored markers and the normal test; for the comparison of Table in-out. */
 /* IMGA_OPT_DETERMINISTIC (value 1 on, the default; 0 off): how imga_residual / imga_jvp (and

@@ -1395,6 +1395,8 @@ struct Timed {
     }
 };
 
+bool cut_is_split(const Mesh& m) { return (int64_t)m.cut_list.size() <= (int64_t)kSplitCut * m.n_sm; }   // float32
+
 template <class T, bool JV>
 void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt, bool generic = false) {
     const int64_t nc = (int64_t)m.cut_list.size();
@@ -1405,7 +1407,7 @@ void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt, 
         else vms_cut64<JV, 4><<<(unsigned)nc, 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts, order);
     } else {
         const void* pts = m.d.cut_pts_f;
-        if (nc <= (int64_t)kSplitCut * m.n_sm) {
+        if (cut_is_split(m)) {
             vms_cut_split<T, JV><<<(unsigned)nc, 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order);
             return;
         }
@@ -1443,7 +1445,9 @@ int autotune_cut(Mesh& m, Args A, cudaStream_t s) {
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     float best = 1e30f;
-    for (int wi = 0; wi < nw && nc > 0; ++wi)
+    // (vms_cut_split has one shape, four warps: the others are not measured)
+    const bool split = sizeof(T) == 4 && cut_is_split(m);
+    for (int wi = split ? 1 : 0; wi < (split ? 2 : nw) && nc > 0; ++wi)
         for (int lpt = 0; lpt < 2; ++lpt) {
             launch_cut<T, JV>(m, A, s, wpbs[wi], lpt);
             cudaEventRecord(e0, s);

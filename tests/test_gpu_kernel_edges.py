@@ -320,3 +320,15 @@ def test_fused_launch_in_mixed_solves(dev, graphs):
     n = {k: c for k, (_, c) in g.profile_read().items()}
     g.profile(False)
     assert n["fused"] > 0 and n["out_elements"] == 0 and n["cut_elements"] == 0
+
+
+def test_tuning_reports_the_one_shape_of_few_cut_elements(dev):
+    g, _ = pair(I.icosphere(2, 0.2, C, 1e-3, 5), 4, lmax=1)
+    assert g.info["n_cut"] <= 16 * torch.cuda.get_device_properties(dev).multi_processor_count
+    u, up, v = (T(a, dev) for a in I.state(g.n_nodes, 3))
+    ph = I.Physics(mu=0.01, dt=0.02)
+    want = g.jvp(ph, u, up, v, precision=api.PRECISION_MIXED)
+    g.autotune(True)
+    assert torch.equal(g.jvp(ph, u, up, v, precision=api.PRECISION_MIXED), want)
+    wpb, lpt, ms = g.tuning()[(api.PRECISION_MIXED, "jvp")]
+    assert wpb == 4 and lpt in (0, 1) and min(ms[2:4]) > 0 and ms[:2] + ms[4:] == [0.0] * 4
