@@ -332,3 +332,33 @@ def test_tuning_reports_the_one_shape_of_few_cut_elements(dev):
     assert torch.equal(g.jvp(ph, u, up, v, precision=api.PRECISION_MIXED), want)
     wpb, lpt, ms = g.tuning()[(api.PRECISION_MIXED, "jvp")]
     assert wpb == 4 and lpt in (0, 1) and min(ms[2:4]) > 0 and ms[:2] + ms[4:] == [0.0] * 4
+
+
+# ---- the V-cycle row by row against the oracle's on the exported matrix: rows on both sides of 32,768, and aggregates
+# that fit the rows a block takes at a time (8 or 32), exceed them, and do not divide the row count ----
+@pytest.mark.parametrize("level,aggs", [(6, (3, 9, 20)), (7, (6, 41))])
+def test_vcycle_rows_against_oracle(dev, level, aggs):
+    import scipy.sparse as sp
+    from oracle import sparse as S
+    reg = [I.Region(I.REGION_SPHERE_BAND, level, (*C, 0.1, 0.05))]
+    # (without a body: nodes that only slivers reach have nearly singular blocks, and rows of z of 1e12 hide all others)
+    g = api.Mesh((0.0, 0.0, 0.0), (1.0, 1.0, 1.0), 3, reg, None, 1)
+    n = g.n_nodes
+    assert (n >= 32768) == (level == 7)
+    ph = I.Physics(mu=0.02, dt=0.05)
+    u, up, v = (T(a, dev) for a in I.state(n, 5))
+    ptr, idx = g.bsr_pattern()
+    A = sp.bsr_matrix((g.bsr_assemble(ph, u, up).cpu().numpy(), idx, ptr), shape=(4 * n, 4 * n)).tocsr()
+    r = v.cpu().numpy().reshape(-1)
+    for agg in aggs:
+        levels = S.hierarchy(A, agg_size=agg, coarse_max=16)
+        assert n % agg
+        for prec, tol in ((api.PRECISION_FP64, 1e-9), (api.PRECISION_MIXED, 1e-2)):
+            # float64: as the V-cycle's other test; float32: 6e-8 per operation, some hundred of them in a row, block inverses
+            # of entries up to ~1e2.  Row by row: a row or an aggregate gone wrong is off by about the mean row
+            for sweeps in (1, 2):
+                want = S.vcycle(levels, r, nu=sweeps, omega=0.5)
+                g.multilevel_setup(ph, u, up, precision=prec, agg=agg, coarse_max=16, sweeps=sweeps, omega=0.5)
+                assert list(g.multilevel_info()[0]) == [L["n"] for L in levels]
+                z = g.multilevel_apply(v).cpu().numpy().reshape(-1)
+                assert np.abs(z - want).max() <= tol * np.linalg.norm(want) / np.sqrt(want.size), (agg, prec, sweeps)
