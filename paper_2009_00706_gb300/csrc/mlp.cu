@@ -739,7 +739,7 @@ inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)std::min<int64_t
 // MLP object
 // ------------------------------------------------------------------------------------------
 struct Mlp {
-    int nin, nin_pad, w, nout;
+    int nin, nin_pad, w, nout, n_sm = 1;
     int64_t nparam;
     float* P = nullptr;    // master weights: W1 [w][nin_pad], b1 [w], W2 [w][w], b2 [w], W3 [nout][w], b3 [nout]
     float* G = nullptr;    // gradients, same layout
@@ -800,12 +800,12 @@ static void launch_fused(const Mlp& M, const float* X, int64_t ldx, int64_t n, f
 }
 
 // Rows per CTA: 64 (the weights are read from L2 once per 64 rows) when that still gives two CTAs per SM,
-// fewer for fewer rows, so that the chip has work (9,000 rows: 51 us with 32).  From 64 x 2 x 152 rows on 64; the small tile takes 8
-// warps, deep stages and wide chunks because a CTA is alone on its SM (1,024-row training steps: 61 -> 26 us).
+// fewer for fewer rows, so that the chip has work (9,000 rows: 51 us with 32).  The small tile takes 8 warps, deep
+// stages and wide chunks because a CTA is alone on its SM (1,024-row training steps: 61 -> 26 us).
 template <bool TRAIN>
 static void mlp_fused_rows(const Mlp& M, const float* X, int64_t ldx, int64_t n, float* Y, const MlpTrainIO& io, cudaStream_t s) {
-    if (n >= 64 * 152 * 2) launch_fused<64, 128, 32, 64, 3, TRAIN>(M, X, ldx, n, Y, io, s);
-    else if (n >= 32 * 152) launch_fused<32, 128, 32, 64, 4, TRAIN>(M, X, ldx, n, Y, io, s);
+    if (n >= (int64_t)64 * 2 * M.n_sm) launch_fused<64, 128, 32, 64, 3, TRAIN>(M, X, ldx, n, Y, io, s);
+    else if (n >= (int64_t)32 * M.n_sm) launch_fused<32, 128, 32, 64, 4, TRAIN>(M, X, ldx, n, Y, io, s);
     else launch_fused<16, 256, 64, 128, 4, TRAIN>(M, X, ldx, n, Y, io, s);
 }
 
@@ -870,6 +870,9 @@ int mlp_create(int nin, int width, int nout, uint64_t seed, Mlp** out, std::stri
     M->w = width;
     M->nout = nout;
     M->nparam = M->off(5) + nout;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&M->n_sm, cudaDevAttrMultiProcessorCount, dev);
     std::vector<float> h(M->nparam, 0.f);
     // He-uniform initial weights from SplitMix64 (biases zero)
     uint64_t st = seed * 0x9E3779B97F4A7C15ull + 1;
