@@ -169,17 +169,18 @@ __device__ __forceinline__ void add_diag(const Args& A, int32_t id, const double
         for (int q = 0; q < 16; ++q) atomicAdd(D + 16 * (int64_t)hp[p] + q, w2 * blk[q]);
 }
 
-template <class T> struct JacShape { static constexpr int EPB = 16; };
+constexpr int kOutEpb = 16;   // Out elements per block
 
 // Bound by issue and dependent chains, so no indexed local arrays (the seeds are selected, see seed_fields) and
 // registers for five blocks per SM, 2.8 waves instead of 3.5 on 33.7 k Out elements: an assembly of 43.6 k
 // elements 1,858 -> 1,505 us with the selected seeds here and in jac_cut, 1,450 with the fifth block and the
 // 16-byte accesses below.
-template <class T, int MODE>
-__global__ void __launch_bounds__(8 * JacShape<T>::EPB, sizeof(T) == 4 ? 5 : 1) jac_out(Args A, const int32_t* __restrict__ list, int64_t n,
-                                                                const int32_t* __restrict__ slot, double* __restrict__ K,
-                                                                double* __restrict__ D) {
-    constexpr int EPB = JacShape<T>::EPB;
+template <int MODE>
+__global__ void __launch_bounds__(8 * kOutEpb, 5) jac_out(Args A, const int32_t* __restrict__ list, int64_t n,
+                                                          const int32_t* __restrict__ slot, double* __restrict__ K,
+                                                          double* __restrict__ D) {
+    typedef float T;
+    constexpr int EPB = kOutEpb;
     __shared__ __align__(16) T s_nd[EPB][8][CS];
     // a Gauss point's coefficients, in fours (component i: phi and gradient coefficients), for 16-byte accesses;
     // the strides keep the four elements of a warp, and its points, on different banks
@@ -287,11 +288,12 @@ constexpr int JWPB = 4;   // warps per element of jac_cut
 // An Intercepted element: a block of four warps, lane = sub-cell point (32 at a time), each warp the seeds
 // of two corners.  A warp alone with an element ran its hundreds of points 32 seeds deep while most of the
 // chip had nothing left (7.3 k element sphere, 776 elements: 660 -> 361 us an assembly).
-template <class T, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __restrict__ list,
                                                      const int64_t* __restrict__ off, const void* __restrict__ pts,
                                                      const int32_t* __restrict__ order, const int32_t* __restrict__ slot,
                                                      double* __restrict__ K, double* __restrict__ D) {
+    typedef float T;
     constexpr int NB = 8 / JWPB;                    // corners (of the seeds) per warp
     __shared__ __align__(16) T s_nd[8][CS];
     // a point's coefficients for the four seeds of a corner, in fours (component c: phi and gradient
@@ -407,12 +409,13 @@ __global__ void __launch_bounds__(32 * JWPB) jac_cut(Args A, const int32_t* __re
     }
 }
 
-template <class T, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(128) jac_nitsche(Args A, const int32_t* __restrict__ el,
                                                    const double* __restrict__ xr, const double* __restrict__ nr,
                                                    const double* __restrict__ wr, const double* __restrict__ taub,
                                                    int64_t n, const int32_t* __restrict__ slot, double* __restrict__ K,
                                                    double* __restrict__ D) {
+    typedef float T;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int32_t e = el[i];
@@ -1021,28 +1024,25 @@ __global__ void fill_slots(int64_t n, const int32_t* __restrict__ list, int32_t*
     if (i < n) slot[list[i]] = (int32_t)i;
 }
 
-template <class T, int MODE>
+template <int MODE>
 void launch_jac(const Mesh& m, Args A, const int32_t* slot, double* K, double* D, cudaStream_t s) {
     const int64_t next = m.n_nodes() + m.n_hang();
-    T* ndv = node_workspace<T>(m, nullptr);
+    float* ndv = node_workspace<float>(m, nullptr);
     A.ndv = ndv;
     A.ndt = ndv + 8 * next;
     A.ndf = A.F ? ndv + 16 * next : nullptr;
     if (next > 0)
-        launch_node_prep<T, false>(A, ndv, ndv + 8 * next, (T*)A.ndf, s);
+        launch_node_prep<float, false>(A, ndv, ndv + 8 * next, (float*)A.ndf, s);
     const int64_t no = (int64_t)m.out_list.size(), nc = (int64_t)m.cut_list.size(), ns = (int64_t)m.sq.size() / 10;
-    constexpr int EPB = JacShape<T>::EPB;
+    constexpr int EPB = kOutEpb;
     JacFork f(m, s, MODE == FULL);
-    if (no > 0) jac_out<T, MODE><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, slot, K, D);
-    if (nc > 0) {
-        const void* pts = sizeof(T) == 4 ? (const void*)m.d.cut_pts_f : (const void*)m.d.cut_pts;
-        jac_cut<T, MODE><<<(unsigned)nc, 32 * JWPB, 0, f.cut>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order,
-                                                                               slot, K, D);
-    }
+    if (no > 0) jac_out<MODE><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, slot, K, D);
+    if (nc > 0)
+        jac_cut<MODE><<<(unsigned)nc, 32 * JWPB, 0, f.cut>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts_f, m.d.cut_order, slot, K, D);
     f.join();
     if (ns > 0)
-        jac_nitsche<T, MODE><<<(unsigned)((ns + 31) / 32), 32, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w,
-                                                                        m.d.sq_taub, ns, slot, K, D);
+        jac_nitsche<MODE><<<(unsigned)((ns + 31) / 32), 32, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w, m.d.sq_taub, ns,
+                                                                    slot, K, D);
 }
 
 // k_e of the surface terms (one per host element, slot order) added to the assembled matrix
@@ -1084,29 +1084,25 @@ __global__ void bsr_strong_rows(int64_t nn, const int64_t* __restrict__ ptr, con
             }
 }
 
-template <class T>
 void launch_bsr_assembly(const Mesh& m, Args A, double* val, double* Ks, cudaStream_t s) {
     const int64_t next = m.n_nodes() + m.n_hang();
-    T* ndv = node_workspace<T>(m, nullptr);
+    float* ndv = node_workspace<float>(m, nullptr);
     A.ndv = ndv;
     A.ndt = ndv + 8 * next;
     A.ndf = A.F ? ndv + 16 * next : nullptr;
-    if (next > 0) launch_node_prep<T, false>(A, ndv, ndv + 8 * next, (T*)A.ndf, s);
+    if (next > 0) launch_node_prep<float, false>(A, ndv, ndv + 8 * next, (float*)A.ndf, s);
     const int64_t no = (int64_t)m.out_list.size(), nc = (int64_t)m.cut_list.size(), ns = (int64_t)m.sq.size() / 10;
     const int64_t nh = (int64_t)m.sq_hosts.size();
-    constexpr int EPB = JacShape<T>::EPB;
-    if (no > 0) jac_out<T, BSR><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, nullptr, val, nullptr);
-    if (nc > 0) {
-        const void* pts = sizeof(T) == 4 ? (const void*)m.d.cut_pts_f : (const void*)m.d.cut_pts;
-        jac_cut<T, BSR><<<(unsigned)nc, 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, m.d.cut_order,
-                                                                              nullptr, val, nullptr);
-    }
+    constexpr int EPB = kOutEpb;
+    if (no > 0) jac_out<BSR><<<(unsigned)((no + EPB - 1) / EPB), 8 * EPB, 0, s>>>(A, m.d.out_list, no, nullptr, val, nullptr);
+    if (nc > 0)
+        jac_cut<BSR><<<(unsigned)nc, 32 * JWPB, 0, s>>>(A, m.d.cut_list, m.d.cut_off, m.d.cut_pts_f, m.d.cut_order, nullptr, val, nullptr);
     if (ns > 0 && nh > 0) {
         cudaMemsetAsync(m.d.slot, 0xff, (size_t)m.n_elem() * sizeof(int32_t), s);
         fill_slots<<<(unsigned)((nh + 255) / 256), 256, 0, s>>>(nh, m.d.sq_hosts, m.d.slot);
         cudaMemsetAsync(Ks, 0, (size_t)nh * 1024 * sizeof(double), s);
-        jac_nitsche<T, FULL><<<(unsigned)((ns + 31) / 32), 32, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w,
-                                                                        m.d.sq_taub, ns, m.d.slot, Ks, nullptr);
+        jac_nitsche<FULL><<<(unsigned)((ns + 31) / 32), 32, 0, s>>>(A, m.d.sq_elem, m.d.sq_x, m.d.sq_n, m.d.sq_w, m.d.sq_taub, ns,
+                                                                    m.d.slot, Ks, nullptr);
         scatter_kmat<<<(unsigned)((nh * 256 + 255) / 256), 256, 0, s>>>(A, m.d.sq_hosts, nh, Ks, val);
     }
 }
@@ -1126,7 +1122,7 @@ int bsr_assemble(const Mesh& m, const double* u, const double* up, const double*
     A.bidx = bidx;
     cudaMemsetAsync(val, 0, (size_t)nb * 16 * sizeof(double), s);
     if (precision == 0) launch_jac64<BSR>(m, A, nullptr, 0, nullptr, val, nullptr, s);
-    else launch_bsr_assembly<float>(m, A, val, Ks, s);
+    else launch_bsr_assembly(m, A, val, Ks, s);
     if (nn > 0)
         bsr_strong_rows<<<(unsigned)((8 * nn + 255) / 256), 256, 0, s>>>(nn, bptr, bidx, m.d.bcflag,
                                                                     m.user_bc ? m.d.bcmask_user : nullptr, val);
@@ -1143,7 +1139,7 @@ int element_jacobians(const Mesh& m, const double* u, const double* up, const do
     fill_slots<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, elems, slot);
     cudaMemsetAsync(K, 0, (size_t)n * 1024 * sizeof(double), s);
     if (precision == 0) launch_jac64<FULL>(m, A, elems, n, slot, K, nullptr, s);
-    else launch_jac<float, FULL>(m, A, slot, K, nullptr, s);
+    else launch_jac<FULL>(m, A, slot, K, nullptr, s);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
@@ -1154,7 +1150,7 @@ int block_jacobi_setup(const Mesh& m, const double* u, const double* up, const d
     Args A = make_args(m, u, up, up2, f, ph, nullptr, nullptr);
     cudaMemsetAsync(D, 0, (size_t)nn * 16 * sizeof(double), s);
     if (precision == 0) launch_jac64<DIAG>(m, A, nullptr, 0, nullptr, nullptr, D, s);
-    else launch_jac<float, DIAG>(m, A, nullptr, nullptr, D, s);
+    else launch_jac<DIAG>(m, A, nullptr, nullptr, D, s);
     if (nn > 0) {
         jac_strong_rows<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(nn, m.d.bcflag, m.user_bc ? m.d.bcmask_user : nullptr, D);
         bj_invert<<<(unsigned)((nn + 127) / 128), 128, 0, s>>>(nn, D, Dinv);

@@ -701,19 +701,19 @@ __device__ __forceinline__ void cut_element64(const Args& A, const int32_t* __re
     cut_rows64(A, e, idx, acc, lane);
 }
 
-// W warps per block (a tile shape the autotuner picks); `order` (or null) permutes the list
-template <class T, bool JV, int W>
+// float32: W warps per block (a tile shape the autotuner picks); `order` (or null) permutes the list
+template <bool JV, int W>
 __global__ void __launch_bounds__(32 * W, 16 / W) vms_cut(Args A, const int32_t* __restrict__ list,
                                                     const int64_t* __restrict__ off, const void* __restrict__ pts,
                                                     const int32_t* __restrict__ order, int64_t n) {
-    constexpr int PAD = 16 / (int)sizeof(T), MSTR = 32 + PAD;
-    __shared__ __align__(16) T s_nd[W][8 * CS];
-    __shared__ __align__(16) T s_m[W][32 * MSTR];
+    constexpr int MSTR = 36;
+    __shared__ __align__(16) float s_nd[W][8 * CS];
+    __shared__ __align__(16) float s_m[W][32 * MSTR];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t slot = (int64_t)blockIdx.x * W + w;
     if (A.skip && *A.skip) return;   // a captured solver step after its cycle ended
     if (slot >= n) return;
-    cut_element<T, JV>(A, list, off, pts, order ? (int64_t)order[slot] : slot, &s_nd[w][0], &s_m[w][0], lane);
+    cut_element<float, JV>(A, list, off, pts, order ? (int64_t)order[slot] : slot, &s_nd[w][0], &s_m[w][0], lane);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1412,9 +1412,9 @@ void launch_cut(const Mesh& m, const Args& A, cudaStream_t s, int wpb, int lpt, 
             return;
         }
         switch (wpb) {
-            case 2: vms_cut<T, JV, 2><<<(unsigned)((nc + 1) / 2), 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
-            case 8: vms_cut<T, JV, 8><<<(unsigned)((nc + 7) / 8), 256, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
-            default: vms_cut<T, JV, 4><<<(unsigned)((nc + 3) / 4), 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc);
+            case 2: vms_cut<JV, 2><<<(unsigned)((nc + 1) / 2), 64, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
+            case 8: vms_cut<JV, 8><<<(unsigned)((nc + 7) / 8), 256, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc); break;
+            default: vms_cut<JV, 4><<<(unsigned)((nc + 3) / 4), 128, 0, s>>>(A, m.d.cut_list, m.d.cut_off, pts, order, nc);
         }
     }
 }
