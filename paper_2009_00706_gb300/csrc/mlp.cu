@@ -746,7 +746,7 @@ struct Mlp {
     float* Mm = nullptr;   // Adam moments
     float* Vm = nullptr;
     bf16* Pb = nullptr;    // bf16 copy of the weights
-    int64_t cap = 0;       // batch capacity of the activation buffers
+    int64_t cap = 0, cap_general = 0;   // batch capacity of the activation buffers
     bf16 *xb = nullptr, *h1 = nullptr, *h2 = nullptr, *dyb = nullptr, *dz2 = nullptr, *dz1 = nullptr;
     float *z1 = nullptr, *z2 = nullptr, *y = nullptr, *dh2 = nullptr, *dh1 = nullptr;
     double* loss = nullptr;
@@ -759,29 +759,33 @@ struct Mlp {
     }
 };
 
-static bool mlp_reserve(Mlp& M, int64_t b) {
-    if (b <= M.cap) return true;
-    cudaFree(M.xb); cudaFree(M.h1); cudaFree(M.h2); cudaFree(M.dyb); cudaFree(M.dz2); cudaFree(M.dz1);
-    cudaFree(M.z1); cudaFree(M.z2); cudaFree(M.y); cudaFree(M.dh2); cudaFree(M.dh1);
-    bool ok = cudaMalloc((void**)&M.xb, b * M.nin_pad * sizeof(bf16)) == cudaSuccess &&
-              cudaMalloc((void**)&M.h1, b * M.w * sizeof(bf16)) == cudaSuccess &&
-              cudaMalloc((void**)&M.h2, b * M.w * sizeof(bf16)) == cudaSuccess &&
-              cudaMalloc((void**)&M.dyb, b * M.nout * sizeof(bf16)) == cudaSuccess &&
-              cudaMalloc((void**)&M.dz2, b * M.w * sizeof(bf16)) == cudaSuccess &&
-              cudaMalloc((void**)&M.dz1, b * M.w * sizeof(bf16)) == cudaSuccess &&
-              cudaMalloc((void**)&M.z1, b * M.w * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&M.z2, b * M.w * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&M.y, b * M.nout * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&M.dh2, b * M.w * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&M.dh1, b * M.w * sizeof(float)) == cudaSuccess;
-    M.cap = ok ? b : 0;
-    return ok;
+template <class T> static bool grow(T*& p, int64_t n) {
+    cudaFree(p);
+    p = nullptr;
+    return cudaMalloc((void**)&p, n * sizeof(T)) == cudaSuccess;
+}
+
+// buffers for batches of b rows: those that every path keeps between its kernels, and those of the general path alone
+static bool mlp_reserve(Mlp& M, int64_t b, bool general) {
+    if (b > M.cap) {
+        const bool ok = grow(M.xb, b * M.nin_pad) && grow(M.h1, b * M.w) && grow(M.h2, b * M.w) && grow(M.dyb, b * M.nout) &&
+                        grow(M.dz2, b * M.w) && grow(M.dz1, b * M.w);
+        M.cap = ok ? b : 0;
+        if (!ok) return false;
+    }
+    if (general && b > M.cap_general) {
+        const bool ok = grow(M.z1, b * M.w) && grow(M.z2, b * M.w) && grow(M.y, b * M.nout) && grow(M.dh2, b * M.w) && grow(M.dh1, b * M.w);
+        M.cap_general = ok ? b : 0;
+        if (!ok) return false;
+    }
+    return true;
 }
 
 static void mlp_sync_bf16(Mlp& M, cudaStream_t s) { to_bf16<<<nblk(M.nparam), 256, 0, s>>>(M.nparam, M.P, M.Pb); }
 
 // The fused kernels serve the preconditioner's width; rows of 16 bytes in every bf16 matrix need nout % 8 == 0.
-static bool mlp_fast(const Mlp& M) { return M.w == kW && M.nout % 8 == 0; }
+// Targets are read and results written in pairs.
+static bool mlp_fast(const Mlp& M, const float* pairs) { return M.w == kW && M.nout % 8 == 0 && ((uintptr_t)pairs & 7) == 0; }
 
 template <int BM, int NT, int KT, int NC, int STAGES, bool TRAIN>
 static void launch_fused(const Mlp& M, const float* X, int64_t ldx, int64_t n, float* Y, const MlpTrainIO& io, cudaStream_t s) {
@@ -856,9 +860,9 @@ static void mlp_backward_batch(Mlp& M, const float* T, int64_t b, double n_total
     col_sum<<<(M.w + 127) / 128, 128, 0, s>>>(b, M.w, M.dz1, M.G + M.off(1), beta != 0.f);
 }
 
-// forward and gradient of a batch (targets read in pairs on the fused path)
+// forward and gradient of a batch
 static void mlp_step(Mlp& M, const float* X, int64_t ldx, const float* T, int64_t b, double n_total, float beta, cudaStream_t s) {
-    if (mlp_fast(M) && ((uintptr_t)T & 7) == 0) { mlp_step_fused(M, X, ldx, T, b, n_total, beta, s); return; }
+    if (mlp_fast(M, T)) { mlp_step_fused(M, X, ldx, T, b, n_total, beta, s); return; }
     mlp_forward_batch(M, X, ldx, b, s);
     mlp_backward_batch(M, T, b, n_total, beta, s);
 }
@@ -934,11 +938,11 @@ int mlp_forward(Mlp* M, const float* X, int64_t ldx, int64_t n, float* Y, cudaSt
     const int64_t B = 4096;
     // (in place, or overlapping otherwise: batch by batch, each read whole before its results are written)
     const bool apart = (uintptr_t)(Y + n * M->nout) <= (uintptr_t)X || (uintptr_t)(X + (n - 1) * ldx + M->nin) <= (uintptr_t)Y;
-    if (mlp_fast(*M) && ((uintptr_t)Y & 7) == 0 && (apart || n == 0)) {
+    if (mlp_fast(*M, Y) && (apart || n == 0)) {
         if (n > 0) mlp_fused_rows<false>(*M, X, ldx, n, Y, MlpTrainIO{}, s);
         return cudaGetLastError() == cudaSuccess ? 0 : 1;
     }
-    if (!mlp_reserve(*M, std::min(n, B))) return 1;
+    if (!mlp_reserve(*M, std::min(n, B), true)) return 1;
     for (int64_t r = 0; r < n; r += B) {
         const int64_t b = std::min(B, n - r);
         mlp_forward_batch(*M, X + r * ldx, ldx, b, s);
@@ -950,7 +954,7 @@ int mlp_forward(Mlp* M, const float* X, int64_t ldx, int64_t n, float* Y, cudaSt
 // gradient of the mean loss over all n samples (one pass, no update); returns the loss
 int mlp_gradient(Mlp* M, const float* X, int64_t ldx, const float* T, int64_t n, double* loss, cudaStream_t s) {
     const int64_t B = 4096;
-    if (!mlp_reserve(*M, std::min(n, B))) return 1;
+    if (!mlp_reserve(*M, std::min(n, B), !mlp_fast(*M, T))) return 1;
     cudaMemsetAsync(M->loss, 0, 8, s);
     for (int64_t r = 0; r < n; r += B) {
         const int64_t b = std::min(B, n - r);
@@ -966,7 +970,7 @@ int mlp_gradient(Mlp* M, const float* X, int64_t ldx, const float* T, int64_t n,
 // Adam over shuffled-free mini-batches; loss_hist[e] = mean training loss of epoch e
 int mlp_train(Mlp* M, const float* X, int64_t ldx, const float* T, int64_t n, int epochs, int batch, float lr,
               double* loss_hist, cudaStream_t s) {
-    if (!mlp_reserve(*M, std::min<int64_t>(n, batch))) return 1;
+    if (!mlp_reserve(*M, std::min<int64_t>(n, batch), !mlp_fast(*M, T))) return 1;
     for (int ep = 0; ep < epochs; ++ep) {
         cudaMemsetAsync(M->loss, 0, 8, s);
         for (int64_t r = 0; r < n; r += batch) {

@@ -362,3 +362,17 @@ def test_vcycle_rows_against_oracle(dev, level, aggs):
                 assert list(g.multilevel_info()[0]) == [L["n"] for L in levels]
                 z = g.multilevel_apply(v).cpu().numpy().reshape(-1)
                 assert np.abs(z - want).max() <= tol * np.linalg.norm(want) / np.sqrt(want.size), (agg, prec, sweeps)
+
+
+# ---- targets at a 4-byte address take the general path, whose own buffers grow when it is first taken ----
+def test_mlp_general_path_after_the_fused_one(dev):
+    net = api.Mlp(seed=2)
+    torch.manual_seed(0)
+    X, Y = torch.randn(1500, 1040, device=dev), torch.randn(1500, 1024, device=dev)
+    odd = torch.empty(1500 * 1024 + 1, device=dev)[1:].view(1500, 1024).copy_(Y)
+    assert odd.data_ptr() % 8 == 4
+    for rows in (100, 1500, 700):
+        l1, g1 = net.gradient(X[:rows], Y[:rows])
+        l2, g2 = net.gradient(X[:rows], odd[:rows])
+        # the same products in the same order; a bf16 mask or a float32 sum may fall otherwise at most
+        assert abs(l1 - l2) <= 1e-12 * l1 and np.linalg.norm(g1 - g2) <= 1e-5 * np.linalg.norm(g1)
