@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(32 * J64W, 2) jac_out64(Args A, const int32_t*
     if (mine >= 0) {
         const int lv = A.lev[mine];
         const Const64 C(A, Phys<double>(A, prob_of(A, mine)), lv, A.lc[lv][0], A.lc[lv][1]);
-        const double gam = 1.0 / kInvGauss;
+        const double gam = kGauss;
         jac_point64(A, C, s_col + 96 * le, (lane & 1) ? gam : -gam, (lane & 2) ? gam : -gam, (lane & 4) ? gam : -gam,
                     A.lc[lv][6], s + lane);
     }

@@ -79,7 +79,7 @@ template <class T> struct IntShape {
 template <bool JV>
 __device__ __forceinline__ void interior_element64(const Args& A, const double* nd, double* sw, int lane, int64_t idx,
                                                    bool valid, int lv, int prob, int32_t id) {
-    constexpr double gam = 1.0 / kInvGauss;
+    constexpr double gam = kGauss;
     const int c = lane & 7;
     double* E = sw + (lane >> 3) * 272;   // V [8 columns][8], GX | GY | GZ [8][4], XY | XZ | YZ [8][2]
     __syncwarp();

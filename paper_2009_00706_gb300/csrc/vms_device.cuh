@@ -88,7 +88,10 @@ template <class T, int K> __device__ __forceinline__ Dual<T, K> rcp(Dual<T, K> x
     return {r, -r * r * x.d};
 }
 
-constexpr double kInvGauss = 1.73205080756887729353;   // sqrt(3): 1 / Gauss abscissa
+// Gauss abscissa 1/sqrt(3), and its inverse by which the test sums leave it out of S and H: the inverse of the rounded
+// abscissa, so that their product is 1 to 1.2e-17.  (The other way round, 1 / sqrt(3) in float64 is the abscissa's
+// neighbour, 1.3e-16 off: float64 J v was 1.4 to 1.6 times as far from quad precision, all of it bias.)
+constexpr double kGauss = 0.57735026918962576451, kInvGauss = 1.0 / kGauss;
 
 template <class T> __device__ __forceinline__ T tiny();
 template <> __device__ __forceinline__ float tiny<float>() { return 1e-37f; }

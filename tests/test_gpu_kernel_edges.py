@@ -376,3 +376,67 @@ def test_mlp_general_path_after_the_fused_one(dev):
         l2, g2 = net.gradient(X[:rows], odd[:rows])
         # the same products in the same order; a bf16 mask or a float32 sum may fall otherwise at most
         assert abs(l1 - l2) <= 1e-12 * l1 and np.linalg.norm(g1 - g2) <= 1e-5 * np.linalg.norm(g1)
+
+
+# ---- the float64 Out elements' Gauss abscissa is the correctly rounded one.  At u = 0 on a uniform mesh the momentum rows
+# of J v are c0 rho M + mu (K + K') + rho tau_C (grad div) in closed form; the abscissa enters through the 1D mass
+# matrix h/4 [[1 + g^2, 1 - g^2], [1 - g^2, 1 + g^2]].  Its relative error is what the error of J v has along dJ/dg: a fit
+# over 10^4 entries, whose own roundings (1e-16 each, of either sign) move it by about 1e-18 ----
+def _uniform_momentum(v, h, c0, mu, tauC, g2):
+    L = np.longdouble
+
+    def st(x, ax, lo, mid, hi):
+        return lo * x.take(range(0, x.shape[ax] - 2), ax) + mid * x.take(range(1, x.shape[ax] - 1), ax) + hi * x.take(range(2, x.shape[ax]), ax)
+    M = lambda x, ax: st(x, ax, h / 4 * (1 - g2), h / 2 * (1 + g2), h / 4 * (1 - g2))
+    K = lambda x, ax: st(x, ax, -1 / h, 2 / h, -1 / h)
+    D = lambda x, ax: st(x, ax, L(-0.5), L(0), L(0.5))        # test value, trial derivative; the transpose is -D
+    mass, visc, gd = [], [], []
+    for i in range(3):
+        m = v[..., i]
+        for ax in range(3):
+            m = M(m, ax)
+        mass.append(c0 * m)
+        vi, gi = 0, 0
+        for j in range(3):
+            k = v[..., i]
+            for ax in range(3):
+                k = K(k, ax) if ax == j else M(k, ax)
+            vi = vi + k
+            x = v[..., j]
+            for ax in range(3):                                  # d_i w d_j v_j and d_j w d_i v_j: the same for i != j, both -D D
+                x = K(x, ax) if i == j == ax else -D(x, ax) if ax == i else D(x, ax) if ax == j else M(x, ax)
+            gi = gi + x
+            vi = vi + x
+        visc.append(mu * vi)
+        gd.append(tauC * gi)
+    return [np.stack(q, -1) for q in (mass, visc, gd)]
+
+
+def test_float64_gauss_abscissa(dev):
+    L, lev = np.longdouble, 4
+    n, h, dt, mu = 2 ** lev + 1, 2.0 ** -lev, 2.0 ** -7, 2.0 ** -6
+    g = api.Mesh((0.0, 0.0, 0.0), (1.0, 1.0, 1.0), lev, [], None, 1)
+    assert g.n_nodes == n ** 3
+    at = tuple((g.export()["node_ijk"].astype(np.int64) >> (20 - lev)).T)
+    v = I.state(g.n_nodes, 7)[2].copy()
+    v[:, 3] = 0
+    z = torch.zeros(g.n_nodes, 4, dtype=torch.float64, device=dev)
+    ph = I.Physics(mu=mu, dt=dt)
+    Jv = g.jvp(ph, z, z, T(v, dev)).cpu().numpy()
+    grid = np.zeros((n, n, n, 3), L)
+    got = np.zeros((n, n, n, 3), L)
+    grid[at], got[at] = v[:, :3], Jv[:, :3]
+    got = got[1:-1, 1:-1, 1:-1]
+    g2 = L(2) / L(h)
+    g2 = g2 * g2
+    tauM = 1 / np.sqrt(4 / L(dt) ** 2 + 3 * L(ph.CI) * L(mu) ** 2 * g2 * g2)
+    args = (grid, L(h), 1 / L(dt), L(mu), 1 / (3 * g2 * tauM))
+    third, e = 1 / L(3), L(2) ** -20
+    parts = _uniform_momentum(*args, third)
+    b = (sum(_uniform_momentum(*args, third * (1 + e) ** 2)) - sum(_uniform_momentum(*args, third * (1 - e) ** 2))) / (2 * e)
+    err = got - sum(parts)
+    assert float(np.abs(err).max() / np.abs(sum(parts)).max()) < 1e-14           # the closed form is the operator
+    # (the three parts may each have a constant of their own rounding: tau_C, and the scale of the stresses)
+    fit = np.linalg.lstsq(np.stack([np.asarray(x, np.float64).ravel() for x in (b, *parts)], 1), np.asarray(err, np.float64).ravel(), rcond=None)[0]
+    print("relative error of the abscissa", fit[0])
+    assert abs(fit[0]) <= 2.0 ** -53                                              # correctly rounded
