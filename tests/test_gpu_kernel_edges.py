@@ -440,3 +440,28 @@ def test_float64_gauss_abscissa(dev):
     fit = np.linalg.lstsq(np.stack([np.asarray(x, np.float64).ravel() for x in (b, *parts)], 1), np.asarray(err, np.float64).ravel(), rcond=None)[0]
     print("relative error of the abscissa", fit[0])
     assert abs(fit[0]) <= 2.0 ** -53                                              # correctly rounded
+
+
+# ---- the block-Jacobi blocks themselves: the first Krylov vector of a solve from b is D^-1 b, so one Krylov iteration of
+# one Newton step moves u along it.  Without hanging nodes D is the diagonal of the assembled matrix ----
+@pytest.mark.parametrize("prec,tol", [(api.PRECISION_FP64, 1e-10), (api.PRECISION_MIXED, 1e-3)])
+def test_block_jacobi_blocks(dev, prec, tol):
+    g = api.Mesh((0.0, 0.0, 0.0), (1.0, 1.0, 1.0), 4, [], I.icosphere(2, 0.2, C, 1e-3, 3), 2)
+    assert g.n_hang == 0 and g.info["n_cut"] > 0 and g.info["n_surface_points"] > 0
+    ph = I.Physics(mu=0.02, dt=0.05)
+    u0, up = (T(a, dev) for a in I.state(g.n_nodes, 5)[:2])
+    b = -g.residual(ph, u0, up)
+    u = u0.clone()
+    g.newton_step(ph, u, up, precision=prec, precond=1, max_newton=1, max_krylov=1, line_search=0, raise_on_failure=False)
+    ptr, idx = g.bsr_pattern()
+    rows = np.repeat(np.arange(g.n_nodes), np.diff(ptr))
+    D = g.bsr_assemble(ph, u0, up)[torch.from_numpy(np.flatnonzero(rows == idx)).to(dev)]
+    # D du = s b node by node, s the step along D^-1 b; a node of slivers alone may have no usable block (then the identity)
+    x = torch.einsum("nij,nj->ni", D, u - u0)
+    s = float((x * b).sum() / (b * b).sum())
+    usable = torch.linalg.svdvals(D)[:, -1] > 1e-8 * D.abs().amax((1, 2))
+    assert float(usable.double().mean()) > 0.95 and s != 0
+    scale = torch.einsum("nij,nj->ni", D.abs(), (u - u0).abs()).amax(1) + abs(s) * b.abs().amax(1) + 1e-300
+    off = (x - s * b).abs().amax(1) / scale
+    # float64: an inverse and a product of 4 x 4 blocks; float32 element arithmetic: 6e-8 per operation, some hundred of them
+    assert float(off[usable].max()) <= tol
