@@ -36,3 +36,22 @@ def test_clock_summary_reads_only_the_timed_window(tmp_path):
     c.marks = [len(before), len(before)]
     s = c.summary()
     assert s["samples"] == 1 and s["sm_mhz"] == 2070 and s["window"].startswith("timed region shorter")
+
+
+def test_headline_is_short_and_complete():
+    """The result line keeps every required key and stays small however long the tables get."""
+    import json
+
+    import bench
+    roof = {"kernel": "k", "bound": "alu", "achieved": 1.0, "peak": 2.0, "unit": "TFLOP/s", "frac": 0.5, "traffic": 1,
+            "peaks": {"a": 1.0}, "timing": "t" * 300, "alone": {"frac": 0.6, "avg_launch_ms": 1.0}, "executed": {"frac": 0.4}}
+    line = {k: "x" for k in bench.HEADLINE}
+    line.update(roofline=roof, newton_step={"mixed": {"ms": 3.0, "workload": "w" * 500}, "levels": [1, 2]},
+                inout={"table": ["y" * 50] * 400}, batched={"z": 1})
+    short, rest = bench.headline(line)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+              "dtype", "data", "config", "clocks", "e2e", "gpu_launches"):
+        assert short[k] == "x"
+    assert short["roofline"]["frac"] == 0.5 and short["roofline"]["alone_frac"] == 0.6 and short["newton_ms"] == {"mixed": 3.0}
+    assert len(json.dumps(short)) < 4096
+    assert rest["details"]["inout"] == line["inout"] and rest["details"]["roofline"] == roof and "metric" not in rest["details"]
