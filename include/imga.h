@@ -463,7 +463,8 @@ imga_status imga_gemm_bf16(int M, int N, int K, const float* A, const float* B, 
  * preparation and joined before the node sums, so they run beside the Out-element kernel (direct
  * calls and captured graphs alike).  Off: every kernel on the caller's stream, one after the other
  * (each kernel then runs alone, e.g. to time it).  The results are the same bit for bit with
- * IMGA_OPT_DETERMINISTIC. */
+ * IMGA_OPT_DETERMINISTIC.  imga_element_jacobians likewise launches the Intercepted elements' kernel on a side stream
+ * beside the Out elements' where it is not captured (every matrix has one writer: the same results). */
 enum { IMGA_OPT_GRAPHS = 1, IMGA_OPT_AUTOTUNE = 2, IMGA_OPT_CLASSIFY_RAYS = 3, IMGA_OPT_DETERMINISTIC = 4, IMGA_OPT_FUSED = 5,
        IMGA_OPT_FUSED_SPLIT = 6, IMGA_OPT_CONCURRENT = 7 };
 imga_status imga_set_option(imga_mesh mesh, int option, int64_t value);

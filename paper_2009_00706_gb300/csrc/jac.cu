@@ -171,8 +171,9 @@ __device__ __forceinline__ void add_diag(const Args& A, int32_t id, const double
 
 constexpr int kOutEpb = 16;   // Out elements per block
 
-// Bound by issue and dependent chains, so no indexed local arrays (the seeds are selected, see seed_fields) and
-// registers for five blocks per SM, 2.8 waves instead of 3.5 on 33.7 k Out elements: an assembly of 43.6 k
+// Bound by issue and dependent chains.  The seeds are selected (see seed_fields), as an indexed store would put 240
+// bytes per thread in local memory; only the diagonal form keeps an array there (144 bytes of stack).  Registers for
+// five blocks per SM (8 to 40 bytes of spills): 2.8 waves instead of 3.5 on 33.7 k Out elements.  An assembly of 43.6 k
 // elements 1,858 -> 1,505 us with the selected seeds here and in jac_cut, 1,450 with the fifth block and the
 // 16-byte accesses below.
 template <int MODE>
@@ -477,7 +478,7 @@ __global__ void __launch_bounds__(128) jac_nitsche(Args A, const int32_t* __rest
 //   jac_out64   four Out elements per warp: 4 x 8 Gauss points at once, then the elements in turn
 //   jac_cut64   a block of four warps per Intercepted element, 32 sub-cell points per warp at a time
 //   jac_surf64  a warp per element hosting surface points: no atomics between its points
-// 8,192 of 27 k elements (a ninth of them Intercepted, 288 points each): 35.8 -> 4.5 ms.
+// 8,192 of 33.7 k elements (a ninth of them Intercepted, 288 points each): 35.8 -> 4.5 ms.
 // ------------------------------------------------------------------------------------------
 enum { JX = 0, JU = 3, JG = 6, JUP = 15, JGU = 18, JC = 21, JA = 24, JQ = 27, JDIV = 31, JS = 32, JS2 = 33, JNRR = 34,
        JNRG = 35, JNRM = 36, JMP = 37, JWM = 38, JN = 46 };

@@ -612,7 +612,7 @@ public:
         scale_copy_kernel<<<(unsigned)std::min<int64_t>(4 * M.n_sm, (n + 255) / 256), 256, 0, st>>>(n, a, x, y);
     }
 
-    // float64 evaluations of a mixed-precision solve: the generic element code (kGeneric64 in vms.cu)
+    // float64 evaluations of a mixed-precision solve: the generic element code (generic in vms.cu)
     bool generic64() const { return O.precision != 0; }
 
     int residual(const double* u, double* R) {
@@ -738,8 +738,8 @@ public:
     cudaStream_t cap = nullptr;
 
     // precondition V[k] (vec(4) holds it), J v, CGS2 against V[0..k], Givens update, normalise into V[k+1]:
-    // five launches beside the preconditioner and J v (11 before).  A Newton solve of the 7.3 k
-    // element sphere to 1e-8, with the assembly, the V-cycle and the kernels of J v: 70 -> 35 ms
+    // five launches beside the preconditioner and J v (11 before).  Newton solves of the 7.3 k element sphere to 1e-8
+    // on five surfaces, with the assembly, the V-cycle and the kernels of J v: 63 to 76 -> 32 to 40 ms, the same iterations
     int step_launches(const double* u) {
         GState* G = W.G;
         double* vk = vec(4);

@@ -58,12 +58,14 @@ template <class T> struct IntShape {
     static constexpr size_t smem = (size_t)(2 * EPB * ESTR + EPB * 8 * MSTR) * sizeof(T);
 };
 
-// kGeneric64: the residual and J v of a mixed-precision solve run their float64 evaluations on the generic
-// element code, with the roundings it has always had.  Such a solve turns the last bit of a residual into
-// float32 steps of its preconditioner and matvecs, and those into differences as large as its tolerance
-// (1e-9 to 1e-7 of u at 1e-8), so other roundings there would make other solutions, no nearer and no
-// further from the root.  It costs a solve of the 7.3 k element sphere 1.5 of 35 ms.  Everything else,
-// float64 solves included, takes the kernels below.
+// generic / GEN: the float64 evaluations of a mixed-precision solve (its residuals and the J v of its restarts) run
+// their volume kernels on the generic element code instead of the ones below.  Such a solve turns the last bit of a
+// residual into float32 steps of its preconditioner and matvecs, and those into differences as large as its
+// tolerance (1e-9 to 1e-7 of u at 1e-8): with other roundings it would end at another solution, no nearer and no
+// further from the root.  So this keeps the solutions that a given mesh and state have had; it is no matter of
+// accuracy, and such a residual differs in its last bits from the one imga_residual returns.  It costs a solve of the
+// 7.3 k element sphere 1.5 of 35 ms; at 2.0 M elements a float64 J v of the Out elements takes 20.7 ms this way, 11.2 by
+// interior_element64.  (The penalty with a velocity per surface point has one kernel for all callers.)
 //
 // One Out element in float64 on 8 lanes of a warp (c = lane & 7); nd its 8 corner rows, sw the warp's
 // 4 x 272 doubles.  FP64 instructions are the cost (see Const64), so the work goes to lanes by what
@@ -321,7 +323,7 @@ __device__ __forceinline__ void gauss_monomials(int c, T m[8]) {
 // group's 16 elements (interior_element).
 // MINB: resident blocks per SM the register allocation is made for (4: up to 128 registers per thread;
 // 5: up to 102, a few spills, one more block of warps to hide latency with)
-// GEN: float64 elements by the code of the float32 ones (see kGeneric64)
+// GEN: float64 elements by the code of the float32 ones (see generic / GEN above)
 template <class T, bool JV, int MINB = (sizeof(T) == 4 ? 4 : 2), bool GEN = false>
 __global__ void __launch_bounds__(IntShape<T>::THREADS, MINB) vms_interior(Args A, const int32_t* __restrict__ oconn,
                                                     const uint8_t* __restrict__ olev,
