@@ -136,51 +136,11 @@ __device__ __forceinline__ uint32_t cvt2(float lo, float hi) {   // one conversi
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// A thread's sum of squares, no less exact than a float64 one: the square is exact in two floats, and the sum is
-// kept in three (TwoSum: hi + mid exactly what was added but for mid's own rounding errors, which lo adds up), 72 bits
-// against 53.  Where a value's square or its low part leaves the float32 range (below 2^-51, from 2^58 on, inf, NaN)
-// the N values go to a float64 sum.  One float64 multiply-add per value instead cost a training step of 1,024 rows 6 of 79 us:
-// the FP64 pipe takes a warp's instruction every 19 cycles and 64 of the SMs had all of them.
-struct SquareSum {
-    float hi = 0.f, mid = 0.f, lo = 0.f;
-    double wide = 0.0;
-    static __device__ __forceinline__ float two_sum(float& s, float x) {   // s += x, the rounding error returned
-        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s), e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
-        s = t;
-        return e;
-    }
-    template <int N> __device__ __forceinline__ void add(const float* d) {
-        constexpr uint32_t least = (127u - 51u) << 23, end = (127u + 58u) << 23;
-        uint32_t lowest = ~0u, highest = 0u;   // magnitudes' bits less one: a zero is above all of them, and harmless
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            const uint32_t b = __float_as_uint(d[k]) & 0x7FFFFFFFu;
-            lowest = min(lowest, b - 1u);
-            highest = max(highest, b);
-        }
-        if (lowest >= least - 1u && highest < end) {
-#pragma unroll
-            for (int k = 0; k < N; ++k) {
-                const float p = __fmul_rn(d[k], d[k]), e = __fmaf_rn(d[k], d[k], -p);
-                const float a = two_sum(mid, two_sum(hi, p)), b = two_sum(mid, e);
-                lo = __fadd_rn(lo, __fadd_rn(a, b));
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < N; ++k) {
-                const double x = f2d(d[k]);
-                wide = fma(x, x, wide);
-            }
-        }
-    }
-    __device__ __forceinline__ double total() const { return (double)hi + ((double)mid + ((double)lo + wide)); }
-};
-
 struct MlpTrainIO {           // what a training step keeps of the forward pass
     const float* T;           // targets [n][nout]
     float inv_scale;
     bf16 *xb, *h1, *h2, *dy;  // inputs and activations in bf16, (y - t) * inv_scale
-    double* loss;             // += sum (y - t)^2
+    float* err;               // y - t
 };
 
 // BM rows per CTA of NT threads: for BM = 64 two rows of warps, otherwise one, the others over the columns.
@@ -371,7 +331,6 @@ __global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad,
 #pragma unroll
                 for (int q = 0; q < 4; q += 2)
                     put_h(&z2[k][i][j][q], b2, wm + 16 * i + gid + q * 4, k * kNC + wn * (kNC / WN) + 8 * j + 2 * tig, io.h2);
-    SquareSum sq;   // training: this thread's sum of (y - t)^2
     for (int k = kW / kNC; k < nchunk; ++k) {
         const int n0 = (k - kW / kNC) * kNC + wn * (kNC / WN) + 2 * tig;
         float2 tg[TRAIN ? MI : 1][TRAIN ? N2 : 1][2];
@@ -402,39 +361,68 @@ __global__ void __launch_bounds__(NT) mlp_fused(int64_t n, int nin, int nin_pad,
                 for (int q = 0; q < 4; q += 2) {
                     const int64_t r = m0 + wm + 16 * i + gid + q * 4;
                     const int c = n0 + 8 * j;
-                    float &y0 = o[i][j][q], &y1 = o[i][j][q + 1];
-                    if (r >= n || c >= nout) {   // nout is even
-                        y0 = y1 = 0.f;
-                        continue;
-                    }
-                    y0 += __ldg(b3 + c);
-                    y1 += __ldg(b3 + c + 1);
+                    if (r >= n || c >= nout) continue;   // nout is even
+                    const float y0 = o[i][j][q] + __ldg(b3 + c), y1 = o[i][j][q + 1] + __ldg(b3 + c + 1);
                     if constexpr (!TRAIN) {
                         *reinterpret_cast<float2*>(Y + r * nout + c) = make_float2(y0, y1);
-                    } else {   // from here on the errors
+                    } else {
                         const float2 t = tg[i][j][q >> 1];
-                        y0 -= t.x;
-                        y1 -= t.y;
-                        *reinterpret_cast<uint32_t*>(io.dy + r * nout + c) = cvt2(y0 * io.inv_scale, y1 * io.inv_scale);
+                        const float d0 = y0 - t.x, d1 = y1 - t.y;
+                        *reinterpret_cast<uint32_t*>(io.dy + r * nout + c) = cvt2(d0 * io.inv_scale, d1 * io.inv_scale);
+                        *reinterpret_cast<float2*>(io.err + r * nout + c) = make_float2(d0, d1);
                     }
                 }
-        if constexpr (TRAIN) sq.template add<MI * N2 * 4>(&o[0][0][0]);
     }
     cp_wait<0>();
-    if constexpr (TRAIN) {
-        double s = sq.total();
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) atomicAdd(io.loss, s);
-    }
 }
+
+// A thread's sum of squares, no less exact than a float64 one: the square is exact in two floats, and the sum is
+// kept in floats of three sizes (TwoSum: hi + mid + mid2 exactly what was added but for the middle parts' own rounding
+// errors, which lo adds up), 72 bits against 53.  Where the largest of N values is outside 2^-40 .. 2^58, squares or
+// their low parts could leave the float32 range, and a float64 sum takes them (inf too; a NaN ends as one on either
+// path); smaller values beside a larger one lose less than 2^-70 of its square.  (The FP64 pipe takes a warp's
+// multiply-add every 19 cycles, 20 instructions here take 5.)
+struct SquareSum {
+    float hi = 0.f, mid = 0.f, mid2 = 0.f, lo = 0.f;
+    double wide = 0.0;
+    static __device__ __forceinline__ float two_sum(float& s, float x) {   // s += x, the rounding error returned
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s), e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+        s = t;
+        return e;
+    }
+    template <int N> __device__ __forceinline__ void add(const float* d) {
+        float most = 0.f;
+#pragma unroll
+        for (int k = 0; k < N; ++k) most = fmaxf(most, fabsf(d[k]));
+        if (most >= 0x1p-40f && most < 0x1p58f) {
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const float p = __fmul_rn(d[k], d[k]), e = __fmaf_rn(d[k], d[k], -p);
+                const float a = two_sum(mid, two_sum(hi, p)), b = two_sum(mid2, e);
+                lo = __fadd_rn(lo, __fadd_rn(a, b));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const double x = f2d(d[k]);
+                wide = fma(x, x, wide);
+            }
+        }
+    }
+    __device__ __forceinline__ double total() const { return (double)hi + (((double)mid + (double)mid2) + ((double)lo + wide)); }
+};
 
 // Gradient products of one layer in one launch, 32 x 32 of the result per CTA, K whole (the sums keep
 // the order of gemm_bf16), 64 of K per stage, four stages in flight.  Bound by the latency of the K chain
 // (64 dependent products for 1024 rows), so the tiles are small: more CTAs, not more work per CTA.
 //   dw CTAs: G [M][N] = alpha D^T H  (D [K][M], H [K][N] rows of the batch);
 //   db CTAs: the column sums of D (the bias gradient), rows in order, 32 columns each;
-//   dh CTAs: Z [K][N] = (D W) masked by H > 0, in bf16 (W [M][N] the layer's weights, H its input).
+//   dh CTAs: Z [K][N] = (D W) masked by H > 0, in bf16 (W [M][N] the layer's weights, H its input);
+//   loss CTAs (output layer): += the sum of the squared float32 errors, kLossPer of them each, on SMs that the chains
+//     leave idle.  In the forward kernel, whose CTAs have 64 SMs at 1,024 rows, the same sum took 1 to 2 us of a step's
+//     79, a float64 one 6; here a step is 2 us shorter up to 1,024 rows, 1.6 us (of 106) longer at 2,048.
 constexpr int kBT = 32, kBK = 64, kBStages = 4;
+constexpr int64_t kLossPer = 8192;
 struct BackArgs {
     int64_t K;             // rows of the batch
     int M, N;              // the layer's outputs and inputs
@@ -443,6 +431,10 @@ struct BackArgs {
     bf16* Z;               // null: no dh part
     float beta;
     int dw_n, dw_tiles;    // CTAs along N and in all of the dw part
+    const float* err;      // n_err (a multiple of 4) errors; the loss CTAs are the last, from loss_at on
+    int64_t n_err;
+    double* loss;
+    unsigned loss_at;
 };
 
 __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
@@ -451,6 +443,30 @@ __global__ void __launch_bounds__(128) mlp_back(BackArgs P) {
     __shared__ __align__(16) bf16 sA[kBStages][AS], sB[kBStages][AS];
     static_assert(kBT * DS <= AS, "stage size");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
+    if (blockIdx.x >= P.loss_at) {
+        __shared__ double s_sum[4];
+        const int64_t i0 = (int64_t)(blockIdx.x - P.loss_at) * kLossPer;
+        SquareSum sq;
+        for (int k = 0; k < kLossPer; k += 16 * 128) {
+            float d[16];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t i = i0 + k + 4 * (128 * j + tid);
+                const float4 v = i < P.n_err ? *reinterpret_cast<const float4*>(P.err + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                d[4 * j] = v.x;
+                d[4 * j + 1] = v.y;
+                d[4 * j + 2] = v.z;
+                d[4 * j + 3] = v.w;
+            }
+            sq.add<16>(d);
+        }
+        double s = sq.total();
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) s_sum[warp] = s;
+        __syncthreads();
+        if (tid == 0) atomicAdd(P.loss, (s_sum[0] + s_sum[1]) + (s_sum[2] + s_sum[3]));
+        return;
+    }
     const int wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
     // the db CTAs come first (their serial sums are the longest chain), then dw, then dh
     const int b0 = (int)blockIdx.x - (P.M + kBT - 1) / kBT;
@@ -769,12 +785,12 @@ template <class T> static bool grow(T*& p, int64_t n) {
 static bool mlp_reserve(Mlp& M, int64_t b, bool general) {
     if (b > M.cap) {
         const bool ok = grow(M.xb, b * M.nin_pad) && grow(M.h1, b * M.w) && grow(M.h2, b * M.w) && grow(M.dyb, b * M.nout) &&
-                        grow(M.dz2, b * M.w) && grow(M.dz1, b * M.w);
+                        grow(M.dz2, b * M.w) && grow(M.dz1, b * M.w) && grow(M.y, b * M.nout);
         M.cap = ok ? b : 0;
         if (!ok) return false;
     }
     if (general && b > M.cap_general) {
-        const bool ok = grow(M.z1, b * M.w) && grow(M.z2, b * M.w) && grow(M.y, b * M.nout) && grow(M.dh2, b * M.w) && grow(M.dh1, b * M.w);
+        const bool ok = grow(M.z1, b * M.w) && grow(M.z2, b * M.w) && grow(M.dh2, b * M.w) && grow(M.dh1, b * M.w);
         M.cap_general = ok ? b : 0;
         if (!ok) return false;
     }
@@ -816,18 +832,19 @@ static void mlp_fused_rows(const Mlp& M, const float* X, int64_t ldx, int64_t n,
 // forward and backward of a batch on the fused path: gradients into M.G, loss added to M.loss
 static void mlp_step_fused(Mlp& M, const float* X, int64_t ldx, const float* T, int64_t b, double n_total, float beta,
                            cudaStream_t s) {
-    const MlpTrainIO io = {T, (float)(1.0 / n_total), M.xb, M.h1, M.h2, M.dyb, M.loss};
+    const MlpTrainIO io = {T, (float)(1.0 / n_total), M.xb, M.h1, M.h2, M.dyb, M.y};
     mlp_fused_rows<true>(M, X, ldx, b, nullptr, io, s);
-    auto back = [&](int m, int nn, const bf16* D, const bf16* H, int k, bf16* Z) {
-        BackArgs P = {b, m, nn, D, H, M.Pb + M.off(k), M.G + M.off(k), M.G + M.off(k + 1), Z, beta, 0, 0};
+    auto back = [&](int m, int nn, const bf16* D, const bf16* H, int k, bf16* Z, int64_t n_err) {
+        BackArgs P = {b, m, nn, D, H, M.Pb + M.off(k), M.G + M.off(k), M.G + M.off(k + 1), Z, beta, 0, 0, M.y, n_err, M.loss, 0};
         P.dw_n = (nn + kBT - 1) / kBT;
         P.dw_tiles = P.dw_n * ((m + kBT - 1) / kBT);
         const int64_t dh = Z ? P.dw_n * ((b + kBT - 1) / kBT) : 0;
-        mlp_back<<<(unsigned)((m + kBT - 1) / kBT + P.dw_tiles + dh), 128, 0, s>>>(P);
+        P.loss_at = (unsigned)((m + kBT - 1) / kBT + P.dw_tiles + dh);
+        mlp_back<<<P.loss_at + (unsigned)((n_err + kLossPer - 1) / kLossPer), 128, 0, s>>>(P);
     };
-    back(M.nout, M.w, M.dyb, M.h2, 4, M.dz2);
-    back(M.w, M.w, M.dz2, M.h1, 2, M.dz1);
-    back(M.w, M.nin_pad, M.dz1, M.xb, 0, nullptr);
+    back(M.nout, M.w, M.dyb, M.h2, 4, M.dz2, b * M.nout);
+    back(M.w, M.w, M.dz2, M.h1, 2, M.dz1, 0);
+    back(M.w, M.nin_pad, M.dz1, M.xb, 0, nullptr, 0);
 }
 
 // forward of a batch: X float [b][ldx] (first nin columns) -> M.y float [b][nout]
